@@ -133,8 +133,8 @@ typedef enum {
                                       bucket unit, a Step-2 sublist of
                                       t = 32768) is sorted by comparisons
                                       (register networks and merges) instead
-                                      of by 7-bit digits over the bits that
-                                      vary in the unit (the default).  Same
+                                      of by bins of its key range (the
+                                      default).  Same
                                       result; kept to measure one against the
                                       other */
 

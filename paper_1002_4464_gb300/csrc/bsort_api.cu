@@ -75,7 +75,7 @@ struct Plan {
         off_units, off_units2, off_srcb, off_blk, off_cum, off_jr, off_rs, total;
     bool rec_radix;  // Steps 4-5 by the radix sort of the records (else chunks + merges)
     bool relocate;  // materialise Step 8 (else fused into Step 9's load)
-    bool radix;     // 32768-key chunks of 32-bit keys sorted by digits
+    bool bins;      // 32768-key chunks of 32-bit keys sorted by bins
     // two-level plans (n' >= 2^32): 64-bit bucket offsets, bucket starts,
     // and the workspace of the bucket sorts
     uint64_t off_off64, off_csum, off_cpre, off_starts, off_child, child_bytes;
@@ -365,7 +365,7 @@ bsort_status make_plan_two_level(bsort_t h, bsort_key_type kt, uint64_t n, Plan 
     P->kb = 4;
     P->vb = 0;
     P->relocate = true;
-    P->radix = !(h && (h->flags & BSORT_FLAG_MERGE_SORT));
+    P->bins = !(h && (h->flags & BSORT_FLAG_MERGE_SORT));
     bsort_plan_info &I = P->info;
     const uint64_t t = 32768;
     const uint64_t m = (n + t - 1) / t;
@@ -677,7 +677,7 @@ bsort_status make_plan_with(bsort_t h, bsort_key_type kt, uint32_t vb, uint64_t 
         return at;
     };
     P->relocate = P->wide || !(h && (h->flags & BSORT_FLAG_LOW_MEMORY));
-    P->radix = !P->pairs && !P->wide && !(h && (h->flags & BSORT_FLAG_MERGE_SORT));
+    P->bins = !P->pairs && !P->wide && !(h && (h->flags & BSORT_FLAG_MERGE_SORT));
     P->off_hdr = take(kAlign);  // error word (int) + scan ticket (uint32)
     if (!I.single_tile) {
         const uint64_t np = I.n_padded;
@@ -911,7 +911,7 @@ bsort_status run_sort_two_level(bsort_t h, const Plan &P, bsort_key_type kt, con
     unsigned char *child_ws = ws + P.off_child;
     // Steps 1-3
     SEQ(launch_sublist_sort_keys(P.tile_chunk, 1, kin, n, I.m, is_f32, I.s, tiles_k, samples, st,
-                                 0, P.radix),
+                                 0, P.bins),
         "step1_3_sublist_sort");
     // Steps 4-5
     const bool one_chunk = P.n_rec_pad == (uint32_t)kRecordChunk;
@@ -1150,7 +1150,7 @@ bsort_status run_sort(bsort_t h, bsort_key_type kt, const void *kin, const void 
                                                1, n, n, is_f32, (int)vb, kout, vout, err, none,
                                                st)
                     : launch_bucket_sort_keys(P.unit_chunk, (int)I.unit_ctas, kin, nullptr, 1, n,
-                                              n, is_f32, kout, err, none, st, P.radix),
+                                              n, is_f32, kout, err, none, st, P.bins),
             "step9_single_unit");
         return BSORT_OK;
     }
@@ -1193,7 +1193,7 @@ bsort_status run_sort(bsort_t h, bsort_key_type kt, const void *kin, const void 
                 if (e != cudaSuccess) return cuda_fail(h, e, "host-to-device copy");
             }
             SEQ(launch_sublist_sort_keys(P.tile_chunk, (int)I.tile_ctas, kin, n, mc, is_f32,
-                                         I.s, tiles_k, samples, st, t0, P.radix),
+                                         I.s, tiles_k, samples, st, t0, P.bins),
                 "step1_3_sublist_sort");
         }
     } else {
@@ -1201,7 +1201,7 @@ bsort_status run_sort(bsort_t h, bsort_key_type kt, const void *kin, const void 
                                                 I.m, is_f32, (int)vb, I.s, tiles_k, tiles_v,
                                                 samples, st)
                     : launch_sublist_sort_keys(P.tile_chunk, (int)I.tile_ctas, kin, n, I.m,
-                                               is_f32, I.s, tiles_k, samples, st, 0, P.radix),
+                                               is_f32, I.s, tiles_k, samples, st, 0, P.bins),
             "step1_3_sublist_sort");
     }
     // Steps 4-5: the records by digits (large sample sets), or in chunks
@@ -1310,12 +1310,12 @@ bsort_status run_sort(bsort_t h, bsort_key_type kt, const void *kin, const void 
         const uint32_t g2 = std::max(1u, (uint32_t)((sms * 7 / 8) / (int)I.unit_ctas));
         for (int g = 0; g < G; ++g) {
             SEQ(launch_bucket_sort_keys_range(c1, k1, s9k, units, r1 + g, g1, n, I.n_padded,
-                                              is_f32, kout, err, st, P.radix),
+                                              is_f32, kout, err, st, P.bins),
                 "step9_bucket_sort");
             if (units2)
                 SEQ(launch_bucket_sort_keys_range(P.unit_chunk, (int)I.unit_ctas, s9k, units2,
                                                   r2 + g, g2, n, I.n_padded, is_f32, kout, err,
-                                                  st, P.radix),
+                                                  st, P.bins),
                     "step9_bucket_sort_large");
             const uint64_t p0 = std::min<uint64_t>((uint64_t)g * np / G, n);
             const uint64_t p1 = std::min<uint64_t>((uint64_t)(g + 1) * np / G, n);
@@ -1335,7 +1335,7 @@ bsort_status run_sort(bsort_t h, bsort_key_type kt, const void *kin, const void 
     SEQ(P.pairs ? launch_bucket_sort_pairs(c1, k1, s9k, s9v, units, I.b, n, I.n_padded, is_f32,
                                            (int)vb, kout, vout, err, g, st)
                 : launch_bucket_sort_keys(c1, k1, s9k, units, I.b, n, I.n_padded, is_f32, kout,
-                                          err, g, st, P.radix),
+                                          err, g, st, P.bins),
         "step9_bucket_sort");
     if (P.small_chunk) {
         const uint32_t u2 = large_units_max(I.n_padded, q1, I.b);
@@ -1343,7 +1343,7 @@ bsort_status run_sort(bsort_t h, bsort_key_type kt, const void *kin, const void 
                                                u2, n, I.n_padded, is_f32, (int)vb, kout, vout,
                                                err, g, st)
                     : launch_bucket_sort_keys(P.unit_chunk, (int)I.unit_ctas, s9k, units2, u2, n,
-                                              I.n_padded, is_f32, kout, err, g, st, P.radix),
+                                              I.n_padded, is_f32, kout, err, g, st, P.bins),
             "step9_bucket_sort_large");
     }
     return BSORT_OK;
@@ -1777,7 +1777,7 @@ bsort_status run_batch(bsort_t h, bsort_key_type kt, const void *kin, void *kout
             SEQ(launch_relocate(tiles, nullptr, offsets, srcb, blk, B.runs, (uint32_t)B.n_pad, 0,
                                 reloc, nullptr, st),
                 "batch_step8_relocate");
-            SEQ(launch_seg_bucket_sort((int)kBatchUnit, reloc, units, B.info.buckets, segs,
+            SEQ(launch_seg_bucket_sort(reloc, units, B.info.buckets, segs,
                                        offsets, is_f32, ko, err, st),
                 "batch_step9_bucket_sort");
         }

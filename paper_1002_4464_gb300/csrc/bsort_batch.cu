@@ -23,7 +23,7 @@
 // over all counts gives every run its place in the padded space.
 #include "bsort_device.cuh"
 #include "bsort_internal.h"
-#include "bsort_radix.cuh"
+#include "bsort_sort.cuh"
 
 namespace bsort {
 
@@ -31,8 +31,8 @@ namespace bsort {
 // Cluster u sorts segment u = [seg[2u], seg[2u+1]) of the input (at most
 // C*T*E keys, guaranteed by the host) into the same range of the output.
 // K: uint32_t (uint32 / float32 keys) or uint64_t (64-bit keys).
-template <typename K, int T, int E, int C>
-__global__ void __launch_bounds__(T, 1)
+template <typename K, int T, int E, int C, bool BINS>
+__global__ void __launch_bounds__(T, (min_ctas<T, E, C, BINS>()))
 k_seg_sort(const K *__restrict__ keys_in, K *__restrict__ keys_out,
            const uint32_t *__restrict__ seg, int is_f32, int *err)
 {
@@ -54,18 +54,8 @@ k_seg_sort(const K *__restrict__ keys_in, K *__restrict__ keys_out,
     const int ustart = r * per;
     const int uend = min(ustart + per, len);
     K v[E];
-#pragma unroll
-    for (int k = 0; k < E; ++k) {
-        const int x = ustart + wb_pos<E>(warp, lane, k);
-        K key = KeyMax<K>::v;
-        if (x < uend) {
-            key = keys_in[L + x];
-            if constexpr (sizeof(K) == 4)
-                if (is_f32) key = f32_encode(key);
-        }
-        v[k] = key;
-    }
-    cta_sort<K, T, E>(v, sm, uend > ustart ? uend - ustart : 0);
+    load_keys<K, T, E>(v, keys_in + L + ustart, uend - ustart, is_f32 != 0);
+    chunk_sort<K, T, E, BINS>(v, sm, uend > ustart ? uend - ustart : 0, is_f32 != 0);
     cluster_merge<K, T, E, C>(sm, len, per);
     const int off = r * CH;
 #pragma unroll 4
@@ -85,13 +75,7 @@ k_seg_sort(const K *__restrict__ keys_in, K *__restrict__ keys_out,
 // segment, i = g - g0, padded with the maximal key; writes the sorted
 // sublist to tiles[g*t ...] and its s samples (ranks (k+1)w - 1) as
 // key << 32 | (g*t + rank) to the segment's record array.  The sublist is
-// sorted by digits (cta_radix_sort, 7-bit digits over the bits that vary
-// in it): 6.3 against 6.6 ms by comparisons for the 25,000 sublists of the
-// 20,000-array workload; its buckets, whose keys span most of the 32 bits
-// (few buckets per segment), sort as fast by comparisons, so Step 9 keeps
-// them.
-constexpr int kSegRadixBits = 7;
-
+// sorted by bins (cta_bin_sort).
 template <int T, int E>
 __global__ void __launch_bounds__(T, 1)
 k_seg_sublist_sort(const uint32_t *__restrict__ keys_in, int is_f32,
@@ -110,17 +94,8 @@ k_seg_sublist_sort(const uint32_t *__restrict__ keys_in, int is_f32,
     const int len = sg.n - first < (uint32_t)TT ? (int)(sg.n - first) : TT;
     const uint64_t src = (uint64_t)sg.out + first;
     uint32_t v[E];
-#pragma unroll
-    for (int k = 0; k < E; ++k) {
-        const int x = wb_pos<E>(warp, lane, k);
-        uint32_t key = 0xFFFFFFFFu;
-        if (x < len) {
-            key = keys_in[src + x];
-            if (is_f32) key = f32_encode(key);
-        }
-        v[k] = key;
-    }
-    cta_radix_sort<T, E, kSegRadixBits>(v, sm, len);
+    load_keys<uint32_t, T, E>(v, keys_in + src, len, is_f32 != 0);
+    cta_bin_sort<uint32_t, T, E>(v, sm, len, is_f32 != 0);
     const uint64_t base = (uint64_t)g * TT;
 #pragma unroll 4
     for (int k = 0; k < E; ++k) {
@@ -229,8 +204,8 @@ k_seg_sample_index(const uint32_t *__restrict__ tiles_k, const uint64_t *__restr
 // relocated array, and writes its ranks that hold real items (position -
 // g0*t < n) to the segment's output range.  K: uint32_t (uint32 / float32
 // keys) or uint64_t (64-bit keys).
-template <typename K, int T, int E>
-__global__ void __launch_bounds__(T, 1)
+template <typename K, int T, int E, bool BINS>
+__global__ void __launch_bounds__(T, (min_ctas<T, E, 1, BINS>()))
 k_seg_bucket_sort(const K *__restrict__ reloc_k, const uint32_t *__restrict__ units,
                   const SegInfo *__restrict__ segs, const uint32_t *__restrict__ offsets,
                   uint32_t t, int is_f32, K *__restrict__ keys_out, int *err)
@@ -253,12 +228,8 @@ k_seg_bucket_sort(const K *__restrict__ reloc_k, const uint32_t *__restrict__ un
     const int len = (int)(R - L);
     if (len == 0) return;
     K v[E];
-#pragma unroll
-    for (int k = 0; k < E; ++k) {
-        const int x = wb_pos<E>(warp, lane, k);
-        v[k] = x < len ? reloc_k[L + x] : KeyMax<K>::v;
-    }
-    cta_sort<K, T, E>(v, sm, len);
+    load_keys<K, T, E>(v, reloc_k + L, len, false);
+    chunk_sort<K, T, E, BINS>(v, sm, len, is_f32 != 0);
     // ranks below lim hold real items of the segment (its padding sorts last)
     const uint32_t rel = L - P;
     const int lim = rel >= sg.n ? 0 : (sg.n - rel < (uint32_t)len ? (int)(sg.n - rel) : len);
@@ -439,11 +410,11 @@ cudaError_t set_smem_attr(KernelT k, int bytes, bool nonportable = false)
     return e;
 }
 
-template <typename K, int T, int E, int C>
+template <typename K, int T, int E, int C, bool BINS>
 cudaError_t launch_seg_sort_t(const void *keys_in, void *keys_out, const uint32_t *seg,
                               uint32_t nseg, int is_f32, int *err, cudaStream_t st)
 {
-    const int sm = padded_elems<K>(T * E) * (int)sizeof(K);
+    const int sm = sort_smem_bytes<K, T, E, BINS>();
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(nseg * C, 1, 1);
     cfg.blockDim = dim3(T, 1, 1);
@@ -456,14 +427,14 @@ cudaError_t launch_seg_sort_t(const void *keys_in, void *keys_out, const uint32_
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = C > 1 ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, k_seg_sort<K, T, E, C>, static_cast<const K *>(keys_in),
+    return cudaLaunchKernelEx(&cfg, k_seg_sort<K, T, E, C, BINS>, static_cast<const K *>(keys_in),
                               static_cast<K *>(keys_out), seg, is_f32, err);
 }
 
-template <typename K, int T, int E, int C>
+template <typename K, int T, int E, int C, bool BINS>
 cudaError_t init_seg_sort_t()
 {
-    return set_smem_attr(k_seg_sort<K, T, E, C>, padded_elems<K>(T * E) * (int)sizeof(K));
+    return set_smem_attr(k_seg_sort<K, T, E, C, BINS>, sort_smem_bytes<K, T, E, BINS>());
 }
 
 }  // namespace
@@ -479,7 +450,7 @@ bool batch_wide_cluster16()
         // non-portable cluster size: usable only if the device schedules it
         const int sm = padded_elems<uint64_t>(16384) * 8;
         int n = 0;
-        cudaError_t q = set_smem_attr(k_seg_sort<uint64_t, 1024, 16, 16>, sm, true);
+        cudaError_t q = set_smem_attr(k_seg_sort<uint64_t, 1024, 16, 16, false>, sm, true);
         if (q == cudaSuccess) {
             cudaLaunchConfig_t cfg = {};
             cfg.gridDim = dim3(16, 1, 1);
@@ -492,7 +463,7 @@ bool batch_wide_cluster16()
             attr[0].val.clusterDim.z = 1;
             cfg.attrs = attr;
             cfg.numAttrs = 1;
-            q = cudaOccupancyMaxActiveClusters(&n, k_seg_sort<uint64_t, 1024, 16, 16>, &cfg);
+            q = cudaOccupancyMaxActiveClusters(&n, k_seg_sort<uint64_t, 1024, 16, 16, false>, &cfg);
         }
         if (q != cudaSuccess) cudaGetLastError();  // (not an error: the shape is left out)
         g_wide16 = q == cudaSuccess && n >= 1 ? 1 : 0;
@@ -504,38 +475,36 @@ cudaError_t init_batch_kernels()
 {
     cudaError_t e = cudaSuccess;
     batch_wide_cluster16();
-    if (e == cudaSuccess) e = init_seg_sort_t<uint32_t, 128, 16, 1>();
-    if (e == cudaSuccess) e = init_seg_sort_t<uint32_t, 256, 16, 1>();
-    if (e == cudaSuccess) e = init_seg_sort_t<uint32_t, 512, 16, 1>();
-    if (e == cudaSuccess) e = init_seg_sort_t<uint32_t, 1024, 16, 1>();
-    if (e == cudaSuccess) e = init_seg_sort_t<uint32_t, 1024, 32, 1>();
-    if (e == cudaSuccess) e = init_seg_sort_t<uint32_t, 1024, 32, 2>();
-    if (e == cudaSuccess) e = init_seg_sort_t<uint32_t, 1024, 32, 4>();
-    if (e == cudaSuccess) e = init_seg_sort_t<uint32_t, 1024, 32, 8>();
-    if (e == cudaSuccess) e = init_seg_sort_t<uint64_t, 128, 16, 1>();
-    if (e == cudaSuccess) e = init_seg_sort_t<uint64_t, 256, 16, 1>();
-    if (e == cudaSuccess) e = init_seg_sort_t<uint64_t, 512, 16, 1>();
-    if (e == cudaSuccess) e = init_seg_sort_t<uint64_t, 1024, 16, 1>();
-    if (e == cudaSuccess) e = init_seg_sort_t<uint64_t, 1024, 16, 2>();
-    if (e == cudaSuccess) e = init_seg_sort_t<uint64_t, 1024, 16, 4>();
-    if (e == cudaSuccess) e = init_seg_sort_t<uint64_t, 1024, 16, 8>();
+    if (e == cudaSuccess) e = init_seg_sort_t<uint32_t, 128, 16, 1, true>();
+    if (e == cudaSuccess) e = init_seg_sort_t<uint32_t, 256, 16, 1, true>();
+    if (e == cudaSuccess) e = init_seg_sort_t<uint32_t, 256, 32, 1, true>();
+    if (e == cudaSuccess) e = init_seg_sort_t<uint32_t, 512, 32, 1, true>();
+    if (e == cudaSuccess) e = init_seg_sort_t<uint32_t, 512, 64, 1, true>();
+    if (e == cudaSuccess) e = init_seg_sort_t<uint32_t, 1024, 32, 2, false>();
+    if (e == cudaSuccess) e = init_seg_sort_t<uint32_t, 1024, 32, 4, false>();
+    if (e == cudaSuccess) e = init_seg_sort_t<uint32_t, 1024, 32, 8, false>();
+    if (e == cudaSuccess) e = init_seg_sort_t<uint64_t, 128, 16, 1, false>();
+    if (e == cudaSuccess) e = init_seg_sort_t<uint64_t, 256, 16, 1, false>();
+    if (e == cudaSuccess) e = init_seg_sort_t<uint64_t, 512, 16, 1, false>();
+    if (e == cudaSuccess) e = init_seg_sort_t<uint64_t, 1024, 16, 1, false>();
+    if (e == cudaSuccess) e = init_seg_sort_t<uint64_t, 1024, 16, 2, false>();
+    if (e == cudaSuccess) e = init_seg_sort_t<uint64_t, 1024, 16, 4, false>();
+    if (e == cudaSuccess) e = init_seg_sort_t<uint64_t, 1024, 16, 8, false>();
     if (e == cudaSuccess)
-        e = set_smem_attr(k_seg_sublist_sort<256, 128>, RadixSmem<256, 128, kSegRadixBits>::kBytes);
+        e = set_smem_attr(k_seg_sublist_sort<512, 64>,
+                          BinSmem<uint32_t, 512, 64>::kBytes);
     if (e == cudaSuccess)
         e = set_smem_attr(k_seg_records<1024, 16>, padded_elems<uint64_t>(kRecordChunk) * 8);
     if (e == cudaSuccess)
-        e = set_smem_attr(k_seg_bucket_sort<uint32_t, 1024, 16>,
-                          padded_elems<uint32_t>(16384) * 4);
-    if (e == cudaSuccess)
-        e = set_smem_attr(k_seg_bucket_sort<uint32_t, 1024, 32>,
-                          padded_elems<uint32_t>(32768) * 4);
+        e = set_smem_attr(k_seg_bucket_sort<uint32_t, 512, 64, true>,
+                          BinSmem<uint32_t, 512, 64>::kBytes);
     if (e == cudaSuccess)
         e = set_smem_attr(k_seg_sublist_sort_u64<1024, 16>,
                           padded_elems<uint64_t>(kSegTileU64) * 8);
     if (e == cudaSuccess)
         e = set_smem_attr(k_seg_records_u64<1024>, (int)(kSegRecordsU64 * sizeof(Rec128)));
     if (e == cudaSuccess)
-        e = set_smem_attr(k_seg_bucket_sort<uint64_t, 1024, 16>,
+        e = set_smem_attr(k_seg_bucket_sort<uint64_t, 1024, 16, false>,
                           padded_elems<uint64_t>(kSegTileU64) * 8);
     return e;
 }
@@ -545,41 +514,41 @@ cudaError_t launch_seg_sort(int chunk, int ctas, bool wide, const void *keys_in,
                             cudaStream_t st)
 {
     if (nseg == 0) return cudaSuccess;
-#define L(K_, T_, E_, C_) \
-    return launch_seg_sort_t<K_, T_, E_, C_>(keys_in, keys_out, seg, nseg, is_f32, err, st)
+#define L(K_, T_, E_, C_, B_) \
+    return launch_seg_sort_t<K_, T_, E_, C_, B_>(keys_in, keys_out, seg, nseg, is_f32, err, st)
     if (wide) {
         if (ctas == 1) {
             switch (chunk) {
-            case 2048: L(uint64_t, 128, 16, 1);
-            case 4096: L(uint64_t, 256, 16, 1);
-            case 8192: L(uint64_t, 512, 16, 1);
-            case 16384: L(uint64_t, 1024, 16, 1);
+            case 2048: L(uint64_t, 128, 16, 1, false);
+            case 4096: L(uint64_t, 256, 16, 1, false);
+            case 8192: L(uint64_t, 512, 16, 1, false);
+            case 16384: L(uint64_t, 1024, 16, 1, false);
             }
         } else if (chunk == 16384) {
             switch (ctas) {
-            case 2: L(uint64_t, 1024, 16, 2);
-            case 4: L(uint64_t, 1024, 16, 4);
-            case 8: L(uint64_t, 1024, 16, 8);
+            case 2: L(uint64_t, 1024, 16, 2, false);
+            case 4: L(uint64_t, 1024, 16, 4, false);
+            case 8: L(uint64_t, 1024, 16, 8, false);
             case 16:
                 if (!batch_wide_cluster16()) return cudaErrorInvalidValue;
-                L(uint64_t, 1024, 16, 16);
+                L(uint64_t, 1024, 16, 16, false);
             }
         }
         return cudaErrorInvalidValue;
     }
     if (ctas == 1) {
         switch (chunk) {
-        case 2048: L(uint32_t, 128, 16, 1);
-        case 4096: L(uint32_t, 256, 16, 1);
-        case 8192: L(uint32_t, 512, 16, 1);
-        case 16384: L(uint32_t, 1024, 16, 1);
-        case 32768: L(uint32_t, 1024, 32, 1);
+        case 2048: L(uint32_t, 128, 16, 1, true);
+        case 4096: L(uint32_t, 256, 16, 1, true);
+        case 8192: L(uint32_t, 256, 32, 1, true);
+        case 16384: L(uint32_t, 512, 32, 1, true);
+        case 32768: L(uint32_t, 512, 64, 1, true);
         }
     } else if (chunk == 32768) {
         switch (ctas) {
-        case 2: L(uint32_t, 1024, 32, 2);
-        case 4: L(uint32_t, 1024, 32, 4);
-        case 8: L(uint32_t, 1024, 32, 8);
+        case 2: L(uint32_t, 1024, 32, 2, false);
+        case 4: L(uint32_t, 1024, 32, 4, false);
+        case 8: L(uint32_t, 1024, 32, 8, false);
         }
     }
 #undef L
@@ -591,9 +560,9 @@ cudaError_t launch_seg_sublist_sort(const uint32_t *keys_in, int is_f32, const u
                                     uint64_t *samples, cudaStream_t st)
 {
     if (nsub == 0) return cudaSuccess;
-    static_assert(kSegTile == 256 * 128, "a sublist is one radix CTA's unit");
-    const int sm = RadixSmem<256, 128, kSegRadixBits>::kBytes;
-    k_seg_sublist_sort<256, 128><<<nsub, 256, sm, st>>>(keys_in, is_f32, sub_seg, segs, tiles_k,
+    static_assert(kSegTile == 512 * 64, "a sublist is one CTA's unit");
+    const int sm = BinSmem<uint32_t, 512, 64>::kBytes;
+    k_seg_sublist_sort<512, 64><<<nsub, 512, sm, st>>>(keys_in, is_f32, sub_seg, segs, tiles_k,
                                                         samples);
     return cudaGetLastError();
 }
@@ -618,22 +587,14 @@ cudaError_t launch_seg_sample_index(const uint32_t *tiles_k, const uint64_t *sam
     return cudaGetLastError();
 }
 
-cudaError_t launch_seg_bucket_sort(int chunk, const uint32_t *reloc_k, const uint32_t *units,
-                                   uint32_t nunits, const SegInfo *segs, const uint32_t *offsets,
-                                   int is_f32, uint32_t *keys_out, int *err, cudaStream_t st)
+cudaError_t launch_seg_bucket_sort(const uint32_t *reloc_k, const uint32_t *units, uint32_t nunits,
+                                   const SegInfo *segs, const uint32_t *offsets, int is_f32,
+                                   uint32_t *keys_out, int *err, cudaStream_t st)
 {
     if (nunits == 0) return cudaSuccess;
-    if (chunk == 16384) {
-        k_seg_bucket_sort<uint32_t, 1024, 16>
-            <<<nunits, 1024, padded_elems<uint32_t>(16384) * 4, st>>>(
-                reloc_k, units, segs, offsets, (uint32_t)kSegTile, is_f32, keys_out, err);
-    } else if (chunk == 32768) {
-        k_seg_bucket_sort<uint32_t, 1024, 32>
-            <<<nunits, 1024, padded_elems<uint32_t>(32768) * 4, st>>>(
-                reloc_k, units, segs, offsets, (uint32_t)kSegTile, is_f32, keys_out, err);
-    } else {
-        return cudaErrorInvalidValue;
-    }
+    k_seg_bucket_sort<uint32_t, 512, 64, true>
+        <<<nunits, 512, BinSmem<uint32_t, 512, 64>::kBytes, st>>>(
+            reloc_k, units, segs, offsets, (uint32_t)kSegTile, is_f32, keys_out, err);
     return cudaGetLastError();
 }
 
@@ -674,7 +635,7 @@ cudaError_t launch_seg_bucket_sort_u64(const uint64_t *reloc_k, const uint32_t *
                                        cudaStream_t st)
 {
     if (nunits == 0) return cudaSuccess;
-    k_seg_bucket_sort<uint64_t, 1024, 16>
+    k_seg_bucket_sort<uint64_t, 1024, 16, false>
         <<<nunits, 1024, padded_elems<uint64_t>(kSegTileU64) * 8, st>>>(
             reloc_k, units, segs, offsets, (uint32_t)kSegTileU64, 0, keys_out, err);
     return cudaGetLastError();

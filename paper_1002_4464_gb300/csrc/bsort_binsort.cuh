@@ -1,0 +1,577 @@
+// bsort_binsort.cuh -- one-pass distribution sort of the keys held by one
+// CTA (Step 2, Step 9 and whole units of GPU Bucket Sort, Dehne & Zaboli,
+// Section 4, Algorithm 1, which may use any exact sort).
+//
+// Equal keys of a keys-only sort are indistinguishable, so nothing has to be
+// stable, and one counting pass over many bins replaces the digit passes (or
+// merge levels): the NB bins cut the unit's key range [kmin, kmax] linearly
+// (float keys: their values), about one key per bin;
+//   1. every key adds one to its bin's 16-bit counter (shared-memory
+//      reductions; two bins per word: bin b is the low half of word b for
+//      b < NB/2, the high half of word b - NB/2 otherwise);
+//   2. one exclusive scan of the counters, and the largest bin's count G;
+//   3. an atomic add on its bin's counter gives each key its rank, where it
+//      is stored;
+//   4. the keys are now sorted by bin, so every key is within G of its place:
+//      each thread reloads E consecutive keys and G phases of odd-even
+//      transposition (one min and one max per pair, neighbouring lanes by
+//      shuffles) order them.  Groups of one bin that straddle two warps are
+//      merged afterwards, 32 keys either side.
+// What bounds it: the shared-memory pipe (60 % busy; a random-bank atomic
+// takes about six wavefronts per warp, the scatter three) and the barriers
+// between the steps with one or two CTAs per SM.  2^26 keys on a GB300, load
+// and store included: as 32768-key units 255 us (512 threads x 64 keys; five
+// 7-bit digit passes took 513 us, for 19 varying bits three passes 338 us),
+// as 16384-key units 203 us (two CTAs of 512 x 32 per SM; comparison sort
+// 588 us), 8192: 189 us (448), 4096: 191 us (369), 2048: 174 us (314).  1024
+// threads x 32 keys for 32768 keys measured 283 us (64 registers spill).
+// A range below NB gives every value a bin of its own (several, when there
+// are fewer values than lanes, so that a warp's atomics do not meet on one
+// counter) and needs no step 4.
+//
+// Skewed keys (bin_skewed; a bin of more than kBinPhases keys): every bin b
+// of n_b keys is cut once more, linearly into n_b bins at positions
+// [P_b, P_b + n_b) of the order, so that crowded stretches of the range get
+// as many bins as they hold keys, and two repeated values that shared a bin
+// part.  (A bin with an eighth of the unit or more takes every 16th of those
+// positions, and its keys are spread over the 16 by lane: a value repeated
+// that often would otherwise meet on one counter.)  What is left unordered
+// inside the refined bins is put right by up to kBinPhases phases, by a
+// comparison sort of the warps where that is not enough, and by merging all
+// runs when two warps still overlap.  When a bin holds a quarter of the unit
+// and its keys differ (one key far from the others, keys spread over their
+// logarithm), refining would not part them: the unit is sorted by digits
+// or comparisons instead.  (1024 values, Zipf 1.1: 445 us against 515 by
+// digits as 32768-key units, 381 against 584 by comparisons as 16384; 2048:
+// 337 against 314; keys spread over their logarithm: 755 against 512.)
+#pragma once
+
+#include <cstdint>
+
+#include "bsort_device.cuh"
+#include "bsort_radix.cuh"
+
+namespace bsort {
+
+constexpr uint32_t kBinPhases = 32;  // largest bin ordered by phases alone
+
+// Bins of a unit of T*E keys.
+template <typename K, int T, int E>
+constexpr int bin_count() { return T * E; }
+
+// Shared memory of cta_bin_sort: the keys in the padded layout, then NB
+// 16-bit counters (16-byte aligned) and a spare word per lane; at least what
+// the digit sort of crowded units takes.
+template <typename K, int T, int E>
+struct BinSmem {
+    static constexpr int kKeyBytes = (padded_elems<K>(T * E) * (int)sizeof(K) + 15) & ~15;
+    static constexpr int kBins = kKeyBytes + bin_count<K, T, E>() * 2 + 32 * 4;
+    static constexpr int digits()
+    {
+        if constexpr (sizeof(K) == 4 && T * E == 32768) return RadixSmem<T, E, 6>::kBytes;
+        else return 0;
+    }
+    static constexpr int kBytes = kBins > digits() ? kBins : digits();
+};
+
+// One phase pair (even, then odd positions) of odd-even transposition over
+// the warp's 32*E keys in blocked order.
+template <typename K, int E>
+__device__ __forceinline__ void transpose_phases(K (&v)[E], int lane)
+{
+#pragma unroll
+    for (int k = 0; k + 1 < E; k += 2) cmp_swap(v[k], v[k + 1]);
+#pragma unroll
+    for (int k = 1; k + 1 < E; k += 2) cmp_swap(v[k], v[k + 1]);
+    const K x = __shfl_down_sync(0xFFFFFFFFu, v[0], 1);
+    const K y = __shfl_up_sync(0xFFFFFFFFu, v[E - 1], 1);
+    if (lane < 31) v[E - 1] = kmin<K>(v[E - 1], x);
+    if (lane > 0) v[0] = kmax<K>(v[0], y);
+}
+
+// Whether the warp's keys (blocked order) still hold an inversion.
+template <typename K, int E>
+__device__ __forceinline__ bool warp_inverted(const K (&v)[E], int lane)
+{
+    bool bad = false;
+#pragma unroll
+    for (int k = 0; k + 1 < E; ++k) bad |= v[k] > v[k + 1];
+    const K x = __shfl_down_sync(0xFFFFFFFFu, v[0], 1);
+    bad |= lane < 31 && v[E - 1] > x;
+    return __any_sync(0xFFFFFFFFu, bad) != 0;
+}
+
+// Monotone maps of a unit's keys, kmin = lo < kmax = hi, to bins [0, NB):
+// bin(key), and fine(key) = the key's place inside its bin as a 32-bit
+// fraction.
+//
+// By key value.
+template <typename K, int NB> struct BinMap;
+
+template <int NB> struct BinMap<uint32_t, NB> {
+    uint32_t base, mult;
+    int lz;
+    __device__ BinMap(uint32_t lo, uint32_t hi)
+    {
+        base = lo;
+        lz = __clz((int)(hi - lo));
+        mult = (uint32_t)((((uint64_t)NB << 32) - 1) / ((uint64_t)((hi - lo) << lz) + 1));
+    }
+    __device__ uint32_t bin(uint32_t key) const { return __umulhi((key - base) << lz, mult); }
+    __device__ uint32_t fine(uint32_t key) const { return ((key - base) << lz) * mult; }
+};
+
+template <int NB> struct BinMap<uint64_t, NB> {
+    uint64_t base;
+    uint32_t mult;
+    int sr, sl;  // the top 32 bits of key - base: >> sr, then << sl
+    __device__ BinMap(uint64_t lo, uint64_t hi)
+    {
+        base = lo;
+        const int z = __clzll((long long)(hi - lo));
+        sr = z < 32 ? 32 - z : 0;
+        sl = z < 32 ? 0 : z - 32;
+        mult = (uint32_t)((((uint64_t)NB << 32) - 1) / ((uint64_t)top(hi) + 1));
+    }
+    __device__ uint32_t top(uint64_t key) const { return (uint32_t)((key - base) >> sr) << sl; }
+    __device__ uint32_t bin(uint64_t key) const { return __umulhi(top(key), mult); }
+    __device__ uint32_t fine(uint64_t key) const { return top(key) * mult; }
+};
+
+// Codes of floats by float value: equal-width bins of [fmin, fmax].  The
+// difference, the product and the rounding to 2^-23 of the range are each
+// monotone, so the map is.
+template <int NB> struct BinMapF32 {
+    float lo, scale;
+    bool ok;
+    __device__ BinMapF32(uint32_t lo_code, uint32_t hi_code)
+    {
+        lo = __uint_as_float(f32_decode(lo_code));
+        const float d = __uint_as_float(f32_decode(hi_code)) - lo;
+        // (the margin keeps the rounded product inside [0, 2^23))
+        scale = 8388600.0f / d;
+        ok = d > 0.0f && d < 3.0e38f && scale > 0.0f && scale < 3.0e38f;  // false with NaN, inf
+    }
+    __device__ uint32_t place(uint32_t key) const  // 2^23 + place, as float bits
+    {
+        return __float_as_uint(
+            fmaf(__uint_as_float(f32_decode(key)) - lo, scale, 8388608.0f));
+    }
+    static constexpr int kShift = 23 - __builtin_ctz(NB);
+    __device__ uint32_t bin(uint32_t key) const { return (place(key) >> kShift) & (uint32_t)(NB - 1); }
+    __device__ uint32_t fine(uint32_t key) const { return place(key) << (32 - kShift); }
+};
+
+// Ranges below NB: value x of the range has the rep bins [x*rep, (x+1)*rep),
+// a power of two up to 32, spread over the lanes.
+template <typename K, int NB> struct BinMapExact {
+    K base;
+    int shift;
+    uint32_t off;
+    __device__ BinMapExact(K lo, K hi, int lane)
+    {
+        base = lo;
+        const uint32_t per = (uint32_t)NB / ((uint32_t)(hi - lo) + 1u);  // >= 1
+        shift = min(31 - __clz((int)per), 5);
+        off = (uint32_t)lane & ((1u << shift) - 1u);
+    }
+    __device__ uint32_t bin(K key) const { return ((uint32_t)(key - base) << shift) + off; }
+};
+
+// The shape of one CTA's bin sort and its steps.
+template <typename K, int T, int E>
+struct BinSort {
+    static constexpr int NB = bin_count<K, T, E>();
+    static constexpr int CAP = T * E;
+    static constexpr int W = 32 * E;      // keys of a warp
+    static constexpr int NWARP = T / 32;
+    static constexpr int NW = NB / 2;     // counter words
+    static constexpr int IT = NW / NWARP / 128;  // 16-byte words a lane scans
+    static constexpr int SK = E / 8;      // keys per thread of bin_skewed's test
+    static_assert(T % 32 == 0 && T >= 64 && T <= 1024 && E % 8 == 0, "whole warps");
+    static_assert((NB & (NB - 1)) == 0 && NB <= 32768 && IT >= 1, "power-of-two bins, whole words");
+    static_assert(CAP <= 32768, "counts and ranks fit 16 bits");
+
+    K *sm;
+    int len, tid, lane, warp;
+    bool full, act;  // the warp holds no padding / any real key
+    uint32_t cbase;  // shared address of the counters
+
+    __device__ BinSort(K *sm_, int len_) : sm(sm_), len(len_)
+    {
+        tid = (int)threadIdx.x;
+        lane = tid & 31;
+        warp = tid >> 5;
+        full = (warp + 1) * W <= len;
+        act = warp * W < len;
+        cbase = smem_u32addr(sm) + (uint32_t)BinSmem<K, T, E>::kKeyBytes;
+    }
+    // shared address of bin b's counter word and the bin's half
+    __device__ uint32_t word(uint32_t b) const { return cbase + ((b & (uint32_t)(NW - 1)) << 2); }
+    static __device__ uint32_t half(uint32_t b) { return (b / (uint32_t)NW) << 4; }
+    __device__ bool real(int k) const { return wb_pos<E>(warp, lane, k) < len; }
+    __device__ uint32_t spare() const { return cbase + 4u * (uint32_t)(NW + lane); }
+    __device__ uint4 *counters() const
+    {
+        return reinterpret_cast<uint4 *>(reinterpret_cast<unsigned char *>(sm) +
+                                         BinSmem<K, T, E>::kKeyBytes);
+    }
+
+    template <bool FULL, typename F>
+    __device__ __forceinline__ void count(const K (&v)[E], const F &map) const
+    {
+#pragma unroll
+        for (int k = 0; k < E; ++k) {
+            const uint32_t b = map.bin(v[k]);
+            red_add_shared(FULL || real(k) ? word(b) : spare(), 1u << half(b));
+        }
+    }
+    // Exclusive scan of the counters at `in` (NB of them) into `out`, in bin
+    // order; returns the largest count.  s_a, s_b: a word per warp.
+    __device__ __forceinline__ uint32_t scan(const uint4 *in, uint4 *out, uint32_t *s_a,
+                                             uint32_t *s_b) const
+    {
+        // warp w scans words [w*NW/NWARP, (w+1)*NW/NWARP), 128 at a time
+        const int at = warp * (NW / NWARP / 4) + lane;
+        uint32_t gm = 0, s = 0;
+#pragma unroll 2  // (the keys stay live in registers)
+        for (int i = 0; i < IT; ++i) {
+            const uint4 c = in[at + i * 32];
+            gm = __vmaxu2(gm, __vmaxu2(__vmaxu2(c.x, c.y), __vmaxu2(c.z, c.w)));
+            s += c.x + c.y + c.z + c.w;
+        }
+        s = __reduce_add_sync(0xFFFFFFFFu, s);
+        gm = __reduce_max_sync(0xFFFFFFFFu, max(gm & 0xFFFFu, gm >> 16));
+        if (lane == 0) {
+            s_a[warp] = s;
+            s_b[warp] = gm;
+        }
+        __syncthreads();
+        uint32_t inc = lane < NWARP ? s_a[lane % NWARP] : 0u;
+        const uint32_t own = inc;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, inc, d);
+            if (lane >= d) inc += y;
+        }
+        const uint32_t total = __shfl_sync(0xFFFFFFFFu, inc, 31);
+        uint32_t run = __shfl_sync(0xFFFFFFFFu, inc - own, warp);
+        const uint32_t G = __reduce_max_sync(0xFFFFFFFFu, s_b[lane % NWARP]);
+        run += (total & 0xFFFFu) << 16;  // high-half bins follow every low-half one
+#pragma unroll 1
+        for (int i = 0; i < IT; ++i) {
+            const uint4 c = in[at + i * 32];
+            const uint32_t sum = c.x + c.y + c.z + c.w;
+            inc = sum;
+#pragma unroll
+            for (int d = 1; d < 32; d <<= 1) {
+                const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, inc, d);
+                if (lane >= d) inc += y;
+            }
+            uint4 o;
+            o.x = run + inc - sum;
+            o.y = o.x + c.x;
+            o.z = o.y + c.y;
+            o.w = o.z + c.z;
+            out[at + i * 32] = o;
+            run += __shfl_sync(0xFFFFFFFFu, inc, 31);
+        }
+        __syncthreads();
+        return G;
+    }
+    template <bool FULL, typename F>
+    __device__ __forceinline__ void scatter(const K (&v)[E], const F &map) const
+    {
+        constexpr int GB = 4;  // atomics in flight per batch
+#pragma unroll
+        for (int k0 = 0; k0 < E; k0 += GB) {
+            uint32_t r[GB];
+#pragma unroll
+            for (int j = 0; j < GB; ++j) {
+                const uint32_t b = map.bin(v[k0 + j]);
+                const uint32_t a = FULL || real(k0 + j) ? word(b) : spare();
+                // (a rank is below CAP; the mask keeps every store inside
+                // the key area whatever the counters hold)
+                r[j] = (atom_add_shared(a, 1u << half(b)) >> half(b)) & (uint32_t)(CAP - 1);
+            }
+#pragma unroll
+            for (int j = 0; j < GB; ++j)
+                if (FULL || real(k0 + j)) sm[pidx<K>((int)r[j])] = v[k0 + j];
+        }
+    }
+    __device__ __forceinline__ void pad() const  // the positions behind the real keys
+    {
+        for (int x = len + tid; x < CAP; x += T) sm[pidx<K>(x)] = KeyMax<K>::v;
+    }
+};
+
+// Sort of a unit whose first bins are crowded, the largest with G keys (out
+// of line: its comparison sorts must not take registers from the usual
+// path).  The keys are in sm at their warp-blocked positions, the first bins'
+// exclusive prefix P in the counters.
+template <typename K, int T, int E, typename F>
+__device__ __noinline__ void bin_skewed(K *sm, int len, const F map, uint32_t G)
+{
+    using B = BinSort<K, T, E>;
+    constexpr int CAP = B::CAP, W = B::W, NWARP = B::NWARP, NW = B::NW;
+    static_assert(B::NB == CAP, "the refined bins are positions of the order");
+    static_assert(CAP * 2 <= BinSmem<K, T, E>::kKeyBytes, "their counters fit the key area");
+    __shared__ uint32_t s_a[NWARP], s_b[NWARP];
+    const B s(sm, len);
+    const int tid = s.tid, lane = s.lane, warp = s.warp;
+    K v[E];
+#pragma unroll
+    for (int k = 0; k < E; ++k) v[k] = sm[pidx<K>(wb_pos<E>(warp, lane, k))];
+    __syncthreads();
+    if (G > (uint32_t)len / 4u) {
+        // of an eighth of the keys, those whose bin also holds another value:
+        // one key of each bin is left in the key area (any), the others compare
+#pragma unroll
+        for (int k = 0; k < B::SK; ++k)
+            if (s.real(k)) sm[map.bin(v[k]) & (uint32_t)(CAP - 1)] = v[k];
+        __syncthreads();
+        uint32_t mixed = 0, cnt = 0;
+#pragma unroll
+        for (int k = 0; k < B::SK; ++k) {
+            if (s.real(k)) {
+                ++cnt;
+                mixed += sm[map.bin(v[k]) & (uint32_t)(CAP - 1)] != v[k];
+            }
+        }
+        mixed = __reduce_add_sync(0xFFFFFFFFu, mixed);
+        cnt = __reduce_add_sync(0xFFFFFFFFu, cnt);
+        if (lane == 0) {
+            s_a[warp] = mixed;
+            s_b[warp] = cnt;
+        }
+        __syncthreads();
+        mixed = __reduce_add_sync(0xFFFFFFFFu, lane < NWARP ? s_a[lane % NWARP] : 0u);
+        cnt = __reduce_add_sync(0xFFFFFFFFu, lane < NWARP ? s_b[lane % NWARP] : 0u);
+        __syncthreads();  // s_a and the key area are written again
+        if (mixed > cnt / 4u) {
+            if constexpr (sizeof(K) == 4 && CAP == 32768) cta_radix_sort<T, E, 6>(v, sm, len);
+            else cta_sort<K, T, E>(v, sm, len);
+            return;
+        }
+    }
+    uint32_t *fine = reinterpret_cast<uint32_t *>(sm);  // the refined bins' counters
+    for (int i = tid; i < CAP / 8; i += T)
+        reinterpret_cast<uint4 *>(fine)[i] = make_uint4(0u, 0u, 0u, 0u);
+    __syncthreads();
+    const uint32_t *P = reinterpret_cast<const uint32_t *>(s.counters());
+    const uint32_t fbase = smem_u32addr(fine);
+    uint32_t bins[E / 2];  // the keys' refined bins, two to a word
+    auto recount = [&](auto full) {
+        constexpr int GB = 8;
+#pragma unroll
+        for (int k0 = 0; k0 < E; k0 += GB) {
+            uint32_t p0[GB], p1[GB];
+#pragma unroll
+            for (int j = 0; j < GB; ++j) {
+                const uint32_t b = map.bin(v[k0 + j]) & (uint32_t)(B::NB - 1), e = b + 1;
+                p0[j] = (P[b & (uint32_t)(NW - 1)] >> B::half(b)) & 0xFFFFu;
+                p1[j] = e < (uint32_t)B::NB ? (P[e & (uint32_t)(NW - 1)] >> B::half(e)) & 0xFFFFu
+                                            : (uint32_t)len;
+            }
+#pragma unroll
+            for (int j = 0; j < GB; ++j) {
+                const int k = k0 + j;
+                const uint32_t w = p1[j] - p0[j];
+                const int sh = w >= (uint32_t)(CAP / 8) ? 4 : 0;
+                const uint32_t b2 = (p0[j] + (__umulhi(map.fine(v[k]), w >> sh) << sh) +
+                                     ((uint32_t)lane & ((1u << sh) - 1u))) & (uint32_t)(CAP - 1);
+                if (k & 1) bins[k / 2] |= b2 << 16;
+                else bins[k / 2] = b2;
+                red_add_shared(decltype(full)::value || s.real(k)
+                                   ? fbase + ((b2 & (uint32_t)(NW - 1)) << 2) : s.spare(),
+                               1u << B::half(b2));
+            }
+        }
+    };
+    if (s.full) recount(std::true_type{});
+    else if (s.act) recount(std::false_type{});
+    __syncthreads();
+    s.scan(reinterpret_cast<const uint4 *>(fine), s.counters(), s_a, s_b);
+    auto place = [&](auto full) {
+        constexpr int GB = 8;
+#pragma unroll
+        for (int k0 = 0; k0 < E; k0 += GB) {
+            uint32_t r[GB];
+#pragma unroll
+            for (int j = 0; j < GB; ++j) {
+                const int k = k0 + j;
+                const uint32_t b = (bins[k / 2] >> (16 * (k & 1))) & 0xFFFFu;
+                const uint32_t a = decltype(full)::value || s.real(k) ? s.word(b) : s.spare();
+                r[j] = (atom_add_shared(a, 1u << B::half(b)) >> B::half(b)) & (uint32_t)(CAP - 1);
+            }
+#pragma unroll
+            for (int j = 0; j < GB; ++j)
+                if (decltype(full)::value || s.real(k0 + j)) sm[pidx<K>((int)r[j])] = v[k0 + j];
+        }
+    };
+    if (s.full) place(std::true_type{});
+    else if (s.act) place(std::false_type{});
+    s.pad();
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < E; ++k) v[k] = sm[pidx<K>(tid * E + k)];
+    if (s.act) {
+        bool bad = warp_inverted<K, E>(v, lane);
+#pragma unroll 1
+        for (uint32_t p = 0; bad && p < kBinPhases; p += 8) {
+#pragma unroll 1
+            for (int q = 0; q < 4; ++q) transpose_phases<K, E>(v, lane);
+            bad = warp_inverted<K, E>(v, lane);
+        }
+        if (bad) {
+            sort_network<E>(v);
+            warp_merge_levels<K, E>(v, lane);
+        }
+#pragma unroll
+        for (int k = 0; k < E; ++k) sm[pidx<K>(tid * E + k)] = v[k];
+    }
+    __syncthreads();
+    const int b = warp * W;
+    if (__syncthreads_or(warp > 0 && s.act && sm[pidx<K>(b - 1)] > sm[pidx<K>(b)])) {
+        // (runs of odd warps are stored descending for the merge levels)
+        store_run<K, E>(sm, b, W, lane * E, (warp & 1) != 0, v);
+        __syncthreads();
+        cta_merge_runs<K, T, E>(sm, W);
+    }
+}
+
+// Sort the CTA's T*E keys v ascending into sm (padded layout pidx, then the
+// counters: BinSmem<K, T, E>::kBytes in all).  On entry v holds the keys in
+// the warp-blocked layout; positions >= len are padding holding the maximal
+// key.  On return sm[pidx(x)] is the x-th smallest key, padding after the
+// len real ones, as cta_sort leaves it.  is_f32: 32-bit keys are codes of
+// floats.  Ends with __syncthreads().
+template <typename K, int T, int E>
+__device__ __forceinline__ void cta_bin_sort(K (&v)[E], K *sm, int len, bool is_f32)
+{
+    using B = BinSort<K, T, E>;
+    constexpr int W = B::W, NWARP = B::NWARP, NB = B::NB;
+    __shared__ K s_lo[NWARP], s_hi[NWARP];
+    __shared__ uint32_t s_a[NWARP], s_b[NWARP];
+    const B s(sm, len);
+    const int lane = s.lane, warp = s.warp;
+    // smallest and largest real key; counters to zero
+    K lo = KeyMax<K>::v, hi = 0;
+    if (s.full) {
+#pragma unroll
+        for (int k = 0; k < E; ++k) {
+            lo = kmin<K>(lo, v[k]);
+            hi = kmax<K>(hi, v[k]);
+        }
+    } else if (s.act) {
+#pragma unroll
+        for (int k = 0; k < E; ++k)
+            if (s.real(k)) {
+                lo = kmin<K>(lo, v[k]);
+                hi = kmax<K>(hi, v[k]);
+            }
+    }
+    auto warp_lo = [&](K x) {
+        if constexpr (sizeof(K) == 4) {
+            return __reduce_min_sync(0xFFFFFFFFu, x);
+        } else {
+#pragma unroll
+            for (int d = 16; d >= 1; d >>= 1) x = kmin<K>(x, __shfl_xor_sync(0xFFFFFFFFu, x, d));
+            return x;
+        }
+    };
+    auto warp_hi = [&](K x) {
+        if constexpr (sizeof(K) == 4) {
+            return __reduce_max_sync(0xFFFFFFFFu, x);
+        } else {
+#pragma unroll
+            for (int d = 16; d >= 1; d >>= 1) x = kmax<K>(x, __shfl_xor_sync(0xFFFFFFFFu, x, d));
+            return x;
+        }
+    };
+    lo = warp_lo(lo);
+    hi = warp_hi(hi);
+    if (lane == 0) {
+        s_lo[warp] = lo;
+        s_hi[warp] = hi;
+    }
+    uint4 *cnt = s.counters();
+    for (int i = s.tid; i < NB / 8; i += T) cnt[i] = make_uint4(0u, 0u, 0u, 0u);
+    __syncthreads();
+    lo = warp_lo(s_lo[lane % NWARP]);
+    hi = warp_hi(s_hi[lane % NWARP]);
+    if (hi <= lo) {  // no real key, or all of them equal
+#pragma unroll 4
+        for (int k = 0; k < E; ++k) {
+            const int x = k * T + s.tid;
+            sm[pidx<K>(x)] = x < len ? lo : KeyMax<K>::v;
+        }
+        __syncthreads();
+        return;
+    }
+    uint32_t G = 0;
+    // steps 1-3: true when step 4 is still to do
+    auto distribute = [&](const auto &map, auto fill) -> bool {
+        if (s.full) s.template count<true>(v, map);
+        else if (s.act) s.template count<false>(v, map);
+        __syncthreads();
+        G = s.scan(cnt, cnt, s_a, s_b);
+        if constexpr (decltype(fill)::value) {
+            if (G > kBinPhases) {
+#pragma unroll
+                for (int k = 0; k < E; ++k) sm[pidx<K>(wb_pos<E>(warp, lane, k))] = v[k];
+                __syncthreads();
+                bin_skewed<K, T, E>(sm, len, map, G);
+                return false;
+            }
+        }
+        if (s.full) s.template scatter<true>(v, map);
+        else if (s.act) s.template scatter<false>(v, map);
+        s.pad();
+        __syncthreads();
+        return decltype(fill)::value;
+    };
+    if (hi - lo < (K)NB) {
+        distribute(BinMapExact<K, NB>(lo, hi, lane), std::false_type{});
+        return;
+    }
+    bool more;
+    if constexpr (sizeof(K) == 4) {
+        const BinMapF32<NB> fmap(lo, hi);
+        if (is_f32 && fmap.ok) more = distribute(fmap, std::true_type{});
+        else more = distribute(BinMap<K, NB>(lo, hi), std::true_type{});
+    } else {
+        more = distribute(BinMap<K, NB>(lo, hi), std::true_type{});
+    }
+    if (!more) return;
+    // 4. order the keys inside the bins
+    if (s.act) {
+#pragma unroll
+        for (int k = 0; k < E; ++k) v[k] = sm[pidx<K>(s.tid * E + k)];
+#pragma unroll 1
+        for (uint32_t p = 0; p < G; p += 2) transpose_phases<K, E>(v, lane);
+#pragma unroll
+        for (int k = 0; k < E; ++k) sm[pidx<K>(s.tid * E + k)] = v[k];
+    }
+    __syncthreads();
+    if (warp > 0 && s.act) {
+        // bins that straddle this warp's first key: the last 32 keys before
+        // it and the first 32 from it, each ascending
+        const int b = warp * W;
+        const K x = sm[pidx<K>(b - 32 + lane)], y = sm[pidx<K>(b + 31 - lane)];
+        K l = kmin<K>(x, y), h = kmax<K>(x, y);
+#pragma unroll
+        for (int d = 16; d >= 1; d >>= 1) {
+            const K xl = __shfl_xor_sync(0xFFFFFFFFu, l, d);
+            const K xh = __shfl_xor_sync(0xFFFFFFFFu, h, d);
+            const bool low = (lane & d) == 0;
+            l = low ? kmin<K>(l, xl) : kmax<K>(l, xl);
+            h = low ? kmin<K>(h, xh) : kmax<K>(h, xh);
+        }
+        sm[pidx<K>(b - 32 + lane)] = l;
+        sm[pidx<K>(b + lane)] = h;
+    }
+    __syncthreads();
+}
+
+}  // namespace bsort

@@ -29,24 +29,24 @@ cudaError_t init_sort_pairs_kernels();
 // `ctas` CTAs of `chunk` items each; write the sorted sublists (keys, and
 // values for pairs) and s sample records per sublist.
 // Steps 1-3 for sublists tile0 .. tile0 + m - 1.
-// radix: a sublist of 32768 keys sorted by one CTA is sorted by digits
-// (cta_radix_sort) instead of by comparisons; both give the same sublists.
+// bins: a sublist of 32768 keys sorted by one CTA is sorted by bins
+// (cta_bin_sort) instead of by comparisons; both give the same sublists.
 cudaError_t launch_sublist_sort_keys(int chunk, int ctas, const void *keys_in, uint64_t n,
                                      uint32_t m, int is_f32, uint32_t s, uint32_t *tiles_k,
                                      uint64_t *samples, cudaStream_t st, uint32_t tile0 = 0,
-                                     bool radix = false);
-// The radix-sorting forms (bsort_sort_keys_radix.cu) that the functions
-// above call for units of 32768 keys sorted by one CTA when `radix` is set.
-cudaError_t init_sort_keys_radix_kernels();
-cudaError_t launch_sublist_sort_keys_radix(int ctas, const void *keys_in, uint64_t n, uint32_t m,
+                                     bool bins = false);
+// The forms by bins (bsort_sort_keys_bins.cu) that the functions
+// above call for units of 32768 keys sorted by one CTA when `bins` is set.
+cudaError_t init_sort_keys_bins_kernels();
+cudaError_t launch_sublist_sort_keys_bins(int ctas, const void *keys_in, uint64_t n, uint32_t m,
                                            int is_f32, uint32_t s, uint32_t *tiles_k,
                                            uint64_t *samples, cudaStream_t st, uint32_t tile0);
 struct GatherSrc;
-cudaError_t launch_bucket_sort_keys_radix(int ctas, const void *src_k, const uint32_t *units,
+cudaError_t launch_bucket_sort_keys_bins(int ctas, const void *src_k, const uint32_t *units,
                                           uint32_t max_units, uint64_t n, uint64_t n_pad,
                                           int is_f32, void *out_k, int *err, const GatherSrc &g,
                                           cudaStream_t st);
-cudaError_t launch_bucket_sort_keys_range_radix(int ctas, const void *src_k,
+cudaError_t launch_bucket_sort_keys_range_bins(int ctas, const void *src_k,
                                                 const uint32_t *units, const uint32_t *range,
                                                 uint32_t grid_units, uint64_t n, uint64_t n_pad,
                                                 int is_f32, void *out_k, int *err,
@@ -79,14 +79,14 @@ constexpr uint32_t kLoopUnits = 256;
 cudaError_t launch_bucket_sort_keys(int chunk, int ctas, const void *src_k, const uint32_t *units,
                                     uint32_t max_units, uint64_t n, uint64_t n_pad, int is_f32,
                                     void *out_k, int *err, const GatherSrc &g, cudaStream_t st,
-                                    bool radix = false);
+                                    bool bins = false);
 // Step 9 (keys) over units range[0] .. range[1] - 1 of a list, range in
 // device memory, by a grid of grid_units units that loop over them.
 cudaError_t launch_bucket_sort_keys_range(int chunk, int ctas, const void *src_k,
                                           const uint32_t *units, const uint32_t *range,
                                           uint32_t grid_units, uint64_t n, uint64_t n_pad,
                                           int is_f32, void *out_k, int *err, cudaStream_t st,
-                                          bool radix = false);
+                                          bool bins = false);
 // For G position slices [g*n_pad/G, (g+1)*n_pad/G): ranges[g] = first unit of
 // the list whose begin is at or above g*n_pad/G (ranges[G] = the count).
 cudaError_t launch_unit_ranges(const uint32_t *units, uint32_t n_pad, uint32_t G,
@@ -306,10 +306,11 @@ cudaError_t launch_seg_sample_index(const uint32_t *tiles_k, const uint64_t *sam
                                     const uint64_t *spl, const uint32_t *sub_seg, uint32_t nsub,
                                     const SegInfo *segs, uint32_t *counts, uint32_t *srcb,
                                     cudaStream_t st);
-// Step 9: unit u = bucket units[2u+1] of segment units[2u], `chunk` keys max.
-cudaError_t launch_seg_bucket_sort(int chunk, const uint32_t *reloc_k, const uint32_t *units,
-                                   uint32_t nunits, const SegInfo *segs, const uint32_t *offsets,
-                                   int is_f32, uint32_t *keys_out, int *err, cudaStream_t st);
+// Step 9: unit u = bucket units[2u+1] of segment units[2u], at most kSegTile
+// keys.
+cudaError_t launch_seg_bucket_sort(const uint32_t *reloc_k, const uint32_t *units, uint32_t nunits,
+                                   const SegInfo *segs, const uint32_t *offsets, int is_f32,
+                                   uint32_t *keys_out, int *err, cudaStream_t st);
 // Sampled segments of 64-bit keys: the same steps with sublists of
 // kSegTileU64 keys, sample records (key, p) of 16 bytes (Steps 4-5 need
 // m*s <= 8192) and Step-9 units of at most kSegTileU64 keys; Steps 7-8 are

@@ -10,33 +10,63 @@
 // each value from its position afterwards.
 #pragma once
 
+#include "bsort_binsort.cuh"
 #include "bsort_device.cuh"
 #include "bsort_internal.h"
-#include "bsort_radix.cuh"
 
 namespace bsort {
 
-// Digit width of the radix-sorting CTAs (128 digits per pass).
-constexpr int kRadixBits = 7;
-
-// Dynamic shared memory of one sorting CTA: the padded tile, plus the radix
-// sort's counters when the CTA sorts 32-bit keys by digits (RADIX).
-template <typename K, int T, int E, bool RADIX>
+// Dynamic shared memory of one sorting CTA: the padded tile, plus the
+// counters when the CTA sorts 32-bit keys by bins (BINS).
+template <typename K, int T, int E, bool BINS>
 constexpr int sort_smem_bytes()
 {
-    return RADIX ? RadixSmem<T, E, kRadixBits>::kBytes : padded_elems<K>(T * E) * (int)sizeof(K);
+    return BINS ? BinSmem<K, T, E>::kBytes : padded_elems<K>(T * E) * (int)sizeof(K);
 }
 
-// The in-CTA sort of one chunk: the comparison sort (cta_sort) or, for
-// 32-bit keys, the radix sort (cta_radix_sort); both leave the same result.
-template <typename K, int T, int E, bool RADIX>
-__device__ __forceinline__ void chunk_sort(K (&v)[E], K *sm, int len)
+// CTAs per SM that the registers leave room for: the distribution sort of
+// up to 16384 keys takes 64 registers a thread, so that the CTAs of an SM
+// overlap one's memory phases with another's arithmetic (16384-key units on
+// 2^26 keys: 205 us with two 512-thread CTAs per SM, 263 us with one of 1024).
+template <int T, int E, int C, bool BINS>
+constexpr int min_ctas()
 {
-    if constexpr (RADIX) {
-        static_assert(sizeof(K) == 4, "the radix sort takes 32-bit keys");
-        cta_radix_sort<T, E, kRadixBits>(v, sm, len);
+    return BINS && C == 1 && T * E <= 16384 ? 1024 / T : 1;
+}
+
+// The in-CTA sort of one chunk: the comparison sort (cta_sort) or the
+// distribution sort (cta_bin_sort); both leave the same result.
+template <typename K, int T, int E, bool BINS>
+__device__ __forceinline__ void chunk_sort(K (&v)[E], K *sm, int len, bool is_f32)
+{
+    if constexpr (BINS) cta_bin_sort<K, T, E>(v, sm, len, is_f32);
+    else cta_sort<K, T, E>(v, sm, len);
+}
+
+// The warp-blocked load of a chunk: keys src[x] for x < len (all loads of
+// a thread in flight together; float keys are encoded afterwards), the
+// maximal key behind them.
+template <typename K, int T, int E>
+__device__ __forceinline__ void load_keys(K (&v)[E], const K *__restrict__ src, int len,
+                                          bool is_f32)
+{
+    const int lane = (int)threadIdx.x & 31, warp = (int)threadIdx.x >> 5;
+    if ((warp + 1) * 32 * E <= len) {  // no padding in this warp
+#pragma unroll
+        for (int k = 0; k < E; ++k) v[k] = src[wb_pos<E>(warp, lane, k)];
     } else {
-        cta_sort<K, T, E>(v, sm, len);
+#pragma unroll
+        for (int k = 0; k < E; ++k) {
+            const int x = wb_pos<E>(warp, lane, k);
+            v[k] = x < len ? src[x] : KeyMax<K>::v;
+        }
+    }
+    if constexpr (sizeof(K) == 4) {
+        if (is_f32) {
+#pragma unroll
+            for (int k = 0; k < E; ++k)
+                if (wb_pos<E>(warp, lane, k) < len) v[k] = f32_encode(v[k]);
+        }
     }
 }
 
@@ -46,8 +76,8 @@ __device__ __forceinline__ void chunk_sort(K (&v)[E], K *sm, int len)
 // [r*T*E, (r+1)*T*E): it writes them to the sorted-sublist array and emits
 // the samples (ranks (k+1)w - 1) that fall in that range as key << 32 | p,
 // p = i*t + r.
-template <int T, int E, bool PAIRS, int C, bool RADIX = false>
-__global__ void __launch_bounds__(T, 1)
+template <int T, int E, bool PAIRS, int C, bool BINS = false>
+__global__ void __launch_bounds__(T, (min_ctas<T, E, C, BINS>()))
 k_sublist_sort(const uint32_t *__restrict__ keys_in, const void *__restrict__ vals_in,
                uint64_t n, int is_f32, int val_bytes, uint32_t s,
                uint32_t *__restrict__ tiles_k, void *__restrict__ tiles_v,
@@ -72,19 +102,22 @@ k_sublist_sort(const uint32_t *__restrict__ keys_in, const void *__restrict__ va
     }
 
     K v[E];
+    if constexpr (PAIRS) {
 #pragma unroll
-    for (int k = 0; k < E; ++k) {
-        const int x = off + wb_pos<E>(warp, lane, k);
-        uint32_t key = 0xFFFFFFFFu;  // pad sentinel (position >= n)
-        if (x < len) {
-            key = keys_in[base + x];
-            if (is_f32) key = f32_encode(key);
+        for (int k = 0; k < E; ++k) {
+            const int x = off + wb_pos<E>(warp, lane, k);
+            uint32_t key = 0xFFFFFFFFu;  // pad sentinel (position >= n)
+            if (x < len) {
+                key = keys_in[base + x];
+                if (is_f32) key = f32_encode(key);
+            }
+            v[k] = ((uint64_t)key << 32) | (uint32_t)x;
         }
-        if constexpr (PAIRS) v[k] = ((uint64_t)key << 32) | (uint32_t)x;
-        else v[k] = (K)key;
+    } else {
+        load_keys<uint32_t, T, E>(v, keys_in + base + off, len - off, is_f32 != 0);
     }
     const int clen = len - off;
-    chunk_sort<K, T, E, RADIX>(v, sm, clen < 0 ? 0 : (clen > CH ? CH : clen));
+    chunk_sort<K, T, E, BINS>(v, sm, clen < 0 ? 0 : (clen > CH ? CH : clen), is_f32 != 0);
     cluster_merge<K, T, E, C>(sm, len);
 
 #pragma unroll 4
@@ -137,7 +170,7 @@ k_sublist_sort(const uint32_t *__restrict__ keys_in, const void *__restrict__ va
 // each value from that position.
 // prefetch_stride: units between this one and the next this CTA's SM will
 // most likely sort (0: no prefetch), whose keys are then fetched into L2.
-template <int T, int E, bool PAIRS, int C, bool RADIX>
+template <int T, int E, bool PAIRS, int C, bool BINS>
 __device__ __forceinline__ void
 bucket_sort_unit(uint32_t u, const uint32_t *__restrict__ src_k, const void *__restrict__ src_v,
                  const uint32_t *__restrict__ units, uint64_t n, uint64_t n_pad, int is_f32,
@@ -182,7 +215,10 @@ bucket_sort_unit(uint32_t u, const uint32_t *__restrict__ src_k, const void *__r
     const int ustart = r * per;
     const int uend = min(ustart + per, len);
     K v[E];
-    if (!gather) {
+    if (!PAIRS && !gather) {
+        if constexpr (!PAIRS)
+            load_keys<uint32_t, T, E>(v, src_k + L + ustart, uend - ustart, direct && is_f32);
+    } else if (!gather) {
 #pragma unroll
         for (int k = 0; k < E; ++k) {
             const int x = ustart + wb_pos<E>(warp, lane, k);
@@ -234,7 +270,7 @@ bucket_sort_unit(uint32_t u, const uint32_t *__restrict__ src_k, const void *__r
             else v[k] = (K)key;
         }
     }
-    chunk_sort<K, T, E, RADIX>(v, sm, uend > ustart ? uend - ustart : 0);
+    chunk_sort<K, T, E, BINS>(v, sm, uend > ustart ? uend - ustart : 0, is_f32 != 0);
     cluster_merge<K, T, E, C>(sm, len, per);
     const uint64_t lim64 = min((unsigned long long)len, (unsigned long long)(n > L ? n - L : 0));
     const int lim = (int)lim64;
@@ -261,14 +297,14 @@ bucket_sort_unit(uint32_t u, const uint32_t *__restrict__ src_k, const void *__r
 }
 
 // Cluster u of the grid sorts unit u (clusters beyond the unit count exit).
-template <int T, int E, bool PAIRS, int C, bool RADIX = false>
-__global__ void __launch_bounds__(T, 1)
+template <int T, int E, bool PAIRS, int C, bool BINS = false>
+__global__ void __launch_bounds__(T, (min_ctas<T, E, C, BINS>()))
 k_bucket_sort(const uint32_t *__restrict__ src_k, const void *__restrict__ src_v,
               const uint32_t *__restrict__ units, uint64_t n, uint64_t n_pad, int is_f32,
               int val_bytes, uint32_t *__restrict__ out_k, void *__restrict__ out_v, int *err,
               GatherSrc g)
 {
-    bucket_sort_unit<T, E, PAIRS, C, RADIX>(blockIdx.x / C, src_k, src_v, units, n, n_pad, is_f32,
+    bucket_sort_unit<T, E, PAIRS, C, BINS>(blockIdx.x / C, src_k, src_v, units, n, n_pad, is_f32,
                                      val_bytes, out_k, out_v, err, g, num_sms() / C);
 }
 
@@ -277,8 +313,8 @@ k_bucket_sort(const uint32_t *__restrict__ src_k, const void *__restrict__ src_v
 // device memory, range[0] .. range[1] - 1): a small grid whose cluster c
 // sorts units lo + c, lo + c + G, ... (G clusters; every CTA of a cluster
 // takes the same units).
-template <int T, int E, bool PAIRS, int C, bool RADIX = false>
-__global__ void __launch_bounds__(T, 1)
+template <int T, int E, bool PAIRS, int C, bool BINS = false>
+__global__ void __launch_bounds__(T, (min_ctas<T, E, C, BINS>()))
 k_bucket_sort_loop(const uint32_t *__restrict__ src_k, const void *__restrict__ src_v,
                    const uint32_t *__restrict__ units, uint64_t n, uint64_t n_pad, int is_f32,
                    int val_bytes, uint32_t *__restrict__ out_k, void *__restrict__ out_v,
@@ -288,7 +324,7 @@ k_bucket_sort_loop(const uint32_t *__restrict__ src_k, const void *__restrict__ 
     const uint32_t count = range != nullptr ? range[1] : units[0];
 #pragma unroll 1
     for (uint32_t u = lo + blockIdx.x / C; u < count; u += gridDim.x / C) {
-        bucket_sort_unit<T, E, PAIRS, C, RADIX>(u, src_k, src_v, units, n, n_pad, is_f32, val_bytes,
+        bucket_sort_unit<T, E, PAIRS, C, BINS>(u, src_k, src_v, units, n, n_pad, is_f32, val_bytes,
                                          out_k, out_v, err, g, gridDim.x / C);
         __syncthreads();  // shared memory is reused by the next unit
     }
@@ -314,44 +350,44 @@ inline cudaError_t launch_maybe_cluster(KernelT kern, unsigned grid, int block, 
     return cudaLaunchKernelEx(&cfg, kern, args...);
 }
 
-template <int T, int E, bool PAIRS, int C, bool RADIX = false>
+template <int T, int E, bool PAIRS, int C, bool BINS = false>
 inline cudaError_t init_sort_pair_of_kernels()
 {
     using K = typename std::conditional<PAIRS, uint64_t, uint32_t>::type;
-    const int sm = sort_smem_bytes<K, T, E, RADIX>();
-    cudaError_t e = cudaFuncSetAttribute(k_sublist_sort<T, E, PAIRS, C, RADIX>,
+    const int sm = sort_smem_bytes<K, T, E, BINS>();
+    cudaError_t e = cudaFuncSetAttribute(k_sublist_sort<T, E, PAIRS, C, BINS>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
     if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(k_bucket_sort<T, E, PAIRS, C, RADIX>,
+    e = cudaFuncSetAttribute(k_bucket_sort<T, E, PAIRS, C, BINS>,
                              cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
     if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(k_bucket_sort_loop<T, E, PAIRS, C, RADIX>,
+    e = cudaFuncSetAttribute(k_bucket_sort_loop<T, E, PAIRS, C, BINS>,
                              cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
     if (e != cudaSuccess) return e;
     if (C > 8) {
-        e = cudaFuncSetAttribute(k_sublist_sort<T, E, PAIRS, C, RADIX>,
+        e = cudaFuncSetAttribute(k_sublist_sort<T, E, PAIRS, C, BINS>,
                                  cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
         if (e != cudaSuccess) return e;
-        e = cudaFuncSetAttribute(k_bucket_sort<T, E, PAIRS, C, RADIX>,
+        e = cudaFuncSetAttribute(k_bucket_sort<T, E, PAIRS, C, BINS>,
                                  cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     }
     return e;
 }
 
-template <int T, int E, bool PAIRS, int C, bool RADIX = false>
+template <int T, int E, bool PAIRS, int C, bool BINS = false>
 inline cudaError_t launch_sublist_sort_t(const void *keys_in, const void *vals_in, uint64_t n,
                                          uint32_t m, int is_f32, int val_bytes, uint32_t s,
                                          uint32_t *tiles_k, void *tiles_v, uint64_t *samples,
                                          uint32_t tile0, cudaStream_t st)
 {
     using K = typename std::conditional<PAIRS, uint64_t, uint32_t>::type;
-    const int sm = sort_smem_bytes<K, T, E, RADIX>();
-    return launch_maybe_cluster(k_sublist_sort<T, E, PAIRS, C, RADIX>, m * C, T, sm, C, st,
+    const int sm = sort_smem_bytes<K, T, E, BINS>();
+    return launch_maybe_cluster(k_sublist_sort<T, E, PAIRS, C, BINS>, m * C, T, sm, C, st,
                                 static_cast<const uint32_t *>(keys_in), vals_in, n, is_f32,
                                 val_bytes, s, tiles_k, tiles_v, samples, tile0);
 }
 
-template <int T, int E, bool PAIRS, int C, bool RADIX = false>
+template <int T, int E, bool PAIRS, int C, bool BINS = false>
 inline cudaError_t launch_bucket_sort_t(const void *src_k, const void *src_v,
                                         const uint32_t *units, uint32_t max_units, uint64_t n,
                                         uint64_t n_pad, int is_f32, int val_bytes, void *out_k,
@@ -359,14 +395,14 @@ inline cudaError_t launch_bucket_sort_t(const void *src_k, const void *src_v,
                                         cudaStream_t st)
 {
     using K = typename std::conditional<PAIRS, uint64_t, uint32_t>::type;
-    const int sm = sort_smem_bytes<K, T, E, RADIX>();
+    const int sm = sort_smem_bytes<K, T, E, BINS>();
     const unsigned grid = (units ? max_units : 1u) * C;
     if (C > 1 && units != nullptr && max_units <= kLoopUnits)
-        return launch_maybe_cluster(k_bucket_sort_loop<T, E, PAIRS, C, RADIX>, grid, T, sm, C, st,
+        return launch_maybe_cluster(k_bucket_sort_loop<T, E, PAIRS, C, BINS>, grid, T, sm, C, st,
                                     static_cast<const uint32_t *>(src_k), src_v, units, n, n_pad,
                                     is_f32, val_bytes, static_cast<uint32_t *>(out_k), out_v,
                                     err, g, (const uint32_t *)nullptr);
-    return launch_maybe_cluster(k_bucket_sort<T, E, PAIRS, C, RADIX>, grid, T, sm, C, st,
+    return launch_maybe_cluster(k_bucket_sort<T, E, PAIRS, C, BINS>, grid, T, sm, C, st,
                                 static_cast<const uint32_t *>(src_k), src_v, units, n, n_pad,
                                 is_f32, val_bytes, static_cast<uint32_t *>(out_k), out_v, err, g);
 }
@@ -374,27 +410,27 @@ inline cudaError_t launch_bucket_sort_t(const void *src_k, const void *src_v,
 // Step 9 over the units range[0] .. range[1] - 1 of a list (device memory),
 // by a grid of grid_units clusters (C > 1) or of grid_units SMs' worth of
 // CTAs (C = 1) that loop over them.
-template <int T, int E, bool PAIRS, int C, bool RADIX = false>
+template <int T, int E, bool PAIRS, int C, bool BINS = false>
 inline cudaError_t launch_bucket_sort_range_t(const void *src_k, const uint32_t *units,
                                               const uint32_t *range, uint32_t grid_units,
                                               uint64_t n, uint64_t n_pad, int is_f32,
                                               void *out_k, int *err, cudaStream_t st)
 {
     using K = typename std::conditional<PAIRS, uint64_t, uint32_t>::type;
-    const int sm = sort_smem_bytes<K, T, E, RADIX>();
+    const int sm = sort_smem_bytes<K, T, E, BINS>();
     const GatherSrc none;
     if (C == 1) {
         // grid_units counts SMs: as many CTAs as fit on them at once
         static const int per_sm = [sm] {
             int o = 0;
             if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-                    &o, k_bucket_sort_loop<T, E, PAIRS, C, RADIX>, T, sm) != cudaSuccess)
+                    &o, k_bucket_sort_loop<T, E, PAIRS, C, BINS>, T, sm) != cudaSuccess)
                 o = 1;
             return o < 1 ? 1 : o;
         }();
         grid_units *= (uint32_t)per_sm;
     }
-    return launch_maybe_cluster(k_bucket_sort_loop<T, E, PAIRS, C, RADIX>, grid_units * C, T, sm, C, st,
+    return launch_maybe_cluster(k_bucket_sort_loop<T, E, PAIRS, C, BINS>, grid_units * C, T, sm, C, st,
                                 static_cast<const uint32_t *>(src_k), (const void *)nullptr, units,
                                 n, n_pad, is_f32, 0, static_cast<uint32_t *>(out_k),
                                 (void *)nullptr, err, none, range);
