@@ -32,7 +32,7 @@ namespace bsort {
 // C*T*E keys, guaranteed by the host) into the same range of the output.
 // K: uint32_t (uint32 / float32 keys) or uint64_t (64-bit keys).
 template <typename K, int T, int E, int C, bool BINS>
-__global__ void __launch_bounds__(T, (min_ctas<T, E, C, BINS>()))
+__global__ void __launch_bounds__(T, (min_ctas<K, T, E, C, BINS>()))
 k_seg_sort(const K *__restrict__ keys_in, K *__restrict__ keys_out,
            const uint32_t *__restrict__ seg, int is_f32, int *err)
 {
@@ -40,7 +40,6 @@ k_seg_sort(const K *__restrict__ keys_in, K *__restrict__ keys_out,
     extern __shared__ __align__(16) unsigned char smem_raw[];
     K *sm = reinterpret_cast<K *>(smem_raw);
     const int tid = threadIdx.x;
-    const int lane = tid & 31, warp = tid >> 5;
     const uint32_t u = blockIdx.x / C;
     const int r = (int)(blockIdx.x % C);
     const uint32_t L = seg[2 * u], R = seg[2 * u + 1];
@@ -86,7 +85,6 @@ k_seg_sublist_sort(const uint32_t *__restrict__ keys_in, int is_f32,
     extern __shared__ __align__(16) unsigned char smem_raw[];
     uint32_t *sm = reinterpret_cast<uint32_t *>(smem_raw);
     const int tid = threadIdx.x;
-    const int lane = tid & 31, warp = tid >> 5;
     const uint32_t g = blockIdx.x;
     const SegInfo sg = segs[sub_seg[g]];
     const uint32_t i = g - sg.g0;
@@ -205,7 +203,7 @@ k_seg_sample_index(const uint32_t *__restrict__ tiles_k, const uint64_t *__restr
 // g0*t < n) to the segment's output range.  K: uint32_t (uint32 / float32
 // keys) or uint64_t (64-bit keys).
 template <typename K, int T, int E, bool BINS>
-__global__ void __launch_bounds__(T, (min_ctas<T, E, 1, BINS>()))
+__global__ void __launch_bounds__(T, (min_ctas<K, T, E, 1, BINS>()))
 k_seg_bucket_sort(const K *__restrict__ reloc_k, const uint32_t *__restrict__ units,
                   const SegInfo *__restrict__ segs, const uint32_t *__restrict__ offsets,
                   uint32_t t, int is_f32, K *__restrict__ keys_out, int *err)
@@ -214,7 +212,6 @@ k_seg_bucket_sort(const K *__restrict__ reloc_k, const uint32_t *__restrict__ un
     extern __shared__ __align__(16) unsigned char smem_raw[];
     K *sm = reinterpret_cast<K *>(smem_raw);
     const int tid = threadIdx.x;
-    const int lane = tid & 31, warp = tid >> 5;
     const uint32_t u = blockIdx.x;
     const SegInfo sg = segs[units[2 * u]];
     const uint32_t j = units[2 * u + 1];
@@ -268,7 +265,6 @@ k_seg_sublist_sort_u64(const uint64_t *__restrict__ keys_in, const uint32_t *__r
     extern __shared__ __align__(16) unsigned char smem_raw[];
     uint64_t *sm = reinterpret_cast<uint64_t *>(smem_raw);
     const int tid = threadIdx.x;
-    const int lane = tid & 31, warp = tid >> 5;
     const uint32_t g = blockIdx.x;
     const SegInfo sg = segs[sub_seg[g]];
     const uint32_t i = g - sg.g0;
@@ -276,12 +272,8 @@ k_seg_sublist_sort_u64(const uint64_t *__restrict__ keys_in, const uint32_t *__r
     const int len = sg.n - first < (uint32_t)TT ? (int)(sg.n - first) : TT;
     const uint64_t src = (uint64_t)sg.out + first;
     uint64_t v[E];
-#pragma unroll
-    for (int k = 0; k < E; ++k) {
-        const int x = wb_pos<E>(warp, lane, k);
-        v[k] = x < len ? keys_in[src + x] : KeyMax<uint64_t>::v;
-    }
-    cta_sort<uint64_t, T, E>(v, sm, len);
+    load_keys<uint64_t, T, E>(v, keys_in + src, len, false);
+    cta_bin_sort<uint64_t, T, E>(v, sm, len, false);
     const uint64_t base = (uint64_t)g * TT;
 #pragma unroll 4
     for (int k = 0; k < E; ++k) {
@@ -448,9 +440,9 @@ bool batch_wide_cluster16()
 {
     if (g_wide16 < 0) {
         // non-portable cluster size: usable only if the device schedules it
-        const int sm = padded_elems<uint64_t>(16384) * 8;
+        const int sm = sort_smem_bytes<uint64_t, 1024, 16, true>();
         int n = 0;
-        cudaError_t q = set_smem_attr(k_seg_sort<uint64_t, 1024, 16, 16, false>, sm, true);
+        cudaError_t q = set_smem_attr(k_seg_sort<uint64_t, 1024, 16, 16, true>, sm, true);
         if (q == cudaSuccess) {
             cudaLaunchConfig_t cfg = {};
             cfg.gridDim = dim3(16, 1, 1);
@@ -463,7 +455,7 @@ bool batch_wide_cluster16()
             attr[0].val.clusterDim.z = 1;
             cfg.attrs = attr;
             cfg.numAttrs = 1;
-            q = cudaOccupancyMaxActiveClusters(&n, k_seg_sort<uint64_t, 1024, 16, 16, false>, &cfg);
+            q = cudaOccupancyMaxActiveClusters(&n, k_seg_sort<uint64_t, 1024, 16, 16, true>, &cfg);
         }
         if (q != cudaSuccess) cudaGetLastError();  // (not an error: the shape is left out)
         g_wide16 = q == cudaSuccess && n >= 1 ? 1 : 0;
@@ -483,13 +475,13 @@ cudaError_t init_batch_kernels()
     if (e == cudaSuccess) e = init_seg_sort_t<uint32_t, 1024, 32, 2, false>();
     if (e == cudaSuccess) e = init_seg_sort_t<uint32_t, 1024, 32, 4, false>();
     if (e == cudaSuccess) e = init_seg_sort_t<uint32_t, 1024, 32, 8, false>();
-    if (e == cudaSuccess) e = init_seg_sort_t<uint64_t, 128, 16, 1, false>();
-    if (e == cudaSuccess) e = init_seg_sort_t<uint64_t, 256, 16, 1, false>();
-    if (e == cudaSuccess) e = init_seg_sort_t<uint64_t, 512, 16, 1, false>();
-    if (e == cudaSuccess) e = init_seg_sort_t<uint64_t, 1024, 16, 1, false>();
-    if (e == cudaSuccess) e = init_seg_sort_t<uint64_t, 1024, 16, 2, false>();
-    if (e == cudaSuccess) e = init_seg_sort_t<uint64_t, 1024, 16, 4, false>();
-    if (e == cudaSuccess) e = init_seg_sort_t<uint64_t, 1024, 16, 8, false>();
+    if (e == cudaSuccess) e = init_seg_sort_t<uint64_t, 128, 16, 1, true>();
+    if (e == cudaSuccess) e = init_seg_sort_t<uint64_t, 256, 16, 1, true>();
+    if (e == cudaSuccess) e = init_seg_sort_t<uint64_t, 512, 16, 1, true>();
+    if (e == cudaSuccess) e = init_seg_sort_t<uint64_t, 1024, 16, 1, true>();
+    if (e == cudaSuccess) e = init_seg_sort_t<uint64_t, 1024, 16, 2, true>();
+    if (e == cudaSuccess) e = init_seg_sort_t<uint64_t, 1024, 16, 4, true>();
+    if (e == cudaSuccess) e = init_seg_sort_t<uint64_t, 1024, 16, 8, true>();
     if (e == cudaSuccess)
         e = set_smem_attr(k_seg_sublist_sort<512, 64>,
                           BinSmem<uint32_t, 512, 64>::kBytes);
@@ -499,13 +491,12 @@ cudaError_t init_batch_kernels()
         e = set_smem_attr(k_seg_bucket_sort<uint32_t, 512, 64, true>,
                           BinSmem<uint32_t, 512, 64>::kBytes);
     if (e == cudaSuccess)
-        e = set_smem_attr(k_seg_sublist_sort_u64<1024, 16>,
-                          padded_elems<uint64_t>(kSegTileU64) * 8);
+        e = set_smem_attr(k_seg_sublist_sort_u64<1024, 16>, BinSmem<uint64_t, 1024, 16>::kBytes);
     if (e == cudaSuccess)
         e = set_smem_attr(k_seg_records_u64<1024>, (int)(kSegRecordsU64 * sizeof(Rec128)));
     if (e == cudaSuccess)
-        e = set_smem_attr(k_seg_bucket_sort<uint64_t, 1024, 16, false>,
-                          padded_elems<uint64_t>(kSegTileU64) * 8);
+        e = set_smem_attr(k_seg_bucket_sort<uint64_t, 1024, 16, true>,
+                          BinSmem<uint64_t, 1024, 16>::kBytes);
     return e;
 }
 
@@ -519,19 +510,19 @@ cudaError_t launch_seg_sort(int chunk, int ctas, bool wide, const void *keys_in,
     if (wide) {
         if (ctas == 1) {
             switch (chunk) {
-            case 2048: L(uint64_t, 128, 16, 1, false);
-            case 4096: L(uint64_t, 256, 16, 1, false);
-            case 8192: L(uint64_t, 512, 16, 1, false);
-            case 16384: L(uint64_t, 1024, 16, 1, false);
+            case 2048: L(uint64_t, 128, 16, 1, true);
+            case 4096: L(uint64_t, 256, 16, 1, true);
+            case 8192: L(uint64_t, 512, 16, 1, true);
+            case 16384: L(uint64_t, 1024, 16, 1, true);
             }
         } else if (chunk == 16384) {
             switch (ctas) {
-            case 2: L(uint64_t, 1024, 16, 2, false);
-            case 4: L(uint64_t, 1024, 16, 4, false);
-            case 8: L(uint64_t, 1024, 16, 8, false);
+            case 2: L(uint64_t, 1024, 16, 2, true);
+            case 4: L(uint64_t, 1024, 16, 4, true);
+            case 8: L(uint64_t, 1024, 16, 8, true);
             case 16:
                 if (!batch_wide_cluster16()) return cudaErrorInvalidValue;
-                L(uint64_t, 1024, 16, 16, false);
+                L(uint64_t, 1024, 16, 16, true);
             }
         }
         return cudaErrorInvalidValue;
@@ -604,7 +595,7 @@ cudaError_t launch_seg_sublist_sort_u64(const uint64_t *keys_in, const uint32_t 
 {
     if (nsub == 0) return cudaSuccess;
     static_assert(kSegTileU64 == 1024 * 16, "a sublist is one CTA's unit");
-    k_seg_sublist_sort_u64<1024, 16><<<nsub, 1024, padded_elems<uint64_t>(kSegTileU64) * 8, st>>>(
+    k_seg_sublist_sort_u64<1024, 16><<<nsub, 1024, BinSmem<uint64_t, 1024, 16>::kBytes, st>>>(
         keys_in, sub_seg, segs, tiles_k, samples);
     return cudaGetLastError();
 }
@@ -635,8 +626,8 @@ cudaError_t launch_seg_bucket_sort_u64(const uint64_t *reloc_k, const uint32_t *
                                        cudaStream_t st)
 {
     if (nunits == 0) return cudaSuccess;
-    k_seg_bucket_sort<uint64_t, 1024, 16, false>
-        <<<nunits, 1024, padded_elems<uint64_t>(kSegTileU64) * 8, st>>>(
+    k_seg_bucket_sort<uint64_t, 1024, 16, true>
+        <<<nunits, 1024, BinSmem<uint64_t, 1024, 16>::kBytes, st>>>(
             reloc_k, units, segs, offsets, (uint32_t)kSegTileU64, 0, keys_out, err);
     return cudaGetLastError();
 }

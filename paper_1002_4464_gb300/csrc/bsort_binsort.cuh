@@ -25,6 +25,9 @@
 // as 16384-key units 203 us (two CTAs of 512 x 32 per SM; comparison sort
 // 588 us), 8192: 189 us (448), 4096: 191 us (369), 2048: 174 us (314).  1024
 // threads x 32 keys for 32768 keys measured 283 us (64 registers spill).
+// 2^25 64-bit keys, pairs in brackets: as 16384-item units 240 us (224;
+// comparison sort 771 and 776), 8192: 201 (190; 707), 4096: 176 (160; 519),
+// 2048: 158 (137; 524).
 // A range below NB gives every value a bin of its own (several, when there
 // are fewer values than lanes, so that a warp's atomics do not meet on one
 // counter) and needs no step 4.
@@ -35,7 +38,8 @@
 // as many bins as they hold keys, and two repeated values that shared a bin
 // part.  (A bin with an eighth of the unit or more takes every 16th of those
 // positions, and its keys are spread over the 16 by lane: a value repeated
-// that often would otherwise meet on one counter.)  What is left unordered
+// that often would otherwise meet on one counter; pairs, whose equal keys must
+// keep their order, are instead cut a third time, by position.)  What is left unordered
 // inside the refined bins is put right by up to kBinPhases phases, by a
 // comparison sort of the warps where that is not enough, and by merging all
 // runs when two warps still overlap.  When a bin holds a quarter of the unit
@@ -43,7 +47,8 @@
 // logarithm), refining would not part them: the unit is sorted by digits
 // or comparisons instead.  (1024 values, Zipf 1.1: 445 us against 515 by
 // digits as 32768-key units, 381 against 584 by comparisons as 16384; 2048:
-// 337 against 314; keys spread over their logarithm: 755 against 512.)
+// 344 against 314; 64-bit keys 327 against 764, pairs 398 against 771 as
+// 16384; 32-bit keys spread over their logarithm: 756 against 512.)
 #pragma once
 
 #include <cstdint>
@@ -160,6 +165,14 @@ template <int NB> struct BinMapF32 {
     static constexpr int kShift = 23 - __builtin_ctz(NB);
     __device__ uint32_t bin(uint32_t key) const { return (place(key) >> kShift) & (uint32_t)(NB - 1); }
     __device__ uint32_t fine(uint32_t key) const { return place(key) << (32 - kShift); }
+};
+
+// Pairs (key << 32 | position) by key.
+template <int NB> struct BinMapPairs {
+    BinMap<uint32_t, NB> m;
+    __device__ BinMapPairs(uint32_t lo, uint32_t hi) : m(lo, hi) {}
+    __device__ uint32_t bin(uint64_t x) const { return m.bin((uint32_t)(x >> 32)); }
+    __device__ uint32_t fine(uint64_t x) const { return m.fine((uint32_t)(x >> 32)); }
 };
 
 // Ranges below NB: value x of the range has the rep bins [x*rep, (x+1)*rep),
@@ -299,6 +312,25 @@ struct BinSort {
                 if (FULL || real(k0 + j)) sm[pidx<K>((int)r[j])] = v[k0 + j];
         }
     }
+    // Bins that straddle this warp's first key: merge the last 32 keys before
+    // it and the first 32 from it, each ascending.
+    __device__ __forceinline__ void merge_edge() const
+    {
+        if (warp == 0 || !act) return;
+        const int b = warp * W;
+        const K x = sm[pidx<K>(b - 32 + lane)], y = sm[pidx<K>(b + 31 - lane)];
+        K l = kmin<K>(x, y), h = kmax<K>(x, y);
+#pragma unroll
+        for (int d = 16; d >= 1; d >>= 1) {
+            const K xl = __shfl_xor_sync(0xFFFFFFFFu, l, d);
+            const K xh = __shfl_xor_sync(0xFFFFFFFFu, h, d);
+            const bool low = (lane & d) == 0;
+            l = low ? kmin<K>(l, xl) : kmax<K>(l, xl);
+            h = low ? kmin<K>(h, xh) : kmax<K>(h, xh);
+        }
+        sm[pidx<K>(b - 32 + lane)] = l;
+        sm[pidx<K>(b + lane)] = h;
+    }
     __device__ __forceinline__ void pad() const  // the positions behind the real keys
     {
         for (int x = len + tid; x < CAP; x += T) sm[pidx<K>(x)] = KeyMax<K>::v;
@@ -309,7 +341,7 @@ struct BinSort {
 // of line: its comparison sorts must not take registers from the usual
 // path).  The keys are in sm at their warp-blocked positions, the first bins'
 // exclusive prefix P in the counters.
-template <typename K, int T, int E, typename F>
+template <typename K, int T, int E, bool PAIRS, typename F>
 __device__ __noinline__ void bin_skewed(K *sm, int len, const F map, uint32_t G)
 {
     using B = BinSort<K, T, E>;
@@ -319,6 +351,11 @@ __device__ __noinline__ void bin_skewed(K *sm, int len, const F map, uint32_t G)
     __shared__ uint32_t s_a[NWARP], s_b[NWARP];
     const B s(sm, len);
     const int tid = s.tid, lane = s.lane, warp = s.warp;
+    // the sort key of an item (of a pair, without its position)
+    auto value = [](K x) {
+        if constexpr (PAIRS) return (uint32_t)(x >> 32);
+        else return x;
+    };
     K v[E];
 #pragma unroll
     for (int k = 0; k < E; ++k) v[k] = sm[pidx<K>(wb_pos<E>(warp, lane, k))];
@@ -335,7 +372,7 @@ __device__ __noinline__ void bin_skewed(K *sm, int len, const F map, uint32_t G)
         for (int k = 0; k < B::SK; ++k) {
             if (s.real(k)) {
                 ++cnt;
-                mixed += sm[map.bin(v[k]) & (uint32_t)(CAP - 1)] != v[k];
+                mixed += value(sm[map.bin(v[k]) & (uint32_t)(CAP - 1)]) != value(v[k]);
             }
         }
         mixed = __reduce_add_sync(0xFFFFFFFFu, mixed);
@@ -355,20 +392,23 @@ __device__ __noinline__ void bin_skewed(K *sm, int len, const F map, uint32_t G)
         }
     }
     uint32_t *fine = reinterpret_cast<uint32_t *>(sm);  // the refined bins' counters
-    for (int i = tid; i < CAP / 8; i += T)
-        reinterpret_cast<uint4 *>(fine)[i] = make_uint4(0u, 0u, 0u, 0u);
-    __syncthreads();
     const uint32_t *P = reinterpret_cast<const uint32_t *>(s.counters());
     const uint32_t fbase = smem_u32addr(fine);
-    uint32_t bins[E / 2];  // the keys' refined bins, two to a word
-    auto recount = [&](auto full) {
+    uint32_t bins[E / 2];  // the keys' bins so far, two to a word
+    // Cut every bin by the keys' places in it (BY_POS: by their positions in
+    // the unit, for pairs, whose equal keys keep their order).
+    auto recount = [&](auto full, auto by_pos) {
+        constexpr bool FULL = decltype(full)::value, BY_POS = decltype(by_pos)::value;
         constexpr int GB = 8;
 #pragma unroll
         for (int k0 = 0; k0 < E; k0 += GB) {
             uint32_t p0[GB], p1[GB];
 #pragma unroll
             for (int j = 0; j < GB; ++j) {
-                const uint32_t b = map.bin(v[k0 + j]) & (uint32_t)(B::NB - 1), e = b + 1;
+                const int k = k0 + j;
+                const uint32_t b = BY_POS ? (bins[k / 2] >> (16 * (k & 1))) & 0xFFFFu
+                                          : map.bin(v[k]) & (uint32_t)(B::NB - 1);
+                const uint32_t e = b + 1;
                 p0[j] = (P[b & (uint32_t)(NW - 1)] >> B::half(b)) & 0xFFFFu;
                 p1[j] = e < (uint32_t)B::NB ? (P[e & (uint32_t)(NW - 1)] >> B::half(e)) & 0xFFFFu
                                             : (uint32_t)len;
@@ -377,21 +417,37 @@ __device__ __noinline__ void bin_skewed(K *sm, int len, const F map, uint32_t G)
             for (int j = 0; j < GB; ++j) {
                 const int k = k0 + j;
                 const uint32_t w = p1[j] - p0[j];
-                const int sh = w >= (uint32_t)(CAP / 8) ? 4 : 0;
-                const uint32_t b2 = (p0[j] + (__umulhi(map.fine(v[k]), w >> sh) << sh) +
-                                     ((uint32_t)lane & ((1u << sh) - 1u))) & (uint32_t)(CAP - 1);
-                if (k & 1) bins[k / 2] |= b2 << 16;
+                uint32_t at;
+                if constexpr (BY_POS) {
+                    at = w * (uint32_t)wb_pos<E>(warp, lane, k) / (uint32_t)CAP;
+                } else {
+                    const int sh = !PAIRS && w >= (uint32_t)(CAP / 8) ? 4 : 0;
+                    at = (__umulhi(map.fine(v[k]), w >> sh) << sh) +
+                         ((uint32_t)lane & ((1u << sh) - 1u));
+                }
+                const uint32_t b2 = (p0[j] + at) & (uint32_t)(CAP - 1);
+                if constexpr (BY_POS)
+                    bins[k / 2] = (bins[k / 2] & (0xFFFFu << (16 * (1 - (k & 1))))) |
+                                  (b2 << (16 * (k & 1)));
+                else if (k & 1) bins[k / 2] |= b2 << 16;
                 else bins[k / 2] = b2;
-                red_add_shared(decltype(full)::value || s.real(k)
-                                   ? fbase + ((b2 & (uint32_t)(NW - 1)) << 2) : s.spare(),
+                red_add_shared(FULL || s.real(k) ? fbase + ((b2 & (uint32_t)(NW - 1)) << 2)
+                                                 : s.spare(),
                                1u << B::half(b2));
             }
         }
     };
-    if (s.full) recount(std::true_type{});
-    else if (s.act) recount(std::false_type{});
-    __syncthreads();
-    s.scan(reinterpret_cast<const uint4 *>(fine), s.counters(), s_a, s_b);
+    auto refine = [&](auto by_pos) {
+        for (int i = tid; i < CAP / 8; i += T)
+            reinterpret_cast<uint4 *>(fine)[i] = make_uint4(0u, 0u, 0u, 0u);
+        __syncthreads();
+        if (s.full) recount(std::true_type{}, by_pos);
+        else if (s.act) recount(std::false_type{}, by_pos);
+        __syncthreads();
+        s.scan(reinterpret_cast<const uint4 *>(fine), s.counters(), s_a, s_b);
+    };
+    refine(std::false_type{});
+    if constexpr (PAIRS) refine(std::true_type{});
     auto place = [&](auto full) {
         constexpr int GB = 8;
 #pragma unroll
@@ -431,12 +487,18 @@ __device__ __noinline__ void bin_skewed(K *sm, int len, const F map, uint32_t G)
         for (int k = 0; k < E; ++k) sm[pidx<K>(tid * E + k)] = v[k];
     }
     __syncthreads();
+    s.merge_edge();
+    __syncthreads();
     const int b = warp * W;
-    if (__syncthreads_or(warp > 0 && s.act && sm[pidx<K>(b - 1)] > sm[pidx<K>(b)])) {
-        // (runs of odd warps are stored descending for the merge levels)
-        store_run<K, E>(sm, b, W, lane * E, (warp & 1) != 0, v);
+    if (__syncthreads_or(warp > 0 && s.act &&
+                         (sm[pidx<K>(b - 33)] > sm[pidx<K>(b - 32)] ||
+                          sm[pidx<K>(b + 31)] > sm[pidx<K>(b + 32)]))) {
+        // two warps overlap by more: merge all the runs (a warp's is sorted
+        // again, and stored descending by odd warps for the merge levels)
+#pragma unroll
+        for (int k = 0; k < E; ++k) v[k] = sm[pidx<K>(tid * E + k)];
         __syncthreads();
-        cta_merge_runs<K, T, E>(sm, W);
+        cta_sort<K, T, E>(v, sm, len);
     }
 }
 
@@ -445,47 +507,53 @@ __device__ __noinline__ void bin_skewed(K *sm, int len, const F map, uint32_t G)
 // the warp-blocked layout; positions >= len are padding holding the maximal
 // key.  On return sm[pidx(x)] is the x-th smallest key, padding after the
 // len real ones, as cta_sort leaves it.  is_f32: 32-bit keys are codes of
-// floats.  Ends with __syncthreads().
-template <typename K, int T, int E>
+// floats.  PAIRS: v holds key << 32 | a position that grows with the item's
+// place in the unit.  Ends with __syncthreads().
+template <typename K, int T, int E, bool PAIRS = false>
 __device__ __forceinline__ void cta_bin_sort(K (&v)[E], K *sm, int len, bool is_f32)
 {
     using B = BinSort<K, T, E>;
-    constexpr int W = B::W, NWARP = B::NWARP, NB = B::NB;
-    __shared__ K s_lo[NWARP], s_hi[NWARP];
+    constexpr int NWARP = B::NWARP, NB = B::NB;
+    __shared__ typename std::conditional<PAIRS, uint32_t, K>::type s_lo[NWARP], s_hi[NWARP];
     __shared__ uint32_t s_a[NWARP], s_b[NWARP];
     const B s(sm, len);
     const int lane = s.lane, warp = s.warp;
     // smallest and largest real key; counters to zero
-    K lo = KeyMax<K>::v, hi = 0;
+    using V = typename std::conditional<PAIRS, uint32_t, K>::type;
+    auto value = [](K x) {
+        if constexpr (PAIRS) return (uint32_t)(x >> 32);
+        else return x;
+    };
+    V lo = KeyMax<V>::v, hi = 0;
     if (s.full) {
 #pragma unroll
         for (int k = 0; k < E; ++k) {
-            lo = kmin<K>(lo, v[k]);
-            hi = kmax<K>(hi, v[k]);
+            lo = kmin<V>(lo, value(v[k]));
+            hi = kmax<V>(hi, value(v[k]));
         }
     } else if (s.act) {
 #pragma unroll
         for (int k = 0; k < E; ++k)
             if (s.real(k)) {
-                lo = kmin<K>(lo, v[k]);
-                hi = kmax<K>(hi, v[k]);
+                lo = kmin<V>(lo, value(v[k]));
+                hi = kmax<V>(hi, value(v[k]));
             }
     }
-    auto warp_lo = [&](K x) {
-        if constexpr (sizeof(K) == 4) {
+    auto warp_lo = [&](V x) {
+        if constexpr (sizeof(V) == 4) {
             return __reduce_min_sync(0xFFFFFFFFu, x);
         } else {
 #pragma unroll
-            for (int d = 16; d >= 1; d >>= 1) x = kmin<K>(x, __shfl_xor_sync(0xFFFFFFFFu, x, d));
+            for (int d = 16; d >= 1; d >>= 1) x = kmin<V>(x, __shfl_xor_sync(0xFFFFFFFFu, x, d));
             return x;
         }
     };
-    auto warp_hi = [&](K x) {
-        if constexpr (sizeof(K) == 4) {
+    auto warp_hi = [&](V x) {
+        if constexpr (sizeof(V) == 4) {
             return __reduce_max_sync(0xFFFFFFFFu, x);
         } else {
 #pragma unroll
-            for (int d = 16; d >= 1; d >>= 1) x = kmax<K>(x, __shfl_xor_sync(0xFFFFFFFFu, x, d));
+            for (int d = 16; d >= 1; d >>= 1) x = kmax<V>(x, __shfl_xor_sync(0xFFFFFFFFu, x, d));
             return x;
         }
     };
@@ -500,12 +568,10 @@ __device__ __forceinline__ void cta_bin_sort(K (&v)[E], K *sm, int len, bool is_
     __syncthreads();
     lo = warp_lo(s_lo[lane % NWARP]);
     hi = warp_hi(s_hi[lane % NWARP]);
-    if (hi <= lo) {  // no real key, or all of them equal
-#pragma unroll 4
-        for (int k = 0; k < E; ++k) {
-            const int x = k * T + s.tid;
-            sm[pidx<K>(x)] = x < len ? lo : KeyMax<K>::v;
-        }
+    if (hi <= lo) {  // no real key, or all of them equal (pairs: in order)
+#pragma unroll
+        for (int k = 0; k < E; ++k)
+            sm[pidx<K>(wb_pos<E>(warp, lane, k))] = s.real(k) ? v[k] : KeyMax<K>::v;
         __syncthreads();
         return;
     }
@@ -521,7 +587,7 @@ __device__ __forceinline__ void cta_bin_sort(K (&v)[E], K *sm, int len, bool is_
 #pragma unroll
                 for (int k = 0; k < E; ++k) sm[pidx<K>(wb_pos<E>(warp, lane, k))] = v[k];
                 __syncthreads();
-                bin_skewed<K, T, E>(sm, len, map, G);
+                bin_skewed<K, T, E, PAIRS>(sm, len, map, G);
                 return false;
             }
         }
@@ -531,17 +597,21 @@ __device__ __forceinline__ void cta_bin_sort(K (&v)[E], K *sm, int len, bool is_
         __syncthreads();
         return decltype(fill)::value;
     };
-    if (hi - lo < (K)NB) {
-        distribute(BinMapExact<K, NB>(lo, hi, lane), std::false_type{});
-        return;
-    }
     bool more;
-    if constexpr (sizeof(K) == 4) {
-        const BinMapF32<NB> fmap(lo, hi);
-        if (is_f32 && fmap.ok) more = distribute(fmap, std::true_type{});
-        else more = distribute(BinMap<K, NB>(lo, hi), std::true_type{});
+    if constexpr (PAIRS) {
+        more = distribute(BinMapPairs<NB>(lo, hi), std::true_type{});
     } else {
-        more = distribute(BinMap<K, NB>(lo, hi), std::true_type{});
+        if (hi - lo < (K)NB) {
+            distribute(BinMapExact<K, NB>(lo, hi, lane), std::false_type{});
+            return;
+        }
+        if constexpr (sizeof(K) == 4) {
+            const BinMapF32<NB> fmap(lo, hi);
+            if (is_f32 && fmap.ok) more = distribute(fmap, std::true_type{});
+            else more = distribute(BinMap<K, NB>(lo, hi), std::true_type{});
+        } else {
+            more = distribute(BinMap<K, NB>(lo, hi), std::true_type{});
+        }
     }
     if (!more) return;
     // 4. order the keys inside the bins
@@ -554,23 +624,7 @@ __device__ __forceinline__ void cta_bin_sort(K (&v)[E], K *sm, int len, bool is_
         for (int k = 0; k < E; ++k) sm[pidx<K>(s.tid * E + k)] = v[k];
     }
     __syncthreads();
-    if (warp > 0 && s.act) {
-        // bins that straddle this warp's first key: the last 32 keys before
-        // it and the first 32 from it, each ascending
-        const int b = warp * W;
-        const K x = sm[pidx<K>(b - 32 + lane)], y = sm[pidx<K>(b + 31 - lane)];
-        K l = kmin<K>(x, y), h = kmax<K>(x, y);
-#pragma unroll
-        for (int d = 16; d >= 1; d >>= 1) {
-            const K xl = __shfl_xor_sync(0xFFFFFFFFu, l, d);
-            const K xh = __shfl_xor_sync(0xFFFFFFFFu, h, d);
-            const bool low = (lane & d) == 0;
-            l = low ? kmin<K>(l, xl) : kmax<K>(l, xl);
-            h = low ? kmin<K>(h, xh) : kmax<K>(h, xh);
-        }
-        sm[pidx<K>(b - 32 + lane)] = l;
-        sm[pidx<K>(b + lane)] = h;
-    }
+    s.merge_edge();
     __syncthreads();
 }
 

@@ -25,21 +25,24 @@ constexpr int sort_smem_bytes()
 }
 
 // CTAs per SM that the registers leave room for: the distribution sort of
-// up to 16384 keys takes 64 registers a thread, so that the CTAs of an SM
-// overlap one's memory phases with another's arithmetic (16384-key units on
-// 2^26 keys: 205 us with two 512-thread CTAs per SM, 263 us with one of 1024).
-template <int T, int E, int C, bool BINS>
+// up to 16384 32-bit keys takes 64 registers a thread, so that the CTAs of an
+// SM overlap one's memory phases with another's arithmetic (16384-key units
+// on 2^26 keys: 203 us with two 512-thread CTAs per SM, 263 us with one of
+// 1024); 64-bit words take 80 in the small units.
+template <typename K, int T, int E, int C, bool BINS>
 constexpr int min_ctas()
 {
-    return BINS && C == 1 && T * E <= 16384 ? 1024 / T : 1;
+    if (!BINS || C > 1) return 1;
+    if (sizeof(K) == 8) return T >= 1024 ? 1 : T == 512 ? 2 : 768 / T;
+    return T * E <= 16384 ? 1024 / T : 1;
 }
 
 // The in-CTA sort of one chunk: the comparison sort (cta_sort) or the
 // distribution sort (cta_bin_sort); both leave the same result.
-template <typename K, int T, int E, bool BINS>
+template <typename K, int T, int E, bool BINS, bool PAIRS = false>
 __device__ __forceinline__ void chunk_sort(K (&v)[E], K *sm, int len, bool is_f32)
 {
-    if constexpr (BINS) cta_bin_sort<K, T, E>(v, sm, len, is_f32);
+    if constexpr (BINS) cta_bin_sort<K, T, E, PAIRS>(v, sm, len, is_f32);
     else cta_sort<K, T, E>(v, sm, len);
 }
 
@@ -77,7 +80,7 @@ __device__ __forceinline__ void load_keys(K (&v)[E], const K *__restrict__ src, 
 // the samples (ranks (k+1)w - 1) that fall in that range as key << 32 | p,
 // p = i*t + r.
 template <int T, int E, bool PAIRS, int C, bool BINS = false>
-__global__ void __launch_bounds__(T, (min_ctas<T, E, C, BINS>()))
+__global__ void __launch_bounds__(T, (min_ctas<typename std::conditional<PAIRS, uint64_t, uint32_t>::type, T, E, C, BINS>()))
 k_sublist_sort(const uint32_t *__restrict__ keys_in, const void *__restrict__ vals_in,
                uint64_t n, int is_f32, int val_bytes, uint32_t s,
                uint32_t *__restrict__ tiles_k, void *__restrict__ tiles_v,
@@ -103,21 +106,16 @@ k_sublist_sort(const uint32_t *__restrict__ keys_in, const void *__restrict__ va
 
     K v[E];
     if constexpr (PAIRS) {
+        uint32_t key[E];  // (pad sentinel: the maximal key, position >= n)
+        load_keys<uint32_t, T, E>(key, keys_in + base + off, len - off, is_f32 != 0);
 #pragma unroll
-        for (int k = 0; k < E; ++k) {
-            const int x = off + wb_pos<E>(warp, lane, k);
-            uint32_t key = 0xFFFFFFFFu;  // pad sentinel (position >= n)
-            if (x < len) {
-                key = keys_in[base + x];
-                if (is_f32) key = f32_encode(key);
-            }
-            v[k] = ((uint64_t)key << 32) | (uint32_t)x;
-        }
+        for (int k = 0; k < E; ++k)
+            v[k] = ((uint64_t)key[k] << 32) | (uint32_t)(off + wb_pos<E>(warp, lane, k));
     } else {
         load_keys<uint32_t, T, E>(v, keys_in + base + off, len - off, is_f32 != 0);
     }
     const int clen = len - off;
-    chunk_sort<K, T, E, BINS>(v, sm, clen < 0 ? 0 : (clen > CH ? CH : clen), is_f32 != 0);
+    chunk_sort<K, T, E, BINS, PAIRS>(v, sm, clen < 0 ? 0 : (clen > CH ? CH : clen), is_f32 != 0);
     cluster_merge<K, T, E, C>(sm, len);
 
 #pragma unroll 4
@@ -215,22 +213,18 @@ bucket_sort_unit(uint32_t u, const uint32_t *__restrict__ src_k, const void *__r
     const int ustart = r * per;
     const int uend = min(ustart + per, len);
     K v[E];
-    if (!PAIRS && !gather) {
-        if constexpr (!PAIRS)
-            load_keys<uint32_t, T, E>(v, src_k + L + ustart, uend - ustart, direct && is_f32);
-    } else if (!gather) {
+    if (!gather) {
+        if constexpr (PAIRS) {
+            uint32_t key[E];
+            load_keys<uint32_t, T, E>(key, src_k + L + ustart, uend - ustart, direct && is_f32);
 #pragma unroll
-        for (int k = 0; k < E; ++k) {
-            const int x = ustart + wb_pos<E>(warp, lane, k);
-            uint32_t key = 0xFFFFFFFFu;
-            uint32_t idx = 0xFFFFFFFFu;  // pads sort after every real item
-            if (x < uend) {
-                key = src_k[L + x];
-                if (direct && is_f32) key = f32_encode(key);
-                idx = (uint32_t)x;
+            for (int k = 0; k < E; ++k) {
+                const int x = ustart + wb_pos<E>(warp, lane, k);
+                // (pads sort after every real item)
+                v[k] = ((uint64_t)key[k] << 32) | (x < uend ? (uint32_t)x : 0xFFFFFFFFu);
             }
-            if constexpr (PAIRS) v[k] = ((uint64_t)key << 32) | idx;
-            else v[k] = (K)key;
+        } else {
+            load_keys<uint32_t, T, E>(v, src_k + L + ustart, uend - ustart, direct && is_f32);
         }
     } else {
         // lane's first position, and the run containing it: search the runs
@@ -270,7 +264,7 @@ bucket_sort_unit(uint32_t u, const uint32_t *__restrict__ src_k, const void *__r
             else v[k] = (K)key;
         }
     }
-    chunk_sort<K, T, E, BINS>(v, sm, uend > ustart ? uend - ustart : 0, is_f32 != 0);
+    chunk_sort<K, T, E, BINS, PAIRS>(v, sm, uend > ustart ? uend - ustart : 0, is_f32 != 0);
     cluster_merge<K, T, E, C>(sm, len, per);
     const uint64_t lim64 = min((unsigned long long)len, (unsigned long long)(n > L ? n - L : 0));
     const int lim = (int)lim64;
@@ -298,7 +292,7 @@ bucket_sort_unit(uint32_t u, const uint32_t *__restrict__ src_k, const void *__r
 
 // Cluster u of the grid sorts unit u (clusters beyond the unit count exit).
 template <int T, int E, bool PAIRS, int C, bool BINS = false>
-__global__ void __launch_bounds__(T, (min_ctas<T, E, C, BINS>()))
+__global__ void __launch_bounds__(T, (min_ctas<typename std::conditional<PAIRS, uint64_t, uint32_t>::type, T, E, C, BINS>()))
 k_bucket_sort(const uint32_t *__restrict__ src_k, const void *__restrict__ src_v,
               const uint32_t *__restrict__ units, uint64_t n, uint64_t n_pad, int is_f32,
               int val_bytes, uint32_t *__restrict__ out_k, void *__restrict__ out_v, int *err,
@@ -314,7 +308,7 @@ k_bucket_sort(const uint32_t *__restrict__ src_k, const void *__restrict__ src_v
 // sorts units lo + c, lo + c + G, ... (G clusters; every CTA of a cluster
 // takes the same units).
 template <int T, int E, bool PAIRS, int C, bool BINS = false>
-__global__ void __launch_bounds__(T, (min_ctas<T, E, C, BINS>()))
+__global__ void __launch_bounds__(T, (min_ctas<typename std::conditional<PAIRS, uint64_t, uint32_t>::type, T, E, C, BINS>()))
 k_bucket_sort_loop(const uint32_t *__restrict__ src_k, const void *__restrict__ src_v,
                    const uint32_t *__restrict__ units, uint64_t n, uint64_t n_pad, int is_f32,
                    int val_bytes, uint32_t *__restrict__ out_k, void *__restrict__ out_v,

@@ -5,13 +5,14 @@
 
 namespace bsort {
 
-// chunk shapes: 2048 = 128x16, 4096 = 256x16, 8192 = 512x16, 16384 = 1024x16;
+// Sorted by bins of the key (cta_bin_sort), then by position among equal
+// keys.  chunk shapes: 2048 = 128x16, 4096 = 256x16, 8192 = 512x16, 16384 = 1024x16;
 // clusters of 2, 4, 8 CTAs on the 16384-item chunk.
 cudaError_t init_sort_pairs_kernels()
 {
     cudaError_t e;
 #define I(T_, E_, C_)                                           \
-    e = init_sort_pair_of_kernels<T_, E_, true, C_>();          \
+    e = init_sort_pair_of_kernels<T_, E_, true, C_, true>();          \
     if (e != cudaSuccess) return e
     I(128, 16, 1); I(256, 16, 1); I(512, 16, 1); I(1024, 16, 1);
     I(1024, 16, 2); I(1024, 16, 4); I(1024, 16, 8);
@@ -25,7 +26,7 @@ cudaError_t launch_sublist_sort_pairs(int chunk, int ctas, const void *keys_in,
                                       void *tiles_v, uint64_t *samples, cudaStream_t st)
 {
 #define L(T_, E_, C_)                                                                      \
-    return launch_sublist_sort_t<T_, E_, true, C_>(keys_in, vals_in, n, m, is_f32,          \
+    return launch_sublist_sort_t<T_, E_, true, C_, true>(keys_in, vals_in, n, m, is_f32,          \
                                                    val_bytes, s, tiles_k, tiles_v, samples, \
                                                    0u, st)
     if (ctas == 1) {
@@ -52,7 +53,7 @@ cudaError_t launch_bucket_sort_pairs(int chunk, int ctas, const void *src_k, con
                                      void *out_v, int *err, const GatherSrc &g, cudaStream_t st)
 {
 #define L(T_, E_, C_)                                                                          \
-    return launch_bucket_sort_t<T_, E_, true, C_>(src_k, src_v, units, max_units, n, n_pad,    \
+    return launch_bucket_sort_t<T_, E_, true, C_, true>(src_k, src_v, units, max_units, n, n_pad,    \
                                                   is_f32, val_bytes, out_k, out_v, err, g, st)
     if (ctas == 1) {
         switch (chunk) {

@@ -3,7 +3,7 @@
 // changes is the width of what they move:
 //
 //   sorted sublists and buckets hold 64-bit keys (a CTA sorts 16,384 of
-//     them; clusters of 2, 4, 8 CTAs for larger units);
+//     them by bins, cta_bin_sort; clusters of 2, 4, 8 CTAs for larger units);
 //   a sample record is the pair (key, p), p = i*t + r, stored as two 64-bit
 //     words (16 bytes), compared key first, then p (the composite order);
 //   Step 4 merges the m sorted runs of s records (one per sublist) in
@@ -23,7 +23,7 @@ __device__ __forceinline__ bool rec_lt(const Rec128 &a, const Rec128 &b)
 // Cluster i sorts sublist i (t = C*T*E keys) and emits the samples of its
 // ranks, as k_sublist_sort does for 32-bit keys.
 template <int T, int E, int C>
-__global__ void __launch_bounds__(T, 1)
+__global__ void __launch_bounds__(T, (min_ctas<uint64_t, T, E, C, true>()))
 k_sublist_sort_u64(const uint64_t *__restrict__ keys_in, uint64_t n, uint32_t s,
                    uint64_t *__restrict__ tiles_k, Rec128 *__restrict__ samples)
 {
@@ -32,21 +32,20 @@ k_sublist_sort_u64(const uint64_t *__restrict__ keys_in, uint64_t n, uint32_t s,
     extern __shared__ __align__(16) unsigned char smem_raw[];
     uint64_t *sm = reinterpret_cast<uint64_t *>(smem_raw);
     const int tid = threadIdx.x;
-    const int lane = tid & 31, warp = tid >> 5;
     const uint32_t tile = blockIdx.x / C;
     const int r = (int)(blockIdx.x % C);
     const uint64_t base = (uint64_t)tile * TT;
     const uint64_t avail = n > base ? n - base : 0;
     const int len = avail < (uint64_t)TT ? (int)avail : (int)TT;
     const int off = r * CH;
-    uint64_t v[E];
-#pragma unroll
-    for (int k = 0; k < E; ++k) {
-        const int x = off + wb_pos<E>(warp, lane, k);
-        v[k] = x < len ? keys_in[base + x] : 0xFFFFFFFFFFFFFFFFull;
+    if (tid == 0) {  // the same chunk of the sublist this SM will most likely sort next
+        const uint64_t nb = base + (uint64_t)(num_sms() / C) * TT + off;
+        if (nb < n) prefetch_l2(keys_in + nb, 8 * min((uint64_t)CH, n - nb));
     }
     const int clen = len - off;
-    cta_sort<uint64_t, T, E>(v, sm, clen < 0 ? 0 : (clen > CH ? CH : clen));
+    uint64_t v[E];
+    load_keys<uint64_t, T, E>(v, keys_in + base + off, clen, false);
+    chunk_sort<uint64_t, T, E, true>(v, sm, clen < 0 ? 0 : (clen > CH ? CH : clen), false);
     cluster_merge<uint64_t, T, E, C>(sm, len);
 #pragma unroll 4
     for (int k = 0; k < E; ++k) {
@@ -290,14 +289,13 @@ template <int T, int E, int C>
 __device__ __forceinline__ void
 bucket_sort_unit_u64(uint32_t u, const uint64_t *__restrict__ src,
                      const uint32_t *__restrict__ units, uint64_t n, uint64_t n_pad,
-                     uint64_t *__restrict__ out, int *err)
+                     uint64_t *__restrict__ out, int *err, uint32_t prefetch_stride)
 {
     constexpr int CH = T * E;
     constexpr uint64_t CAP = (uint64_t)C * CH;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     uint64_t *sm = reinterpret_cast<uint64_t *>(smem_raw);
     const int tid = threadIdx.x;
-    const int lane = tid & 31, warp = tid >> 5;
     const int r = (int)(blockIdx.x % C);
     uint64_t L = 0, R = n;
     if (units != nullptr) {
@@ -314,13 +312,17 @@ bucket_sort_unit_u64(uint32_t u, const uint64_t *__restrict__ src,
     const int per = C == 1 ? CH : (len + C - 1) / C;
     const int ustart = r * per;
     const int uend = min(ustart + per, len);
-    uint64_t v[E];
-#pragma unroll
-    for (int k = 0; k < E; ++k) {
-        const int x = ustart + wb_pos<E>(warp, lane, k);
-        v[k] = x < uend ? src[L + x] : 0xFFFFFFFFFFFFFFFFull;
+    if (units != nullptr && threadIdx.x == 0 && r == 0 && prefetch_stride) {
+        // the unit this SM will most likely sort next
+        const uint32_t un = u + prefetch_stride;
+        if (un < units[0]) {
+            const uint32_t pl = units[1 + 2 * un], pr = units[2 + 2 * un];
+            if (pl < pr && pr <= n_pad) prefetch_l2(src + pl, 8ull * (pr - pl));
+        }
     }
-    cta_sort<uint64_t, T, E>(v, sm, uend > ustart ? uend - ustart : 0);
+    uint64_t v[E];
+    load_keys<uint64_t, T, E>(v, src + L + ustart, uend - ustart, false);
+    chunk_sort<uint64_t, T, E, true>(v, sm, uend > ustart ? uend - ustart : 0, false);
     cluster_merge<uint64_t, T, E, C>(sm, len, per);
     const int off = r * CH;
     const uint64_t lim64 = min((unsigned long long)len, (unsigned long long)(n > L ? n - L : 0));
@@ -333,11 +335,11 @@ bucket_sort_unit_u64(uint32_t u, const uint64_t *__restrict__ src,
 }
 
 template <int T, int E, int C>
-__global__ void __launch_bounds__(T, 1)
+__global__ void __launch_bounds__(T, (min_ctas<uint64_t, T, E, C, true>()))
 k_bucket_sort_u64(const uint64_t *__restrict__ src, const uint32_t *__restrict__ units,
                   uint64_t n, uint64_t n_pad, uint64_t *__restrict__ out, int *err)
 {
-    bucket_sort_unit_u64<T, E, C>(blockIdx.x / C, src, units, n, n_pad, out, err);
+    bucket_sort_unit_u64<T, E, C>(blockIdx.x / C, src, units, n, n_pad, out, err, num_sms() / C);
 }
 
 // Cluster c of a small grid sorts units c, c + G, ... of a device-sized list.
@@ -349,7 +351,7 @@ k_bucket_sort_u64_loop(const uint64_t *__restrict__ src, const uint32_t *__restr
     const uint32_t count = units[0];
 #pragma unroll 1
     for (uint32_t u = blockIdx.x / C; u < count; u += gridDim.x / C) {
-        bucket_sort_unit_u64<T, E, C>(u, src, units, n, n_pad, out, err);
+        bucket_sort_unit_u64<T, E, C>(u, src, units, n, n_pad, out, err, gridDim.x / C);
         __syncthreads();  // shared memory is reused by the next unit
     }
 }
@@ -360,7 +362,7 @@ namespace {
 template <int T, int E, int C>
 cudaError_t init_u64_t()
 {
-    const int sm = padded_elems<uint64_t>(T * E) * 8;
+    const int sm = sort_smem_bytes<uint64_t, T, E, true>();
     cudaError_t e = cudaFuncSetAttribute(k_sublist_sort_u64<T, E, C>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
     if (e == cudaSuccess)
@@ -376,7 +378,7 @@ template <int T, int E, int C>
 cudaError_t launch_sublist_u64_t(const void *keys_in, uint64_t n, uint32_t m, uint32_t s,
                                  uint64_t *tiles, Rec128 *samples, cudaStream_t st)
 {
-    const int sm = padded_elems<uint64_t>(T * E) * 8;
+    const int sm = sort_smem_bytes<uint64_t, T, E, true>();
     return launch_maybe_cluster(k_sublist_sort_u64<T, E, C>, m * C, T, sm, C, st,
                                 static_cast<const uint64_t *>(keys_in), n, s, tiles, samples);
 }
@@ -385,7 +387,7 @@ template <int T, int E, int C>
 cudaError_t launch_bucket_u64_t(const void *src, const uint32_t *units, uint32_t max_units,
                                 uint64_t n, uint64_t n_pad, void *out, int *err, cudaStream_t st)
 {
-    const int sm = padded_elems<uint64_t>(T * E) * 8;
+    const int sm = sort_smem_bytes<uint64_t, T, E, true>();
     const unsigned grid = (units ? max_units : 1u) * C;
     if (C > 1 && units != nullptr && max_units <= kLoopUnits)
         return launch_maybe_cluster(k_bucket_sort_u64_loop<T, E, C>, grid, T, sm, C, st,

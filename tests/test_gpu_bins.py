@@ -105,3 +105,44 @@ def test_units_f32(kind, n):
         f[3::79] = np.float32(-0.0)
         f[4::73] = np.float32(1e-45)
     _check(f.view(np.uint32), "f32")
+
+
+@pytest.mark.parametrize("n", [33, 2048, 2049, 8191, 8192, 16383, 16384, 16385, 40001, 300007])
+@pytest.mark.parametrize("kind", KINDS)
+def test_units_u64(kind, n):
+    _check(_keys(kind, n, 64, synth.seed_for(7, 5, n)), "u64")
+
+
+@pytest.mark.parametrize("n", [33, 2047, 2048, 4097, 8192, 16383, 16384, 40001, 300007])
+@pytest.mark.parametrize("kind", KINDS + ["equal"])
+def test_units_pairs(kind, n):
+    """Key-value pairs, value = input index: equal keys keep their order."""
+    keys = (np.full(n, 0xFFFFFFFF, np.uint32) if kind == "equal"
+            else _keys(kind, n, 32, synth.seed_for(7, 6, n)))
+    sorter = pkg.BucketSorter()
+    d_k = torch.from_numpy(keys.view(np.int32)).cuda()
+    d_v = torch.arange(n, dtype=torch.int32, device="cuda")
+    ok, ov = sorter.sort_pairs(d_k, d_v)
+    sorter.sync()
+    order = np.argsort(keys, kind="stable")
+    assert np.array_equal(ok.cpu().numpy().view(np.uint32), keys[order])
+    assert np.array_equal(ov.cpu().numpy(), order.astype(np.int32))
+    sorter.close()
+
+
+@pytest.mark.parametrize("key_type", ["u32", "u64"])
+@pytest.mark.parametrize("kind", KINDS)
+def test_batch_units(kind, key_type):
+    """Batch segments of every unit shape (sizes at the shapes' edges)."""
+    bits = 32 if key_type == "u32" else 64
+    sizes = [2, 33, 2047, 2048, 2049, 4096, 8192, 8193, 16384, 16385, 32767, 32768, 50000, 140001]
+    off = np.concatenate([[0], np.cumsum(sizes)]).astype(np.uint64)
+    keys = _keys(kind, int(off[-1]), bits, synth.seed_for(7, 7))
+    sorter = pkg.BucketSorter()
+    d = torch.from_numpy(keys.view(np.int32 if bits == 32 else np.int64)).cuda()
+    out = sorter.sort_batch(d, off, key_type=key_type)
+    sorter.sync()
+    got = out.cpu().numpy().view(keys.dtype)
+    for a, b in zip(off[:-1].astype(int), off[1:].astype(int)):
+        assert np.array_equal(got[a:b], np.sort(keys[a:b]))
+    sorter.close()
