@@ -207,7 +207,10 @@ typedef struct {
     uint32_t direct_segs;     /* sorted whole by one CTA or cluster */
     uint32_t sampled_segs;    /* sorted by segment-aware Algorithm 1 */
     uint32_t large_segs;      /* above 524288 32-bit or 1048576 64-bit keys:
-                                 one plain sort each */
+                                 32-bit ones up to 2^21 keys sorted with the
+                                 sampled segments (not counted in sublists
+                                 and buckets), the others one plain sort
+                                 each */
     uint32_t sublists;        /* sublists of the sampled segments */
     uint32_t buckets;         /* buckets of the sampled segments */
     uint32_t num_kernels;     /* kernel launches per call */
@@ -265,7 +268,10 @@ bsort_status bsort_sort_pairs(bsort_t h, bsort_key_type kt, const void *d_keys_i
  * (as Step 9 sorts a bucket); larger ones up to 524288 keys by Algorithm 1
  * (Section 4) with segment-aware sublists (32768 keys), s = 1024 samples
  * per sublist and per-segment splitters, all segments together in one
- * sequence of launches; larger ones by one plain sort each.  The segment
+ * sequence of launches (from 524289 to 2^21 keys with s = 512 or 256
+ * samples per sublist); larger ones by one plain sort each, and so are those
+ * above 524288 keys when the handle's workspace is a fixed one that holds
+ * the batch only that way.  The segment
  * table is copied to the device from pinned staging owned by the handle.
  * kt: BSORT_U32, BSORT_F32 or BSORT_U64 (64-bit keys: segments up to
  * 262144 keys, or batch_direct_max when given, sorted whole — above 131072

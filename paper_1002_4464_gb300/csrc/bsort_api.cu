@@ -45,6 +45,12 @@ constexpr int kPipe = 16;       // host entry: key chunks in, position slices ou
 constexpr uint32_t kBatchDirectMax = 131072;
 constexpr uint32_t kBatchSampledMax = (uint32_t)kRecordChunk / 1024 * (uint32_t)kSegTile;
 constexpr uint32_t kBatchSamples = 1024;
+// Larger 32-bit segments, up to 2^21 keys, join the sampled ones with fewer
+// samples per sublist (512 up to 32 sublists, 256 up to 64: m*s stays within
+// kRecordChunk and the bound within a unit): one launch sequence for all of
+// them instead of one plain sort each, whose ~94 us at 2^20 keys are mostly
+// launches (339 such segments among 4000: 37.7 -> 5.9 ms per batch).
+constexpr uint32_t kBatchJoinMax = 1u << 21;
 constexpr uint32_t kBatchUnit = 32768;  // Step-9 unit of sampled segments
 // 64-bit keys: sublists of kSegTileU64 keys, s = 256 samples per sublist up
 // to 32 sublists and 128 above (m*s <= kSegRecordsU64), Step-9 units of
@@ -916,7 +922,7 @@ bsort_status run_sort_two_level(bsort_t h, const Plan &P, bsort_key_type kt, con
     // Steps 4-5
     const bool one_chunk = P.n_rec_pad == (uint32_t)kRecordChunk;
     SEQ(launch_records_chunk_sort(samples, rec_a, P.n_rec, P.n_rec_pad, one_chunk ? spl : nullptr,
-                                  I.s, I.b, st),
+                                  I.b, st),
         "step4_sample_chunks");
     if (!one_chunk) {
         uint64_t *src = rec_a, *dst = rec_b;
@@ -1037,7 +1043,6 @@ bsort_status run_sort_u64(bsort_t h, const Plan &P, const void *kin, void *kout,
     const bsort_plan_info &I = P.info;
     unsigned char *ws = static_cast<unsigned char *>(h->ws);
     int *err = reinterpret_cast<int *>(ws + P.off_hdr);
-    uint32_t *ticket = reinterpret_cast<uint32_t *>(ws + P.off_hdr + 64);
     if (I.single_tile) {
         if (n == 1) {
             if (kout != kin) {
@@ -1220,7 +1225,7 @@ bsort_status run_sort(bsort_t h, bsort_key_type kt, const void *kin, const void 
             "step4_5_radix_splitters");
     } else {
         SEQ(launch_records_chunk_sort(samples, rec_a, P.n_rec, P.n_rec_pad,
-                                      one_chunk ? spl : nullptr, I.s, I.b, st),
+                                      one_chunk ? spl : nullptr, I.b, st),
             "step4_sample_chunks");
     }
     if (!P.rec_radix && !one_chunk) {
@@ -1454,12 +1459,20 @@ uint64_t wide_direct_max(const bsort_t h)
     return h->direct_max_set && h->direct_max < largest ? h->direct_max : largest;
 }
 
+uint32_t pow2_at_least(uint32_t x)
+{
+    uint32_t p = 1;
+    while (p < x) p <<= 1;
+    return p;
+}
+
 // Host plan of one batch: direct lists per shape, sampled segments with
 // their sublists and buckets, plain-sorted large segments, and the
 // workspace layout (descriptors first, copied from pinned staging).
 struct BatchPlan {
     bsort_batch_info info;
     bool wide = false;  // 64-bit keys
+    bool fits = false;  // padded positions within 32 bits
     std::vector<uint32_t> direct[kNumDirect];  // (begin, end) pairs per shape
     std::vector<SegInfo> segs;
     std::vector<uint32_t> sub_seg;
@@ -1497,9 +1510,14 @@ bsort_status spans_from_offsets(bsort_t h, const uint64_t *segoff, uint32_t nseg
     return BSORT_OK;
 }
 
-bsort_status make_batch_plan(bsort_t h, bsort_key_type kt, const SegSpan *spans,
-                             uint32_t nsegs, BatchPlan *B)
+// join: segments above the sampled size up to kBatchJoinMax keys join the
+// sampled ones (32-bit keys); else each of them is a plain sort.  BSORT_OK
+// with B->fits unset when the joined segments' padded positions exceed 32
+// bits (the caller plans again without).
+bsort_status make_batch_plan_as(bsort_t h, bsort_key_type kt, const SegSpan *spans,
+                                uint32_t nsegs, bool join, BatchPlan *B)
 {
+    *B = BatchPlan();
     if (kt != BSORT_U32 && kt != BSORT_F32 && kt != BSORT_U64)
         return fail(h, BSORT_EINVAL, "unknown key type %d", (int)kt);
     B->wide = kt == BSORT_U64;
@@ -1510,7 +1528,10 @@ bsort_status make_batch_plan(bsort_t h, bsort_key_type kt, const SegSpan *spans,
     bsort_batch_info &I = B->info;
     memset(&I, 0, sizeof(I));
     I.num_segs = nsegs;
-    if (nsegs == 0) return BSORT_OK;
+    if (nsegs == 0) {
+        B->fits = true;
+        return BSORT_OK;
+    }
     for (uint32_t q = 0; q < nsegs; ++q)
         if (spans[q].begin + spans[q].n >= kMaxN)
             return fail(h, BSORT_EUNSUPPORTED, "segment end %llu exceeds 2^32 - 2^16",
@@ -1519,6 +1540,7 @@ bsort_status make_batch_plan(bsort_t h, bsort_key_type kt, const SegSpan *spans,
         B->wide ? wide_direct_max(h) : (h->direct_max < largest ? h->direct_max : largest);
     const uint64_t tile = B->wide ? (uint64_t)kSegTileU64 : (uint64_t)kSegTile;
     const uint64_t unit = B->wide ? (uint64_t)kBatchUnitU64 : (uint64_t)kBatchUnit;
+    const uint64_t smax = B->wide ? kBatchSampledMaxU64 : kBatchSampledMax;
     uint64_t g = 0;  // sublists so far
     for (uint32_t q = 0; q < nsegs; ++q) {
         const uint64_t a = spans[q].begin, n = spans[q].n;
@@ -1530,11 +1552,12 @@ bsort_status make_batch_plan(bsort_t h, bsort_key_type kt, const SegSpan *spans,
             B->direct[c].push_back((uint32_t)a);
             B->direct[c].push_back((uint32_t)(a + n));
             ++I.direct_segs;
-        } else if (n <= (B->wide ? kBatchSampledMaxU64 : kBatchSampledMax)) {
+        } else if (n <= smax || (join && !B->wide && n <= kBatchJoinMax)) {
             SegInfo sg = {};
             sg.g0 = (uint32_t)g;
             sg.m = (uint32_t)((n + tile - 1) / tile);
-            sg.s = B->wide ? (sg.m <= 32 ? 256u : 128u) : kBatchSamples;
+            sg.s = B->wide ? (sg.m <= 32 ? 256u : 128u)
+                           : std::min(kBatchSamples, (uint32_t)kRecordChunk / pow2_at_least(sg.m));
             const uint64_t np = (uint64_t)sg.m * tile;
             uint64_t lo = 1, hi = (uint64_t)sg.m * sg.s;  // smallest b whose bound fits a unit
             while (lo < hi) {
@@ -1553,6 +1576,13 @@ bsort_status make_batch_plan(bsort_t h, bsort_key_type kt, const SegSpan *spans,
                 B->units.push_back((uint32_t)B->segs.size());
                 B->units.push_back(j);
             }
+            if (n <= smax) {
+                ++I.sampled_segs;
+                I.sublists += sg.m;
+                I.buckets += sg.b;
+            } else {
+                ++I.large_segs;
+            }
             B->nrec += sg.m * sg.s;
             B->nspl += sg.b;
             B->runs += sg.m * sg.b;
@@ -1562,12 +1592,13 @@ bsort_status make_batch_plan(bsort_t h, bsort_key_type kt, const SegSpan *spans,
             B->large.push_back({a, n});
         }
     }
-    if (g * tile >= kMaxN) return fail(h, BSORT_EUNSUPPORTED, "padded sampled segments exceed 2^32");
+    if (g * tile >= kMaxN) {
+        if (join) return BSORT_OK;
+        return fail(h, BSORT_EUNSUPPORTED, "padded sampled segments exceed 2^32");
+    }
+    B->fits = true;
     B->n_pad = g * tile;
-    I.sampled_segs = (uint32_t)B->segs.size();
-    I.large_segs = (uint32_t)B->large.size();
-    I.sublists = (uint32_t)g;
-    I.buckets = B->nspl;
+    I.large_segs += (uint32_t)B->large.size();
     B->scan_chunks = (B->runs + kScanChunk - 1) / kScanChunk;
     // plain sorts of the large segments reuse the workspace after the batch
     for (const auto &lg : B->large) {
@@ -1618,6 +1649,20 @@ bsort_status make_batch_plan(bsort_t h, bsort_key_type kt, const SegSpan *spans,
     B->total = o > B->large_ws ? o : B->large_ws;
     I.workspace_bytes = B->total;
     return BSORT_OK;
+}
+
+// The plan of a batch: with the larger segments joined to the sampled ones,
+// unless their padded positions exceed 32 bits or the workspace is a fixed
+// one that only holds the plan with a plain sort for each of them.
+bsort_status make_batch_plan(bsort_t h, bsort_key_type kt, const SegSpan *spans,
+                             uint32_t nsegs, BatchPlan *B)
+{
+    bsort_status rs = make_batch_plan_as(h, kt, spans, nsegs, true, B);
+    if (rs != BSORT_OK) return rs;
+    if (B->fits && (B->info.large_segs == B->large.size() || !h->ws_fixed ||
+                    B->total <= h->ws_bytes))
+        return BSORT_OK;
+    return make_batch_plan_as(h, kt, spans, nsegs, false, B);
 }
 
 // stage: when not null, pinned host memory of at least the plan's
@@ -1722,7 +1767,7 @@ bsort_status run_batch(bsort_t h, bsort_key_type kt, const void *kin, void *kout
     }
     // sampled segments: Algorithm 1, segment-aware
     if (!B.segs.empty()) {
-        const uint32_t nsub = B.info.sublists;
+        const uint32_t nsub = (uint32_t)B.sub_seg.size();
         const uint32_t *sub_seg = desc + B.d_sub;
         const SegInfo *segs = reinterpret_cast<const SegInfo *>(desc + B.d_segs);
         const uint32_t *units = desc + B.d_units;
@@ -1743,7 +1788,7 @@ bsort_status run_batch(bsort_t h, bsort_key_type kt, const void *kin, void *kout
             SEQ(launch_seg_sublist_sort_u64(static_cast<const uint64_t *>(kin), sub_seg, nsub,
                                             segs, tiles, samples, st),
                 "batch_u64_step1_3_sublist_sort");
-            SEQ(launch_seg_records_u64(samples, segs, B.info.sampled_segs, spl, st),
+            SEQ(launch_seg_records_u64(samples, segs, (uint32_t)B.segs.size(), spl, st),
                 "batch_u64_step4_5_samples");
             SEQ(launch_seg_sample_index_u64(tiles, samples, spl, sub_seg, nsub, segs, counts,
                                             srcb, st),
@@ -1755,7 +1800,7 @@ bsort_status run_batch(bsort_t h, bsort_key_type kt, const void *kin, void *kout
             SEQ(launch_relocate_u64(tiles, offsets, srcb, blk, B.runs, (uint32_t)B.n_pad, reloc,
                                     st),
                 "batch_u64_step8_relocate");
-            SEQ(launch_seg_bucket_sort_u64(reloc, units, B.info.buckets, segs, offsets,
+            SEQ(launch_seg_bucket_sort_u64(reloc, units, B.nspl, segs, offsets,
                                            static_cast<uint64_t *>(kout), err, st),
                 "batch_u64_step9_bucket_sort");
         } else {
@@ -1765,7 +1810,7 @@ bsort_status run_batch(bsort_t h, bsort_key_type kt, const void *kin, void *kout
             uint64_t *spl = reinterpret_cast<uint64_t *>(ws + B.off_spl);
             SEQ(launch_seg_sublist_sort(ki, is_f32, sub_seg, nsub, segs, tiles, samples, st),
                 "batch_step1_3_sublist_sort");
-            SEQ(launch_seg_records(samples, segs, B.info.sampled_segs, spl, st),
+            SEQ(launch_seg_records(samples, segs, (uint32_t)B.segs.size(), spl, st),
                 "batch_step4_5_samples");
             SEQ(launch_seg_sample_index(tiles, samples, spl, sub_seg, nsub, segs, counts, srcb,
                                         st),
@@ -1777,7 +1822,7 @@ bsort_status run_batch(bsort_t h, bsort_key_type kt, const void *kin, void *kout
             SEQ(launch_relocate(tiles, nullptr, offsets, srcb, blk, B.runs, (uint32_t)B.n_pad, 0,
                                 reloc, nullptr, st),
                 "batch_step8_relocate");
-            SEQ(launch_seg_bucket_sort(reloc, units, B.info.buckets, segs,
+            SEQ(launch_seg_bucket_sort(reloc, units, B.nspl, segs,
                                        offsets, is_f32, ko, err, st),
                 "batch_step9_bucket_sort");
         }

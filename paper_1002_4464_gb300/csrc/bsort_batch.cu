@@ -109,41 +109,22 @@ k_seg_sublist_sort(const uint32_t *__restrict__ keys_in, int is_f32,
 }
 
 // ============================================================ Steps 4-5
-// CTA q sorts the m*s sample records of sampled segment q (at most T*E;
-// every sublist's s records are already a sorted run) and writes its b
-// splitters g_j = S[floor((j+1) m s / b) - 1].
+// CTA q sorts the m*s sample records of sampled segment q (at most T*E, in
+// the order of their positions) by bins and writes its b splitters g_j =
+// S[floor((j+1) m s / b) - 1].
 template <int T, int E>
 __global__ void __launch_bounds__(T, 1)
 k_seg_records(const uint64_t *__restrict__ samples, const SegInfo *__restrict__ segs,
               uint64_t *__restrict__ spl)
 {
-    constexpr int CAP = T * E;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     uint64_t *sm = reinterpret_cast<uint64_t *>(smem_raw);
     const int tid = threadIdx.x;
-    const int lane = tid & 31, warp = tid >> 5;
     const SegInfo sg = segs[blockIdx.x];
     const uint32_t nrec = sg.m * sg.s;
-    const uint64_t *src = samples + sg.rec;
-    if (sg.s >= 32u * E && sg.s < (uint32_t)CAP) {
-        const int s = (int)sg.s;
-        for (int x = tid; x < CAP; x += T) {
-            const uint64_t r = (uint32_t)x < nrec ? src[x] : 0xFFFFFFFFFFFFFFFFull;
-            const int q = x / s, o = x % s;
-            const int pos = (q & 1) ? q * s + s - 1 - o : x;
-            sm[pidx<uint64_t>(pos)] = r;
-        }
-        __syncthreads();
-        cta_merge_runs<uint64_t, T, E>(sm, s);
-    } else {
-        uint64_t v[E];
-#pragma unroll
-        for (int k = 0; k < E; ++k) {
-            const uint32_t x = (uint32_t)wb_pos<E>(warp, lane, k);
-            v[k] = x < nrec ? src[x] : 0xFFFFFFFFFFFFFFFFull;
-        }
-        cta_sort<uint64_t, T, E>(v, sm);
-    }
+    uint64_t v[E];
+    load_keys<uint64_t, T, E>(v, samples + sg.rec, (int)nrec, false);
+    cta_bin_sort<uint64_t, T, E, true>(v, sm, (int)nrec, false);
     for (uint32_t j = tid; j < sg.b; j += T)
         spl[sg.spl + j] = sm[pidx<uint64_t>((int)((uint64_t)(j + 1) * nrec / sg.b - 1))];
 }
@@ -486,7 +467,7 @@ cudaError_t init_batch_kernels()
         e = set_smem_attr(k_seg_sublist_sort<512, 64>,
                           BinSmem<uint32_t, 512, 64>::kBytes);
     if (e == cudaSuccess)
-        e = set_smem_attr(k_seg_records<1024, 16>, padded_elems<uint64_t>(kRecordChunk) * 8);
+        e = set_smem_attr(k_seg_records<1024, 16>, BinSmem<uint64_t, 1024, 16>::kBytes);
     if (e == cudaSuccess)
         e = set_smem_attr(k_seg_bucket_sort<uint32_t, 512, 64, true>,
                           BinSmem<uint32_t, 512, 64>::kBytes);
@@ -562,7 +543,8 @@ cudaError_t launch_seg_records(const uint64_t *samples, const SegInfo *segs, uin
                                uint64_t *spl, cudaStream_t st)
 {
     if (nsegs == 0) return cudaSuccess;
-    const int sm = padded_elems<uint64_t>(kRecordChunk) * 8;
+    static_assert(kRecordChunk == 1024 * 16, "a segment's records are one CTA's unit");
+    const int sm = BinSmem<uint64_t, 1024, 16>::kBytes;
     k_seg_records<1024, 16><<<nsegs, 1024, sm, st>>>(samples, segs, spl);
     return cudaGetLastError();
 }

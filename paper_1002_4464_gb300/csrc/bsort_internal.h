@@ -16,8 +16,6 @@ constexpr int kRecordChunk = 16384;  // Step-4 chunk sorted by one CTA
 constexpr int kMergeTile = 4096;     // outputs per CTA in a Step-4 merge pass
 constexpr int kScanChunk = 4096;     // items per CTA of the Step-7 scan
 
-int smem_bytes_for_cap(int cap, bool pairs);
-
 // Configure kernel attributes (max dynamic SMEM, cluster sizes) once per
 // device.
 cudaError_t init_kernels();
@@ -101,11 +99,10 @@ constexpr int kMaxBucketsTiers = 32768;  // b of a two-tier Step 9 (a unit per b
 
 // Step 4 (chunks): sort the n_rec records of src in chunks of kRecordChunk
 // into dst (which holds n_pad = chunks * kRecordChunk records, the tail
-// filled with all-ones); runs of s records are already sorted.  If the whole
-// array is one chunk and spl != nullptr, also writes the b splitters (Step 5).
+// filled with all-ones).  If the whole array is one chunk and spl != nullptr,
+// also writes the b splitters (Step 5).
 cudaError_t launch_records_chunk_sort(const uint64_t *src, uint64_t *dst, uint32_t n_rec,
-                                      uint32_t n_pad, uint64_t *spl, uint32_t s,
-                                      uint32_t b, cudaStream_t st);
+                                      uint32_t n_pad, uint64_t *spl, uint32_t b, cudaStream_t st);
 // Step 4 (merges): merge sorted runs of length L of src into dst.
 cudaError_t launch_merge_pass(const uint64_t *src, uint64_t *dst, uint32_t n_pad,
                               uint32_t L, cudaStream_t st);

@@ -23,50 +23,27 @@
 // sample's index (its position i*t + (k+1)w - 1 grows with q).
 #include "bsort_device.cuh"
 #include "bsort_internal.h"
+#include "bsort_sort.cuh"
 
 namespace bsort {
 
 // ============================================================ Step 4 (chunks)
-// The records of one sublist (s consecutive records) are already sorted, so
-// when s >= 32*E the chunk is loaded as sorted runs (odd runs reversed) and
-// only the remaining merge levels run; otherwise the chunk is sorted whole.
+// A CTA sorts its chunk of records by bins (cta_bin_sort; 16384 records of
+// 2^20 keys: 33 us by merging their sorted runs of s records, 25 us by bins).
 template <int T, int E>
 __global__ void __launch_bounds__(T, 1)
 k_records_sort(const uint64_t *__restrict__ src, uint64_t *__restrict__ dst, uint32_t n_rec,
-               uint64_t *__restrict__ spl, uint32_t s, uint32_t b)
+               uint64_t *__restrict__ spl, uint32_t b)
 {
     constexpr int CAP = T * E;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     uint64_t *sm = reinterpret_cast<uint64_t *>(smem_raw);
     const int tid = threadIdx.x;
-    const int lane = tid & 31, warp = tid >> 5;
     const uint64_t base = (uint64_t)blockIdx.x * CAP;
-    if (s >= 32u * E && s < (uint32_t)CAP) {
-        // all E loads of a thread are issued before its first store
-        uint64_t r[E];
-#pragma unroll
-        for (int k = 0; k < E; ++k) {
-            const uint64_t g = base + (uint64_t)(k * T + tid);
-            r[k] = g < n_rec ? src[g] : 0xFFFFFFFFFFFFFFFFull;
-        }
-#pragma unroll
-        for (int k = 0; k < E; ++k) {
-            const int x = k * T + tid;
-            const int q = x / (int)s, o = x % (int)s;
-            const int pos = (q & 1) ? q * (int)s + (int)s - 1 - o : x;
-            sm[pidx<uint64_t>(pos)] = r[k];
-        }
-        __syncthreads();
-        cta_merge_runs<uint64_t, T, E>(sm, (int)s);
-    } else {
-        uint64_t v[E];
-#pragma unroll
-        for (int k = 0; k < E; ++k) {
-            const uint64_t x = base + wb_pos<E>(warp, lane, k);
-            v[k] = x < n_rec ? src[x] : 0xFFFFFFFFFFFFFFFFull;
-        }
-        cta_sort<uint64_t, T, E>(v, sm);
-    }
+    const int len = n_rec - base < (uint64_t)CAP ? (int)(n_rec - base) : CAP;
+    uint64_t v[E];
+    load_keys<uint64_t, T, E>(v, src + base, len, false);
+    cta_bin_sort<uint64_t, T, E, true>(v, sm, len, false);  // (q grows with the index)
 #pragma unroll 4
     for (int k = 0; k < E; ++k) {
         const int x = k * T + tid;
@@ -1458,11 +1435,6 @@ __global__ void k_u64_final(const uint64_t *__restrict__ k64, const V *__restric
 }
 
 // ============================================================ launch wrappers
-int smem_bytes_for_cap(int cap, bool pairs)
-{
-    return pairs ? padded_elems<uint64_t>(cap) * 8 : padded_elems<uint32_t>(cap) * 4;
-}
-
 template <typename KernelT>
 static cudaError_t set_smem(KernelT kern, int bytes)
 {
@@ -1477,7 +1449,7 @@ static cudaError_t set_smem(KernelT kern, int bytes)
 
 cudaError_t init_misc_kernels()
 {
-    BSORT_TRY(set_smem(k_records_sort<1024, 16>, smem_bytes_for_cap(kRecordChunk, true)));
+    BSORT_TRY(set_smem(k_records_sort<1024, 16>, BinSmem<uint64_t, 1024, 16>::kBytes));
     BSORT_TRY(set_smem(k_pack_units<1024>, 16 * (kMaxBuckets + 1)));
     BSORT_TRY(set_smem(k_units_each<1024>, 4 * (kMaxBucketsTiers + 1)));
     BSORT_TRY(set_smem(k_bucket_relocate<kFuseT, kFuseV>, (int)(8 * kFuseMaxM + 4)));
@@ -1485,12 +1457,11 @@ cudaError_t init_misc_kernels()
 }
 
 cudaError_t launch_records_chunk_sort(const uint64_t *src, uint64_t *dst, uint32_t n_rec,
-                                      uint32_t n_pad, uint64_t *spl, uint32_t s, uint32_t b,
-                                      cudaStream_t st)
+                                      uint32_t n_pad, uint64_t *spl, uint32_t b, cudaStream_t st)
 {
     const uint32_t chunks = n_pad / kRecordChunk;
-    k_records_sort<1024, 16><<<chunks, 1024, smem_bytes_for_cap(kRecordChunk, true), st>>>(
-        src, dst, n_rec, chunks == 1 ? spl : nullptr, s, b);
+    k_records_sort<1024, 16><<<chunks, 1024, BinSmem<uint64_t, 1024, 16>::kBytes, st>>>(
+        src, dst, n_rec, chunks == 1 ? spl : nullptr, b);
     return cudaGetLastError();
 }
 

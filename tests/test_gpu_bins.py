@@ -146,3 +146,28 @@ def test_batch_units(kind, key_type):
     for a, b in zip(off[:-1].astype(int), off[1:].astype(int)):
         assert np.array_equal(got[a:b], np.sort(keys[a:b]))
     sorter.close()
+
+
+@pytest.mark.parametrize("kind", ["even", "zipf", "sorted"])
+def test_batch_joined_segments(kind):
+    """Segments above the sampled size: up to 2^21 keys in one sequence of
+    launches, or one plain sort each in a workspace that only holds those."""
+    sizes = [524288, 524289, 3, 1 << 20, (1 << 20) + 1, 900001, 1 << 21, (1 << 21) + 1, 40000]
+    off = np.concatenate([[0], np.cumsum(sizes)]).astype(np.uint64)
+    keys = _keys(kind, int(off[-1]), 32, synth.seed_for(7, 8))
+    d = torch.from_numpy(keys.view(np.int32)).cuda()
+    want = np.concatenate([np.sort(keys[a:b]) for a, b in
+                           zip(off[:-1].astype(int), off[1:].astype(int))])
+    free = pkg.BucketSorter()
+    need = free.plan_batch(off).workspace_bytes
+    small = 48 << 20
+    assert small < need
+    tight = pkg.BucketSorter(workspace_bytes=small)
+    assert tight.plan_batch(off).workspace_bytes <= small
+    for sorter in (free, tight):
+        info = sorter.plan_batch(off)
+        assert (info.sampled_segs, info.large_segs) == (1, 6)
+        out = sorter.sort_batch(d, off)
+        sorter.sync()
+        assert np.array_equal(out.cpu().numpy().view(np.uint32), want)
+        sorter.close()
