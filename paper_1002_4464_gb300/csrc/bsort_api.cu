@@ -1180,6 +1180,11 @@ bsort_status run_sort(bsort_t h, bsort_key_type kt, const void *kin, const void 
         if (e != cudaSuccess) return cuda_fail(h, e, "memset(scan ticket)");
     }
 
+    if (P.rec_radix) {
+        e = launch_records_zero(P.n_rec, ws + P.off_rs, st);
+        if (e != cudaSuccess) return cuda_fail(h, e, "memset(record scratch)");
+    }
+
     // Steps 1-3
     if (hp) {
         // chunk c: copy its sublists' keys in, then sort them

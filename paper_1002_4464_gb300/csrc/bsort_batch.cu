@@ -117,6 +117,7 @@ __global__ void __launch_bounds__(T, 1)
 k_seg_records(const uint64_t *__restrict__ samples, const SegInfo *__restrict__ segs,
               uint64_t *__restrict__ spl)
 {
+    grid_dep_wait();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     uint64_t *sm = reinterpret_cast<uint64_t *>(smem_raw);
     const int tid = threadIdx.x;
@@ -141,6 +142,7 @@ k_seg_sample_index(const uint32_t *__restrict__ tiles_k, const uint64_t *__restr
                    const SegInfo *__restrict__ segs, uint32_t t, uint32_t *__restrict__ counts,
                    uint32_t *__restrict__ srcb)
 {
+    grid_dep_wait();
     __shared__ uint32_t c[T + 1];
     const int tid = threadIdx.x;
     const uint32_t g = blockIdx.x;
@@ -189,6 +191,7 @@ k_seg_bucket_sort(const K *__restrict__ reloc_k, const uint32_t *__restrict__ un
                   const SegInfo *__restrict__ segs, const uint32_t *__restrict__ offsets,
                   uint32_t t, int is_f32, K *__restrict__ keys_out, int *err)
 {
+    grid_dep_wait();
     constexpr int CH = T * E;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     K *sm = reinterpret_cast<K *>(smem_raw);
@@ -285,6 +288,7 @@ __global__ void __launch_bounds__(T, 1)
 k_seg_records_u64(const Rec128 *__restrict__ samples, const SegInfo *__restrict__ segs,
                   Rec128 *__restrict__ spl)
 {
+    grid_dep_wait();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     Rec128 *sm = reinterpret_cast<Rec128 *>(smem_raw);
     const SegInfo sg = segs[blockIdx.x];
@@ -323,6 +327,7 @@ k_seg_sample_index_u64(const uint64_t *__restrict__ tiles_k, const Rec128 *__res
                        const SegInfo *__restrict__ segs, uint32_t t, uint32_t *__restrict__ counts,
                        uint32_t *__restrict__ srcb)
 {
+    grid_dep_wait();
     __shared__ uint32_t c[T + 1];
     const int tid = threadIdx.x;
     const uint32_t g = blockIdx.x;
@@ -545,7 +550,7 @@ cudaError_t launch_seg_records(const uint64_t *samples, const SegInfo *segs, uin
     if (nsegs == 0) return cudaSuccess;
     static_assert(kRecordChunk == 1024 * 16, "a segment's records are one CTA's unit");
     const int sm = BinSmem<uint64_t, 1024, 16>::kBytes;
-    k_seg_records<1024, 16><<<nsegs, 1024, sm, st>>>(samples, segs, spl);
+    launch_dep(k_seg_records<1024, 16>, nsegs, 1024, sm, st, samples, segs, spl);
     return cudaGetLastError();
 }
 
@@ -555,8 +560,8 @@ cudaError_t launch_seg_sample_index(const uint32_t *tiles_k, const uint64_t *sam
                                     cudaStream_t st)
 {
     if (nsub == 0) return cudaSuccess;
-    k_seg_sample_index<128><<<nsub, 128, 0, st>>>(tiles_k, samples, spl, sub_seg, segs,
-                                                  (uint32_t)kSegTile, counts, srcb);
+    launch_dep(k_seg_sample_index<128>, nsub, 128, 0, st, tiles_k, samples, spl, sub_seg, segs,
+               (uint32_t)kSegTile, counts, srcb);
     return cudaGetLastError();
 }
 
@@ -565,9 +570,9 @@ cudaError_t launch_seg_bucket_sort(const uint32_t *reloc_k, const uint32_t *unit
                                    uint32_t *keys_out, int *err, cudaStream_t st)
 {
     if (nunits == 0) return cudaSuccess;
-    k_seg_bucket_sort<uint32_t, 512, 64, true>
-        <<<nunits, 512, BinSmem<uint32_t, 512, 64>::kBytes, st>>>(
-            reloc_k, units, segs, offsets, (uint32_t)kSegTile, is_f32, keys_out, err);
+    launch_dep(k_seg_bucket_sort<uint32_t, 512, 64, true>, nunits, 512,
+               BinSmem<uint32_t, 512, 64>::kBytes, st, reloc_k, units, segs, offsets,
+               (uint32_t)kSegTile, is_f32, keys_out, err);
     return cudaGetLastError();
 }
 
@@ -586,8 +591,8 @@ cudaError_t launch_seg_records_u64(const Rec128 *samples, const SegInfo *segs, u
                                    Rec128 *spl, cudaStream_t st)
 {
     if (nsegs == 0) return cudaSuccess;
-    k_seg_records_u64<1024><<<nsegs, 1024, kSegRecordsU64 * sizeof(Rec128), st>>>(samples, segs,
-                                                                                  spl);
+    launch_dep(k_seg_records_u64<1024>, nsegs, 1024, kSegRecordsU64 * sizeof(Rec128), st, samples,
+               segs, spl);
     return cudaGetLastError();
 }
 
@@ -597,8 +602,8 @@ cudaError_t launch_seg_sample_index_u64(const uint64_t *tiles_k, const Rec128 *s
                                         uint32_t *srcb, cudaStream_t st)
 {
     if (nsub == 0) return cudaSuccess;
-    k_seg_sample_index_u64<128><<<nsub, 128, 0, st>>>(tiles_k, samples, spl, sub_seg, segs,
-                                                      (uint32_t)kSegTileU64, counts, srcb);
+    launch_dep(k_seg_sample_index_u64<128>, nsub, 128, 0, st, tiles_k, samples, spl, sub_seg,
+               segs, (uint32_t)kSegTileU64, counts, srcb);
     return cudaGetLastError();
 }
 
@@ -608,9 +613,9 @@ cudaError_t launch_seg_bucket_sort_u64(const uint64_t *reloc_k, const uint32_t *
                                        cudaStream_t st)
 {
     if (nunits == 0) return cudaSuccess;
-    k_seg_bucket_sort<uint64_t, 1024, 16, true>
-        <<<nunits, 1024, BinSmem<uint64_t, 1024, 16>::kBytes, st>>>(
-            reloc_k, units, segs, offsets, (uint32_t)kSegTileU64, 0, keys_out, err);
+    launch_dep(k_seg_bucket_sort<uint64_t, 1024, 16, true>, nunits, 1024,
+               BinSmem<uint64_t, 1024, 16>::kBytes, st, reloc_k, units, segs, offsets,
+               (uint32_t)kSegTileU64, 0, keys_out, err);
     return cudaGetLastError();
 }
 

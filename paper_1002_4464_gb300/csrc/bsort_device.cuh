@@ -74,6 +74,17 @@ __device__ __forceinline__ void prefetch_l2(const void *p, uint64_t bytes)
     }
 }
 
+// First statement of a kernel that launch_dep starts: waits until the kernel
+// before it in the stream has finished and its writes are visible (returns
+// at once in a launch without the attribute).  No kernel calls
+// griddepcontrol.launch_dependents: the next one's CTAs are set up as this
+// one's end (with the call at the top, CTAs set up earlier cost more than
+// they saved: 2^24 uint64 653 us against 596, 2^24 floats 418 against 390).
+__device__ __forceinline__ void grid_dep_wait()
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 template <typename K> struct KeyMax;
 template <> struct KeyMax<uint32_t> { static constexpr uint32_t v = 0xFFFFFFFFu; };
 template <> struct KeyMax<uint64_t> { static constexpr uint64_t v = 0xFFFFFFFFFFFFFFFFull; };

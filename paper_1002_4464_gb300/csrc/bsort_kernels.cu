@@ -35,6 +35,7 @@ __global__ void __launch_bounds__(T, 1)
 k_records_sort(const uint64_t *__restrict__ src, uint64_t *__restrict__ dst, uint32_t n_rec,
                uint64_t *__restrict__ spl, uint32_t b)
 {
+    grid_dep_wait();
     constexpr int CAP = T * E;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     uint64_t *sm = reinterpret_cast<uint64_t *>(smem_raw);
@@ -97,6 +98,7 @@ __global__ void __launch_bounds__(T, 4)
 k_merge_pass(const uint64_t *__restrict__ src, uint64_t *__restrict__ dst, uint32_t n_pad,
              uint32_t L)
 {
+    grid_dep_wait();
     constexpr int TILE = T * E;
     __shared__ uint64_t sm[padded_elems<uint64_t>(TILE)];
     __shared__ uint32_t s_split[2];
@@ -157,6 +159,7 @@ k_merge_pass(const uint64_t *__restrict__ src, uint64_t *__restrict__ dst, uint3
 __global__ void k_select_splitters(const uint64_t *__restrict__ sorted, uint32_t n_rec,
                                    uint32_t b, uint64_t *__restrict__ spl)
 {
+    grid_dep_wait();
     const uint32_t j = blockIdx.x * blockDim.x + threadIdx.x;
     if (j < b) spl[j] = sorted[(uint64_t)(j + 1) * n_rec / b - 1];
 }
@@ -194,6 +197,7 @@ __global__ void k_seg_ranges(const uint32_t *__restrict__ tiles_k, const uint64_
                              uint32_t t, uint32_t s, uint32_t b, uint32_t m, uint32_t nseg,
                              uint32_t seg, uint32_t *__restrict__ jr)
 {
+    grid_dep_wait();
     const uint32_t idx = blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= m * nseg) return;
     const uint32_t i = idx / nseg, k = idx % nseg;
@@ -222,6 +226,7 @@ k_sample_index_grp(const uint32_t *__restrict__ tiles_k, const uint64_t *__restr
                    uint32_t t, uint32_t s, uint32_t b, uint32_t m, uint32_t nseg, uint32_t seg_rt,
                    const uint32_t *__restrict__ jr, uint32_t *__restrict__ cum)
 {
+    grid_dep_wait();
     const uint32_t seg = SEG ? (uint32_t)SEG : seg_rt;
     __shared__ __align__(16) uint32_t sk[kSub6 * kSegRow];
     __shared__ uint32_t s_lo[kSub6], s_hi[kSub6];
@@ -338,6 +343,7 @@ k_scan(const uint32_t *__restrict__ in, uint32_t *__restrict__ out, uint32_t n_i
        uint32_t m, uint32_t t, uint32_t *__restrict__ counts, uint32_t *__restrict__ srcb,
        int spin_limit, int stall_first)
 {
+    grid_dep_wait();
     __shared__ uint32_t s_chunk;
     __shared__ uint32_t s_warp[T / 32];
     __shared__ uint32_t s_prefix;
@@ -488,6 +494,7 @@ __global__ void __launch_bounds__(T)
 k_row_scan(const uint32_t *__restrict__ cum, uint32_t m, uint32_t t, uint32_t *__restrict__ out,
            uint32_t *__restrict__ counts, uint32_t *__restrict__ srcb)
 {
+    grid_dep_wait();
     constexpr int N = T * V;
     constexpr int W = T / 32;
     __shared__ uint32_t s_items[N + N / 32];
@@ -674,6 +681,7 @@ k_relocate(const KT *__restrict__ tiles_k, const void *__restrict__ tiles_v,
            uint32_t n_pad, int val_bytes, KT *__restrict__ reloc_k,
            void *__restrict__ reloc_v)
 {
+    grid_dep_wait();
     constexpr int W = T / 32;
     constexpr int P = kBlockItems / 32;  // positions per lane
     __shared__ uint32_t s_off[W][kRelocRunsCap + 1];
@@ -834,6 +842,7 @@ k_bucket_relocate(const uint32_t *__restrict__ cum, uint32_t m, uint32_t t, uint
                   const void *__restrict__ tiles_v, int val_bytes, uint32_t *__restrict__ offsets,
                   uint32_t *__restrict__ reloc_k, void *__restrict__ reloc_v)
 {
+    grid_dep_wait();
     constexpr int W = T / 32;
     constexpr int P = kBlockItems / 32;  // positions per lane in a block
     static_assert(V % 4 == 0, "V must be a multiple of 4");
@@ -1067,6 +1076,7 @@ k_units_each(const uint32_t *__restrict__ offsets, uint32_t m, uint32_t b, uint3
              uint32_t Q1, uint32_t Q2, uint32_t *__restrict__ units,
              uint32_t *__restrict__ units2, int *err)
 {
+    grid_dep_wait();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     uint32_t *Lb = reinterpret_cast<uint32_t *>(smem_raw);  // b + 1
     __shared__ uint32_t s_warp[T / 32];
@@ -1131,6 +1141,7 @@ k_pack_units(const uint32_t *__restrict__ offsets, uint32_t m, uint32_t b, uint3
              uint32_t Q1, uint32_t Q2, uint32_t *__restrict__ units,
              uint32_t *__restrict__ units2, int *err)
 {
+    grid_dep_wait();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     uint32_t *Lb = reinterpret_cast<uint32_t *>(smem_raw);  // b + 1
     uint32_t *nxt = Lb + (b + 1);                             // b + 1
@@ -1234,6 +1245,7 @@ k_pack_units(const uint32_t *__restrict__ offsets, uint32_t m, uint32_t b, uint3
 __global__ void k_block_index(uint32_t *__restrict__ offsets, uint32_t runs, uint32_t n_pad,
                               uint32_t *__restrict__ blk, uint32_t nblk)
 {
+    grid_dep_wait();
     const uint32_t b = blockIdx.x * blockDim.x + threadIdx.x;
     if (b == 0) offsets[runs] = n_pad;
     if (b >= nblk) return;
@@ -1416,6 +1428,7 @@ __global__ void k_u64_split(const uint64_t *__restrict__ k64, uint32_t *__restri
 __global__ void k_u64_gather_hi(const uint64_t *__restrict__ k64, const uint32_t *__restrict__ p1,
                                 uint32_t *__restrict__ hi, uint64_t n)
 {
+    grid_dep_wait();
     for (uint64_t x = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; x < n;
          x += (uint64_t)gridDim.x * blockDim.x)
         hi[x] = (uint32_t)(k64[p1[x]] >> 32);
@@ -1426,6 +1439,7 @@ __global__ void k_u64_final(const uint64_t *__restrict__ k64, const V *__restric
                             const uint32_t *__restrict__ p1, const uint32_t *__restrict__ p2,
                             uint64_t *__restrict__ out_k, V *__restrict__ out_v, uint64_t n)
 {
+    grid_dep_wait();
     for (uint64_t y = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; y < n;
          y += (uint64_t)gridDim.x * blockDim.x) {
         const uint32_t src = p1[p2[y]];
@@ -1460,8 +1474,8 @@ cudaError_t launch_records_chunk_sort(const uint64_t *src, uint64_t *dst, uint32
                                       uint32_t n_pad, uint64_t *spl, uint32_t b, cudaStream_t st)
 {
     const uint32_t chunks = n_pad / kRecordChunk;
-    k_records_sort<1024, 16><<<chunks, 1024, BinSmem<uint64_t, 1024, 16>::kBytes, st>>>(
-        src, dst, n_rec, chunks == 1 ? spl : nullptr, b);
+    launch_dep(k_records_sort<1024, 16>, chunks, 1024, BinSmem<uint64_t, 1024, 16>::kBytes, st,
+               src, dst, n_rec, chunks == 1 ? spl : nullptr, b);
     return cudaGetLastError();
 }
 
@@ -1472,14 +1486,14 @@ cudaError_t launch_merge_pass(const uint64_t *src, uint64_t *dst, uint32_t n_pad
     // multiples of kRecordChunk, itself a multiple of kMergeTile
     static_assert(kRecordChunk % kMergeTile == 0, "merge tiles must divide record chunks");
     if (n_pad % kRecordChunk != 0 || L % kRecordChunk != 0) return cudaErrorInvalidValue;
-    k_merge_pass<256, 16><<<n_pad / kMergeTile, 256, 0, st>>>(src, dst, n_pad, L);
+    launch_dep(k_merge_pass<256, 16>, n_pad / kMergeTile, 256, 0, st, src, dst, n_pad, L);
     return cudaGetLastError();
 }
 
 cudaError_t launch_select_splitters(const uint64_t *sorted, uint32_t n_rec, uint32_t b,
                                     uint64_t *spl, cudaStream_t st)
 {
-    k_select_splitters<<<(b + 255) / 256, 256, 0, st>>>(sorted, n_rec, b, spl);
+    launch_dep(k_select_splitters, (b + 255) / 256, 256, 0, st, sorted, n_rec, b, spl);
     return cudaGetLastError();
 }
 
@@ -1491,16 +1505,17 @@ cudaError_t launch_sample_index(const uint32_t *tiles_k, const uint64_t *spl, ui
     const uint32_t seg = t < (uint32_t)kSegItems ? t : (uint32_t)kSegItems;
     const uint32_t nseg = t / seg;
     const uint32_t ns = m * nseg;
-    k_seg_ranges<<<(ns + 255) / 256, 256, 0, st>>>(tiles_k, spl, t, s, b, m, nseg, seg, jr);
+    launch_dep(k_seg_ranges, (ns + 255) / 256, 256, 0, st, tiles_k, spl, t, s, b, m, nseg, seg,
+               jr);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     const uint32_t groups = (m + kSub6 - 1) / kSub6;
     if (seg == (uint32_t)kSegItems)
-        k_sample_index_grp<256, kSegItems><<<groups * nseg, 256, 0, st>>>(tiles_k, spl, t, s, b,
-                                                                         m, nseg, seg, jr, cum);
+        launch_dep(k_sample_index_grp<256, kSegItems>, groups * nseg, 256, 0, st, tiles_k, spl, t,
+                   s, b, m, nseg, seg, jr, cum);
     else
-        k_sample_index_grp<256, 0><<<groups * nseg, 256, 0, st>>>(tiles_k, spl, t, s, b, m, nseg,
-                                                                 seg, jr, cum);
+        launch_dep(k_sample_index_grp<256, 0>, groups * nseg, 256, 0, st, tiles_k, spl, t, s, b,
+                   m, nseg, seg, jr, cum);
     return cudaGetLastError();
 }
 
@@ -1508,8 +1523,8 @@ cudaError_t launch_scan(const uint32_t *in, uint32_t *out, uint32_t n_items,
                         unsigned long long *status, uint32_t *ticket, int *err, cudaStream_t st)
 {
     const uint32_t chunks = (n_items + kScanChunk - 1) / kScanChunk;
-    k_scan<256, 16><<<chunks, 256, 0, st>>>(in, out, n_items, status, ticket, err, nullptr, 1u,
-                                            0u, nullptr, nullptr, kSpinLimit, 0);
+    launch_dep(k_scan<256, 16>, chunks, 256, 0, st, in, out, n_items, status, ticket, err,
+               nullptr, 1u, 0u, nullptr, nullptr, kSpinLimit, 0);
     return cudaGetLastError();
 }
 
@@ -1519,10 +1534,9 @@ cudaError_t launch_scan_cum(const uint32_t *cum, uint32_t m, uint32_t t, uint32_
                             cudaStream_t st, bool stall_first)
 {
     const uint32_t chunks = (n_items + kScanChunk - 1) / kScanChunk;
-    k_scan<256, 16><<<chunks, 256, 0, st>>>(nullptr, out, n_items, status, ticket, err, cum, m,
-                                            t, counts, srcb,
-                                            stall_first ? kTestSpinLimit : kSpinLimit,
-                                            stall_first ? 1 : 0);
+    launch_dep(k_scan<256, 16>, chunks, 256, 0, st, nullptr, out, n_items, status, ticket, err,
+               cum, m, t, counts, srcb, stall_first ? kTestSpinLimit : kSpinLimit,
+               stall_first ? 1 : 0);
     return cudaGetLastError();
 }
 
@@ -1534,8 +1548,8 @@ cudaError_t launch_relocate(const uint32_t *tiles_k, const void *tiles_v, const 
     constexpr int T = (kRelocPart / kBlockItems) * 32;
     const uint32_t grid = (n_pad + kRelocPart - 1) / kRelocPart;
     if (srcb == nullptr && (cum == nullptr || m == 0)) return cudaErrorInvalidValue;
-    k_relocate<T, uint32_t><<<grid, T, 0, st>>>(tiles_k, tiles_v, offsets, srcb, cum, m, t, blk,
-                                                runs, n_pad, val_bytes, reloc_k, reloc_v);
+    launch_dep(k_relocate<T, uint32_t>, grid, T, 0, st, tiles_k, tiles_v, offsets, srcb, cum, m,
+               t, blk, runs, n_pad, val_bytes, reloc_k, reloc_v);
     return cudaGetLastError();
 }
 
@@ -1547,8 +1561,8 @@ cudaError_t launch_bucket_relocate(const uint32_t *cum, uint32_t m, uint32_t t, 
                                   void *reloc_v, cudaStream_t st)
 {
     if (!bucket_relocate_fits(m) || b == 0) return cudaErrorInvalidValue;
-    k_bucket_relocate<kFuseT, kFuseV><<<b, kFuseT, 8 * kFuseMaxM + 4, st>>>(
-        cum, m, t, b, n_pad, tiles_k, tiles_v, val_bytes, offsets, reloc_k, reloc_v);
+    launch_dep(k_bucket_relocate<kFuseT, kFuseV>, b, kFuseT, 8 * kFuseMaxM + 4, st, cum, m, t, b,
+               n_pad, tiles_k, tiles_v, val_bytes, offsets, reloc_k, reloc_v);
     return cudaGetLastError();
 }
 
@@ -1557,9 +1571,9 @@ cudaError_t launch_row_scan(const uint32_t *cum, uint32_t m, uint32_t t, uint32_
 {
     if (m == 0 || b == 0) return cudaSuccess;
     if (m <= 2048u)
-        k_row_scan<128, 16><<<b, 128, 0, st>>>(cum, m, t, out, counts, srcb);
+        launch_dep(k_row_scan<128, 16>, b, 128, 0, st, cum, m, t, out, counts, srcb);
     else
-        k_row_scan<512, 16><<<b, 512, 0, st>>>(cum, m, t, out, counts, srcb);
+        launch_dep(k_row_scan<512, 16>, b, 512, 0, st, cum, m, t, out, counts, srcb);
     return cudaGetLastError();
 }
 
@@ -1569,9 +1583,8 @@ cudaError_t launch_relocate_u64(const uint64_t *tiles_k, const uint32_t *offsets
 {
     constexpr int T = (kRelocPart / kBlockItems) * 32;
     const uint32_t grid = (n_pad + kRelocPart - 1) / kRelocPart;
-    k_relocate<T, uint64_t><<<grid, T, 0, st>>>(tiles_k, nullptr, offsets, srcb, nullptr, 1u, 0u,
-                                                blk, runs,
-                                                n_pad, 0, reloc_k, nullptr);
+    launch_dep(k_relocate<T, uint64_t>, grid, T, 0, st, tiles_k, nullptr, offsets, srcb, nullptr,
+               1u, 0u, blk, runs, n_pad, 0, reloc_k, nullptr);
     return cudaGetLastError();
 }
 
@@ -1579,7 +1592,7 @@ cudaError_t launch_block_index(uint32_t *offsets, uint32_t runs, uint32_t n_pad,
                                cudaStream_t st)
 {
     const uint32_t nblk = (n_pad + kBlockItems - 1) / kBlockItems;
-    k_block_index<<<(nblk + 255) / 256, 256, 0, st>>>(offsets, runs, n_pad, blk, nblk);
+    launch_dep(k_block_index, (nblk + 255) / 256, 256, 0, st, offsets, runs, n_pad, blk, nblk);
     return cudaGetLastError();
 }
 
@@ -1589,7 +1602,8 @@ cudaError_t launch_units_each(const uint32_t *offsets, uint32_t m, uint32_t b, u
 {
     if (b > (uint32_t)kMaxBucketsTiers || units2 == nullptr) return cudaErrorInvalidValue;
     const int sm = (int)(4 * (b + 1));
-    k_units_each<1024><<<1, 1024, sm, st>>>(offsets, m, b, n_pad, Q1, Q2, units, units2, err);
+    launch_dep(k_units_each<1024>, 1, 1024, sm, st, offsets, m, b, n_pad, Q1, Q2, units, units2,
+               err);
     return cudaGetLastError();
 }
 
@@ -1598,7 +1612,8 @@ cudaError_t launch_pack_units(const uint32_t *offsets, uint32_t m, uint32_t b, u
                               int *err, cudaStream_t st)
 {
     const int sm = (int)(4 * (b + 1) * 4);
-    k_pack_units<1024><<<1, 1024, sm, st>>>(offsets, m, b, n_pad, Q1, Q2, units, units2, err);
+    launch_dep(k_pack_units<1024>, 1, 1024, sm, st, offsets, m, b, n_pad, Q1, Q2, units, units2,
+               err);
     return cudaGetLastError();
 }
 
@@ -1692,7 +1707,7 @@ cudaError_t launch_u64_split(const uint64_t *k64, uint32_t *lo, uint32_t *iota, 
 cudaError_t launch_u64_gather_hi(const uint64_t *k64, const uint32_t *p1, uint32_t *hi,
                                  uint64_t n, cudaStream_t st)
 {
-    k_u64_gather_hi<<<elementwise_grid(n), 256, 0, st>>>(k64, p1, hi, n);
+    launch_dep(k_u64_gather_hi, elementwise_grid(n), 256, 0, st, k64, p1, hi, n);
     return cudaGetLastError();
 }
 
@@ -1701,13 +1716,13 @@ cudaError_t launch_u64_final(const uint64_t *k64, const void *vals, int val_byte
                              void *out_v, uint64_t n, cudaStream_t st)
 {
     if (val_bytes == 4)
-        k_u64_final<uint32_t><<<elementwise_grid(n), 256, 0, st>>>(
-            k64, static_cast<const uint32_t *>(vals), p1, p2, out_k,
-            static_cast<uint32_t *>(out_v), n);
+        launch_dep(k_u64_final<uint32_t>, elementwise_grid(n), 256, 0, st, k64,
+                   static_cast<const uint32_t *>(vals), p1, p2, out_k,
+                   static_cast<uint32_t *>(out_v), n);
     else
-        k_u64_final<uint64_t><<<elementwise_grid(n), 256, 0, st>>>(
-            k64, static_cast<const uint64_t *>(vals), p1, p2, out_k,
-            static_cast<uint64_t *>(out_v), n);
+        launch_dep(k_u64_final<uint64_t>, elementwise_grid(n), 256, 0, st, k64,
+                   static_cast<const uint64_t *>(vals), p1, p2, out_k,
+                   static_cast<uint64_t *>(out_v), n);
     return cudaGetLastError();
 }
 

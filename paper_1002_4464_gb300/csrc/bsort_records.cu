@@ -80,6 +80,7 @@ __global__ void __launch_bounds__(T)
 k_rec_hist(const uint64_t *__restrict__ rec, uint32_t n, uint32_t *__restrict__ hist,
            uint32_t *__restrict__ done, uint32_t *__restrict__ gbase)
 {
+    grid_dep_wait();
     static_assert(T == 256, "one thread per digit in the final scan");
     __shared__ uint32_t sh[4 * 256];
     for (int i = threadIdx.x; i < 4 * 256; i += T) sh[i] = 0u;
@@ -143,6 +144,7 @@ k_rec_pass(const uint64_t *__restrict__ in, uint64_t *__restrict__ out, uint32_t
            const uint32_t *__restrict__ gfirst, uint32_t *status, uint32_t *ticket, int *err,
            uint64_t *__restrict__ spl, uint32_t b)
 {
+    grid_dep_wait();
     static_assert(T == 512 && T * E == kRsTile, "16 warps, one thread per digit in the first 8");
     constexpr int W = T / 32;
     extern __shared__ __align__(16) uint32_t s_dyn[];
@@ -333,14 +335,17 @@ cudaError_t init_records_kernels()
                                 cudaFuncAttributeMaxDynamicSharedMemorySize, kRsSmemBytes);
 }
 
+cudaError_t launch_records_zero(uint32_t n_rec, void *scratch, cudaStream_t st)
+{
+    return cudaMemsetAsync(scratch, 0, records_radix_scratch_bytes(n_rec), st);
+}
+
 cudaError_t launch_records_hist(const uint64_t *samples, uint32_t n_rec, void *scratch, int sms,
                                 cudaStream_t st)
 {
-    cudaError_t e = cudaMemsetAsync(scratch, 0, records_radix_scratch_bytes(n_rec), st);
-    if (e != cudaSuccess) return e;
     const RsScratch r = rs_layout(scratch);
-    k_rec_hist<256><<<4 * (sms > 0 ? sms : 1), 256, 0, st>>>(samples, n_rec, r.hist,
-                                                              r.tickets + 8, r.gfirst);
+    launch_dep(k_rec_hist<256>,
+               4 * (sms > 0 ? sms : 1), 256, 0, st, samples, n_rec, r.hist, r.tickets + 8, r.gfirst);
     return cudaGetLastError();
 }
 
@@ -352,9 +357,9 @@ cudaError_t launch_records_pass(int p, const uint64_t *in, uint64_t *out, uint32
     if ((p < 3) != (out != nullptr) || (p == 3) != (spl != nullptr)) return cudaErrorInvalidValue;
     const uint32_t tiles = (n_rec + kRsTile - 1) / kRsTile;
     const RsScratch r = rs_layout(scratch);
-    k_rec_pass<kRsT, kRsE><<<tiles, kRsT, kRsSmemBytes, st>>>(
-        in, out, n_rec, 8 * p, r.gfirst + 256 * p, r.status + (uint64_t)p * tiles * 256u,
-        r.tickets + p, err, spl, b);
+    launch_dep(k_rec_pass<kRsT, kRsE>, tiles, kRsT, kRsSmemBytes, st, in, out, n_rec, 8 * p,
+               r.gfirst + 256 * p, r.status + (uint64_t)p * tiles * 256u, r.tickets + p, err, spl,
+               b);
     return cudaGetLastError();
 }
 

@@ -298,6 +298,7 @@ k_bucket_sort(const uint32_t *__restrict__ src_k, const void *__restrict__ src_v
               int val_bytes, uint32_t *__restrict__ out_k, void *__restrict__ out_v, int *err,
               GatherSrc g)
 {
+    grid_dep_wait();
     bucket_sort_unit<T, E, PAIRS, C, BINS>(blockIdx.x / C, src_k, src_v, units, n, n_pad, is_f32,
                                      val_bytes, out_k, out_v, err, g, num_sms() / C);
 }
@@ -396,6 +397,10 @@ inline cudaError_t launch_bucket_sort_t(const void *src_k, const void *src_v,
                                     static_cast<const uint32_t *>(src_k), src_v, units, n, n_pad,
                                     is_f32, val_bytes, static_cast<uint32_t *>(out_k), out_v,
                                     err, g, (const uint32_t *)nullptr);
+    if (C == 1 && units != nullptr)
+        return launch_dep(k_bucket_sort<T, E, PAIRS, C, BINS>, grid, T, (size_t)sm, st,
+                          static_cast<const uint32_t *>(src_k), src_v, units, n, n_pad, is_f32,
+                          val_bytes, static_cast<uint32_t *>(out_k), out_v, err, g);
     return launch_maybe_cluster(k_bucket_sort<T, E, PAIRS, C, BINS>, grid, T, sm, C, st,
                                 static_cast<const uint32_t *>(src_k), src_v, units, n, n_pad,
                                 is_f32, val_bytes, static_cast<uint32_t *>(out_k), out_v, err, g);

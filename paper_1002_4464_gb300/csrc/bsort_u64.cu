@@ -71,6 +71,7 @@ template <int T, int IT>
 __global__ void __launch_bounds__(T)
 k_rec_merge(const Rec128 *__restrict__ src, Rec128 *__restrict__ dst, uint32_t N, uint32_t L)
 {
+    grid_dep_wait();
     const uint64_t o = ((uint64_t)blockIdx.x * T + threadIdx.x) * IT;
     if (o >= N) return;
     const uint64_t a0 = o / (2ull * L) * (2ull * L);
@@ -132,6 +133,7 @@ __global__ void __launch_bounds__(T)
 k_rec_merge_tiled(const Rec128 *__restrict__ src, Rec128 *__restrict__ dst, uint32_t N,
                   uint32_t L)
 {
+    grid_dep_wait();
     constexpr int TILE = T * E;
     __shared__ Rec128 sm[TILE];
     __shared__ uint32_t s_split[2];
@@ -203,6 +205,7 @@ k_rec_merge_tiled(const Rec128 *__restrict__ src, Rec128 *__restrict__ dst, uint
 __global__ void k_select_splitters_u64(const Rec128 *__restrict__ sorted, uint32_t N, uint32_t b,
                                        Rec128 *__restrict__ spl)
 {
+    grid_dep_wait();
     const uint32_t j = blockIdx.x * blockDim.x + threadIdx.x;
     if (j < b) spl[j] = sorted[(uint64_t)(j + 1) * N / b - 1];
 }
@@ -219,6 +222,7 @@ __global__ void k_seg_ranges_u64(const uint64_t *__restrict__ tiles, const Rec12
                                  uint32_t t, uint32_t b, uint32_t m, uint32_t nseg, uint32_t seg,
                                  uint32_t *__restrict__ jr)
 {
+    grid_dep_wait();
     const uint32_t idx = blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= m * nseg) return;
     const uint32_t i = idx / nseg, k = idx % nseg;
@@ -244,6 +248,7 @@ k_sample_index_seg_u64(const uint64_t *__restrict__ tiles, const Rec128 *__restr
                        uint32_t t, uint32_t b, uint32_t m, uint32_t nseg, uint32_t seg,
                        const uint32_t *__restrict__ jr, uint32_t *__restrict__ cum)
 {
+    grid_dep_wait();
     static_assert(kSegItemsU64 % (2 * T) == 0, "whole uint4 loads per thread");
     __shared__ __align__(16) uint64_t sk[kSegItemsU64];
     const uint32_t i = blockIdx.x / nseg, k = blockIdx.x % nseg;
@@ -339,6 +344,7 @@ __global__ void __launch_bounds__(T, (min_ctas<uint64_t, T, E, C, true>()))
 k_bucket_sort_u64(const uint64_t *__restrict__ src, const uint32_t *__restrict__ units,
                   uint64_t n, uint64_t n_pad, uint64_t *__restrict__ out, int *err)
 {
+    grid_dep_wait();
     bucket_sort_unit_u64<T, E, C>(blockIdx.x / C, src, units, n, n_pad, out, err, num_sms() / C);
 }
 
@@ -393,6 +399,10 @@ cudaError_t launch_bucket_u64_t(const void *src, const uint32_t *units, uint32_t
         return launch_maybe_cluster(k_bucket_sort_u64_loop<T, E, C>, grid, T, sm, C, st,
                                     static_cast<const uint64_t *>(src), units, n, n_pad,
                                     static_cast<uint64_t *>(out), err);
+    if (C == 1 && units != nullptr)
+        return launch_dep(k_bucket_sort_u64<T, E, C>, grid, T, (size_t)sm, st,
+                          static_cast<const uint64_t *>(src), units, n, n_pad,
+                          static_cast<uint64_t *>(out), err);
     return launch_maybe_cluster(k_bucket_sort_u64<T, E, C>, grid, T, sm, C, st,
                                 static_cast<const uint64_t *>(src), units, n, n_pad,
                                 static_cast<uint64_t *>(out), err);
@@ -466,17 +476,17 @@ cudaError_t launch_rec_merge(const Rec128 *src, Rec128 *dst, uint32_t N, uint32_
     constexpr int T = 256, IT = 8;
     const uint32_t grid = (uint32_t)(((uint64_t)N + T * IT - 1) / (T * IT));
     if ((2ull * L) % (T * IT) == 0) {  // pairs of runs span whole tiles
-        k_rec_merge_tiled<T, IT><<<grid, T, 0, st>>>(src, dst, N, L);
+        launch_dep(k_rec_merge_tiled<T, IT>, grid, T, 0, st, src, dst, N, L);
         return cudaGetLastError();
     }
-    k_rec_merge<T, IT><<<grid, T, 0, st>>>(src, dst, N, L);
+    launch_dep(k_rec_merge<T, IT>, grid, T, 0, st, src, dst, N, L);
     return cudaGetLastError();
 }
 
 cudaError_t launch_select_splitters_u64(const Rec128 *sorted, uint32_t N, uint32_t b, Rec128 *spl,
                                         cudaStream_t st)
 {
-    k_select_splitters_u64<<<(b + 255) / 256, 256, 0, st>>>(sorted, N, b, spl);
+    launch_dep(k_select_splitters_u64, (b + 255) / 256, 256, 0, st, sorted, N, b, spl);
     return cudaGetLastError();
 }
 
@@ -488,10 +498,11 @@ cudaError_t launch_sample_index_seg_u64(const uint64_t *tiles, const Rec128 *spl
     const uint32_t seg = t < (uint32_t)kSegItemsU64 ? t : (uint32_t)kSegItemsU64;
     const uint32_t nseg = t / seg;
     const uint32_t ns = m * nseg;
-    k_seg_ranges_u64<<<(ns + 255) / 256, 256, 0, st>>>(tiles, spl, t, b, m, nseg, seg, jr);
+    launch_dep(k_seg_ranges_u64, (ns + 255) / 256, 256, 0, st, tiles, spl, t, b, m, nseg, seg, jr);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    k_sample_index_seg_u64<256><<<ns, 256, 0, st>>>(tiles, spl, t, b, m, nseg, seg, jr, cum);
+    launch_dep(k_sample_index_seg_u64<256>, ns, 256, 0, st, tiles, spl, t, b, m, nseg, seg, jr,
+               cum);
     return cudaGetLastError();
 }
 
