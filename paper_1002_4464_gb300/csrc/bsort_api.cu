@@ -329,11 +329,10 @@ double plan_cost(uint64_t np, uint64_t s, uint64_t runs, int tchunk, int tctas, 
            per_run * r;
 }
 
-// Measured plans for keys-only sorts of 32-bit keys whose Step-9 units
-// (and sublists of t = 32768) are radix-sorting CTAs: (t, s) per size
-// class of n, the fastest of a sweep of t in {32768, 65536, 131072} and s in
-// {512, ..., 8192} on GB300 (uniform keys; b chosen by the planner for each
-// pair, as below).  Sizes outside the table use the cost model.
+// Measured plans for keys-only sorts of 32-bit keys whose units are sorted
+// by bins: (t, s) per size class of n, the fastest of sweeps on GB300 (b
+// chosen by the planner for each pair, as below).  Sizes outside the table use
+// the cost model.
 struct TunedPlan {
     int log2n_max;  // n <= 2^log2n_max
     uint32_t t, s;
@@ -341,9 +340,25 @@ struct TunedPlan {
 const TunedPlan kTuned[] = {
 #include "bsort_tuned.inc"
 };
+// The same for pairs with 32-bit keys, by n_max * 1024 items.
+struct TunedPairs {
+    uint32_t n_max, t, s;
+};
+const TunedPairs kTunedPairs[] = {
+#include "bsort_tuned_pairs.inc"
+};
 
-bool tuned_plan(uint64_t n, uint64_t *t, uint64_t *s)
+bool tuned_plan(bool pairs, uint64_t n, uint64_t *t, uint64_t *s)
 {
+    if (pairs) {
+        for (const TunedPairs &e : kTunedPairs)
+            if (n <= (uint64_t)e.n_max << 10) {
+                *t = e.t;
+                *s = e.s;
+                return true;
+            }
+        return false;
+    }
     for (const TunedPlan &e : kTuned) {
         if (n <= (1ull << e.log2n_max)) {
             *t = e.t;
@@ -520,14 +535,15 @@ bsort_status make_plan_with(bsort_t h, bsort_key_type kt, uint32_t vb, uint64_t 
         I.unit_capacity = (uint64_t)uchunk * uctas;
         I.num_kernels = n > 1 ? 1 : 0;
     } else {
-        // keys-only 32-bit sorts with radix units take (t, s) from the table
-        // measured for n's size class; the bucket count is then chosen below
-        // as for any plan
-        const bool radix_ok = vb == 0 && kt != BSORT_U64 &&
-                              !(h && (h->flags & (BSORT_FLAG_MERGE_SORT | BSORT_FLAG_PLAN_MODEL)));
+        // sorts of 32-bit keys take (t, s) from the table measured for n's
+        // size class (keys only: with units sorted by bins); the bucket
+        // count is then chosen below as for any plan
+        const uint32_t off = vb ? BSORT_FLAG_PLAN_MODEL
+                                : BSORT_FLAG_MERGE_SORT | BSORT_FLAG_PLAN_MODEL;
+        const bool table_ok = kt != BSORT_U64 && !(h && (h->flags & off));
         uint64_t tt = 0, ts = 0;
-        if (use_table && radix_ok && !forced_t && !forced_s && !forced_b &&
-            tuned_plan(n, &tt, &ts)) {
+        if (use_table && table_ok && !forced_t && !forced_s && !forced_b &&
+            tuned_plan(vb != 0, n, &tt, &ts)) {
             forced_t = tt;
             forced_s = ts;
             auto_b = true;
