@@ -204,7 +204,11 @@ typedef struct {
 typedef struct {
     uint64_t n;               /* keys in all segments */
     uint32_t num_segs;
-    uint32_t direct_segs;     /* sorted whole by one CTA or cluster */
+    uint32_t direct_segs;     /* up to batch_direct_max keys: sorted whole by
+                                 one CTA or cluster (64-bit keys, with
+                                 batch_direct_max 0 and many of them: those
+                                 above one CTA's unit with the sampled
+                                 segments, not counted there) */
     uint32_t sampled_segs;    /* sorted by segment-aware Algorithm 1 */
     uint32_t large_segs;      /* above 524288 32-bit or 1048576 64-bit keys:
                                  32-bit ones up to 2^21 keys sorted with the
@@ -265,7 +269,9 @@ bsort_status bsort_sort_pairs(bsort_t h, bsort_key_type kt, const void *d_keys_i
  * HOST memory, num_segs + 1 nondecreasing values, the last below 2^32 -
  * 2^16; keys outside every segment are left untouched.  Segments up to
  * batch_direct_max keys are sorted whole by one CTA or thread-block cluster
- * (as Step 9 sorts a bucket); larger ones up to 524288 keys by Algorithm 1
+ * (as Step 9 sorts a bucket; where batch_direct_max is left to the library,
+ * 64-bit segments above one CTA's unit join the larger ones when they hold
+ * 2^22 keys in all); larger ones up to 524288 keys by Algorithm 1
  * (Section 4) with segment-aware sublists (32768 keys), s = 1024 samples
  * per sublist and per-segment splitters, all segments together in one
  * sequence of launches (from 524289 to 2^21 keys with s = 512 or 256

@@ -51,6 +51,13 @@ constexpr uint32_t kBatchSamples = 1024;
 // them instead of one plain sort each, whose ~94 us at 2^20 keys are mostly
 // launches (339 such segments among 4000: 37.7 -> 5.9 ms per batch).
 constexpr uint32_t kBatchJoinMax = 1u << 21;
+// 64-bit direct segments above one CTA's unit (clusters) join the sampled
+// ones too when they hold at least this many keys in all and batch_direct_max
+// is not given: the sampled route sorts 50 Gkeys/s, the clusters, whose merge
+// rounds go through distributed shared memory, 23, but its steps take about
+// 60 us however few the keys.  (32-bit keys: 5.74 ms joined, 5.80 not, for
+// 4000 arrays: left to the clusters.)
+constexpr uint64_t kBatchJoinDirectU64 = 1ull << 22;
 constexpr uint32_t kBatchUnit = 32768;  // Step-9 unit of sampled segments
 // 64-bit keys: sublists of kSegTileU64 keys, s = 256 samples per sublist up
 // to 32 sublists and 128 above (m*s <= kSegRecordsU64), Step-9 units of
@@ -1494,6 +1501,7 @@ struct BatchPlan {
     bsort_batch_info info;
     bool wide = false;  // 64-bit keys
     bool fits = false;  // padded positions within 32 bits
+    bool joined = false;  // segments of other classes take the sampled route
     std::vector<uint32_t> direct[kNumDirect];  // (begin, end) pairs per shape
     std::vector<SegInfo> segs;
     std::vector<uint32_t> sub_seg;
@@ -1532,9 +1540,11 @@ bsort_status spans_from_offsets(bsort_t h, const uint64_t *segoff, uint32_t nseg
 }
 
 // join: segments above the sampled size up to kBatchJoinMax keys join the
-// sampled ones (32-bit keys); else each of them is a plain sort.  BSORT_OK
-// with B->fits unset when the joined segments' padded positions exceed 32
-// bits (the caller plans again without).
+// sampled ones (32-bit keys), else each of them is a plain sort; and so do
+// 64-bit direct segments above one CTA's unit when there are enough of them,
+// else a cluster sorts each.  (The counts of *info go by the size classes.)
+// BSORT_OK with B->fits unset when the joined segments' padded positions
+// exceed 32 bits (the caller plans again without).
 bsort_status make_batch_plan_as(bsort_t h, bsort_key_type kt, const SegSpan *spans,
                                 uint32_t nsegs, bool join, BatchPlan *B)
 {
@@ -1562,12 +1572,19 @@ bsort_status make_batch_plan_as(bsort_t h, bsort_key_type kt, const SegSpan *spa
     const uint64_t tile = B->wide ? (uint64_t)kSegTileU64 : (uint64_t)kSegTile;
     const uint64_t unit = B->wide ? (uint64_t)kBatchUnitU64 : (uint64_t)kBatchUnit;
     const uint64_t smax = B->wide ? kBatchSampledMaxU64 : kBatchSampledMax;
+    uint64_t rmax = dmax;  // largest segment that takes the direct route
+    if (join && B->wide && !h->direct_max_set) {
+        uint64_t keys = 0;
+        for (uint32_t q = 0; q < nsegs; ++q)
+            if (spans[q].n > unit && spans[q].n <= dmax) keys += spans[q].n;
+        if (keys >= kBatchJoinDirectU64) rmax = unit;
+    }
     uint64_t g = 0;  // sublists so far
     for (uint32_t q = 0; q < nsegs; ++q) {
         const uint64_t a = spans[q].begin, n = spans[q].n;
         I.n += n;
         if (n <= 1) continue;  // nothing to order (a copy when out != in)
-        if (n <= dmax) {
+        if (n <= rmax) {
             int c = 0;
             while ((uint64_t)shapes[c][0] * shapes[c][1] < n) ++c;
             B->direct[c].push_back((uint32_t)a);
@@ -1597,13 +1614,16 @@ bsort_status make_batch_plan_as(bsort_t h, bsort_key_type kt, const SegSpan *spa
                 B->units.push_back((uint32_t)B->segs.size());
                 B->units.push_back(j);
             }
-            if (n <= smax) {
+            if (n <= dmax) {
+                ++I.direct_segs;
+            } else if (n <= smax) {
                 ++I.sampled_segs;
                 I.sublists += sg.m;
                 I.buckets += sg.b;
             } else {
                 ++I.large_segs;
             }
+            B->joined |= n <= dmax || n > smax;
             B->nrec += sg.m * sg.s;
             B->nspl += sg.b;
             B->runs += sg.m * sg.b;
@@ -1672,17 +1692,15 @@ bsort_status make_batch_plan_as(bsort_t h, bsort_key_type kt, const SegSpan *spa
     return BSORT_OK;
 }
 
-// The plan of a batch: with the larger segments joined to the sampled ones,
-// unless their padded positions exceed 32 bits or the workspace is a fixed
-// one that only holds the plan with a plain sort for each of them.
+// The plan of a batch: with segments of other classes joined to the sampled
+// ones, unless their padded positions exceed 32 bits or the workspace is a
+// fixed one that only holds the plan without.
 bsort_status make_batch_plan(bsort_t h, bsort_key_type kt, const SegSpan *spans,
                              uint32_t nsegs, BatchPlan *B)
 {
     bsort_status rs = make_batch_plan_as(h, kt, spans, nsegs, true, B);
     if (rs != BSORT_OK) return rs;
-    if (B->fits && (B->info.large_segs == B->large.size() || !h->ws_fixed ||
-                    B->total <= h->ws_bytes))
-        return BSORT_OK;
+    if (B->fits && (!B->joined || !h->ws_fixed || B->total <= h->ws_bytes)) return BSORT_OK;
     return make_batch_plan_as(h, kt, spans, nsegs, false, B);
 }
 

@@ -275,44 +275,84 @@ k_seg_sublist_sort_u64(const uint64_t *__restrict__ keys_in, const uint32_t *__r
     }
 }
 
-// Steps 4-5: CTA q ranks the N = m*s sample records of sampled segment q
-// in shared memory instead of sorting them.  Every sublist's s records are
-// a sorted run and no two records are equal (their positions differ), so
-// the rank of a record is its index in its own run plus, for each other
-// run, the number of that run's records below it (a binary search).  The
-// record of rank floor((j+1) N / b) - 1 is splitter j, the same choice as
-// the 32-bit path's sorted records; each rank is the splitter of at most
-// one j (b <= N), namely j = ceil((rank+1) b / N) - 1 when that j maps back.
-template <int T>
+// Steps 4-5: CTA q picks the b splitters of sampled segment q, the records of
+// rank r_j = floor((j+1) N / b) - 1 of its N = m*s samples in (key, p) order.
+// It keeps the sublists' samples (sorted runs of s keys) in shared memory and
+// sorts a copy of all the keys by bins: the key at r_j is the splitter's.
+// Among the samples of that key, which go by position, it is number
+// r_j - (samples below the key): a warp takes a splitter, its lanes count in
+// two runs each (binary searches), and a prefix over the runs finds the run
+// that holds it.  (Ranking every record by a search of every run took 500 us
+// for 144 segments of 17 to 64 sublists.)
+template <int T, int E>
 __global__ void __launch_bounds__(T, 1)
 k_seg_records_u64(const Rec128 *__restrict__ samples, const SegInfo *__restrict__ segs,
-                  Rec128 *__restrict__ spl)
+                  Rec128 *__restrict__ spl, uint32_t t)
 {
     grid_dep_wait();
+    static_assert(T * E == (int)kSegRecordsU64, "a segment's records are one CTA's unit");
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    Rec128 *sm = reinterpret_cast<Rec128 *>(smem_raw);
+    uint64_t *sm = reinterpret_cast<uint64_t *>(smem_raw);
+    uint64_t *runs = reinterpret_cast<uint64_t *>(smem_raw + BinSmem<uint64_t, T, E>::kBytes);
     const SegInfo sg = segs[blockIdx.x];
-    const uint32_t s = sg.s, N = sg.m * sg.s;
+    const uint32_t s = sg.s, N = sg.m * sg.s, w = t / s;
     const Rec128 *src = samples + sg.rec;
-    for (uint32_t x = threadIdx.x; x < N; x += T) sm[x] = src[x];
-    __syncthreads();
-    for (uint32_t x = threadIdx.x; x < N; x += T) {
-        const Rec128 r = sm[x];
-        const uint32_t own = x / s;
-        uint64_t rank = x - own * s;
-        for (uint32_t i = 0; i < sg.m; ++i) {
-            if (i == own) continue;
-            const Rec128 *run = sm + (uint64_t)i * s;
-            uint32_t lo = 0, hi = s;
-            while (lo < hi) {
-                const uint32_t mid = (lo + hi) >> 1;
-                if (seg_rec_lt(run[mid], r)) lo = mid + 1;
-                else hi = mid;
+    const int lane = (int)threadIdx.x & 31, warp = (int)threadIdx.x >> 5;
+    uint64_t v[E];
+#pragma unroll
+    for (int k = 0; k < E; ++k) {
+        const uint32_t x = (uint32_t)wb_pos<E>(warp, lane, k);
+        v[k] = x < N ? src[x].key : KeyMax<uint64_t>::v;
+    }
+#pragma unroll
+    for (int k = 0; k < E; ++k) runs[wb_pos<E>(warp, lane, k)] = v[k];
+    cta_bin_sort<uint64_t, T, E>(v, sm, (int)N, false);  // (ends with a barrier)
+    for (uint32_t j = (uint32_t)warp; j < sg.b; j += T / 32) {
+        const uint32_t r = (uint32_t)((uint64_t)(j + 1) * N / sg.b - 1);
+        const uint64_t key = sm[pidx<uint64_t>((int)r)];
+        uint32_t first[2], count[2];  // of this key in runs lane and lane + 32
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const uint32_t i = (uint32_t)lane + 32u * h;
+            first[h] = count[h] = 0;
+            if (i < sg.m) {
+                const uint64_t *run = runs + i * s;
+                uint32_t lo = 0, hi = s;
+                while (lo < hi) {
+                    const uint32_t mid = (lo + hi) >> 1;
+                    if (run[mid] < key) lo = mid + 1;
+                    else hi = mid;
+                }
+                first[h] = lo;
+                hi = s;
+                while (lo < hi) {
+                    const uint32_t mid = (lo + hi) >> 1;
+                    if (run[mid] <= key) lo = mid + 1;
+                    else hi = mid;
+                }
+                count[h] = lo - first[h];
             }
-            rank += lo;
         }
-        const uint64_t j = ((rank + 1) * sg.b + N - 1) / N - 1;
-        if (j < sg.b && (j + 1) * N / sg.b - 1 == rank) spl[sg.spl + j] = r;
+        const uint32_t below = __reduce_add_sync(0xFFFFFFFFu, first[0] + first[1]);
+        uint32_t nth = r - below;  // among the key's samples, by position
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            uint32_t inc = count[h];
+#pragma unroll
+            for (int d = 1; d < 32; d <<= 1) {
+                const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, inc, d);
+                if (lane >= d) inc += y;
+            }
+            const uint32_t pre = inc - count[h];
+            if (nth >= pre && nth < inc) {
+                const uint32_t i = (uint32_t)lane + 32u * h, k = first[h] + nth - pre;
+                Rec128 rec;
+                rec.key = key;
+                rec.p = (uint64_t)(sg.g0 + i) * t + (uint64_t)(k + 1) * w - 1;
+                spl[sg.spl + j] = rec;
+            }
+            nth -= __shfl_sync(0xFFFFFFFFu, inc, 31);  // (wraps past the run found: no match)
+        }
     }
 }
 
@@ -375,6 +415,9 @@ k_seg_sample_index_u64(const uint64_t *__restrict__ tiles_k, const Rec128 *__res
         if (tid == 0) c[0] = carry;
     }
 }
+
+constexpr int kSegRecordsU64Smem =
+    BinSmem<uint64_t, 1024, 8>::kBytes + (int)(kSegRecordsU64 * sizeof(uint64_t));
 
 // ============================================================ launching
 namespace {
@@ -479,7 +522,7 @@ cudaError_t init_batch_kernels()
     if (e == cudaSuccess)
         e = set_smem_attr(k_seg_sublist_sort_u64<1024, 16>, BinSmem<uint64_t, 1024, 16>::kBytes);
     if (e == cudaSuccess)
-        e = set_smem_attr(k_seg_records_u64<1024>, (int)(kSegRecordsU64 * sizeof(Rec128)));
+        e = set_smem_attr(k_seg_records_u64<1024, 8>, kSegRecordsU64Smem);
     if (e == cudaSuccess)
         e = set_smem_attr(k_seg_bucket_sort<uint64_t, 1024, 16, true>,
                           BinSmem<uint64_t, 1024, 16>::kBytes);
@@ -591,8 +634,8 @@ cudaError_t launch_seg_records_u64(const Rec128 *samples, const SegInfo *segs, u
                                    Rec128 *spl, cudaStream_t st)
 {
     if (nsegs == 0) return cudaSuccess;
-    launch_dep(k_seg_records_u64<1024>, nsegs, 1024, kSegRecordsU64 * sizeof(Rec128), st, samples,
-               segs, spl);
+    launch_dep(k_seg_records_u64<1024, 8>, nsegs, 1024, kSegRecordsU64Smem, st, samples, segs,
+               spl, (uint32_t)kSegTileU64);
     return cudaGetLastError();
 }
 

@@ -171,3 +171,30 @@ def test_batch_joined_segments(kind):
         sorter.sync()
         assert np.array_equal(out.cpu().numpy().view(np.uint32), want)
         sorter.close()
+
+
+@pytest.mark.parametrize("kind", ["even", "zipf", "few"])
+def test_batch_joined_direct_segments(kind):
+    """Enough 64-bit segments above one CTA's unit take the sampled route (two
+    to eight sublists each); with the limit given they stay with clusters."""
+    unit, most = 16384, 131072
+    sizes = [unit, 5]
+    k = 0
+    while sum(sizes) < (1 << 22) + 2 * unit:
+        sizes.append(unit + 1 + (k * 7919) % (most - unit))
+        k += 1
+    sizes += [unit + 1, 2 * unit, most]
+    off = np.concatenate([[0], np.cumsum(sizes)]).astype(np.uint64)
+    keys = _keys(kind, int(off[-1]), 64, synth.seed_for(7, 9))
+    d = torch.from_numpy(keys.view(np.int64)).cuda()
+    outs = []
+    for limit in (0, most):
+        sorter = pkg.BucketSorter(batch_direct_max=limit)
+        assert sorter.plan_batch(off, "u64").direct_segs == len(sizes)
+        out = sorter.sort_batch(d, off, key_type="u64")
+        sorter.sync()
+        outs.append(out.cpu().numpy().view(keys.dtype))
+        sorter.close()
+    for a, b in zip(off[:-1].astype(int), off[1:].astype(int)):
+        assert np.array_equal(outs[0][a:b], np.sort(keys[a:b]))
+    assert np.array_equal(outs[0], outs[1])
