@@ -832,11 +832,15 @@ k_relocate(const KT *__restrict__ tiles_k, const void *__restrict__ tiles_v,
 // run by a population count, as k_relocate does, with coalesced stores to
 // B_j + y.  Nothing is read back from global memory but the keys (and
 // values) themselves: no run offsets, run starts or run index.
+// A CTA has one thread per kFuseV sublists, at least 128 (m <= 2048): with
+// fewer sublists buckets are smaller too, and eight CTAs of 128 threads share
+// an SM instead of two of 512 (whole sorts: 2^20 keys 77 -> 72 us, 2^26
+// staggered keys, m = 2048, 897 -> 883 us).
 constexpr int kFuseT = 512, kFuseV = 16;
 constexpr uint32_t kFuseMaxM = (uint32_t)(kFuseT * kFuseV);
 
 template <int T, int V>
-__global__ void __launch_bounds__(T, 2)
+__global__ void __launch_bounds__(T, 1024 / T)
 k_bucket_relocate(const uint32_t *__restrict__ cum, uint32_t m, uint32_t t, uint32_t b,
                   uint32_t n_pad, const uint32_t *__restrict__ tiles_k,
                   const void *__restrict__ tiles_v, int val_bytes, uint32_t *__restrict__ offsets,
@@ -1561,9 +1565,13 @@ cudaError_t launch_bucket_relocate(const uint32_t *cum, uint32_t m, uint32_t t, 
                                   void *reloc_v, cudaStream_t st)
 {
     if (!bucket_relocate_fits(m) || b == 0) return cudaErrorInvalidValue;
-    launch_dep(k_bucket_relocate<kFuseT, kFuseV>, b, kFuseT, 8 * kFuseMaxM + 4, st, cum, m, t, b,
-               n_pad, tiles_k, tiles_v, val_bytes, offsets, reloc_k, reloc_v);
-    return cudaGetLastError();
+#define L(T_)                                                                              \
+    return launch_dep(k_bucket_relocate<T_, kFuseV>, b, T_, 8 * T_ * kFuseV + 4, st, cum, m, t, \
+                      b, n_pad, tiles_k, tiles_v, val_bytes, offsets, reloc_k, reloc_v)
+    if (m <= 128u * kFuseV) L(128);
+    if (m <= 256u * kFuseV) L(256);
+    L(512);
+#undef L
 }
 
 cudaError_t launch_row_scan(const uint32_t *cum, uint32_t m, uint32_t t, uint32_t b,
