@@ -75,9 +75,11 @@ UNIT = "Gkeys/s"
 _CSRC = "paper_1002_4464_gb300/csrc/"
 KERNEL_SOURCES = {
     "k_sublist_sort": [_CSRC + "bsort_sort.cuh", _CSRC + "bsort_device.cuh",
-                       _CSRC + "bsort_radix.cuh", _CSRC + "bsort_sort_keys_radix.cu"],
+                       _CSRC + "bsort_binsort.cuh", _CSRC + "bsort_radix.cuh",
+                       _CSRC + "bsort_sort_keys_bins.cu"],
     "k_bucket_sort": [_CSRC + "bsort_sort.cuh", _CSRC + "bsort_device.cuh",
-                      _CSRC + "bsort_radix.cuh", _CSRC + "bsort_sort_keys_radix.cu"],
+                      _CSRC + "bsort_binsort.cuh", _CSRC + "bsort_radix.cuh",
+                       _CSRC + "bsort_sort_keys_bins.cu"],
 }
 KERNEL_SOURCES_DEFAULT = [_CSRC + "bsort_kernels.cu", _CSRC + "bsort_device.cuh"]
 

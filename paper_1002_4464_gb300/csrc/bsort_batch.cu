@@ -229,7 +229,7 @@ k_seg_bucket_sort(const K *__restrict__ reloc_k, const uint32_t *__restrict__ un
 
 // ============================================================ 64-bit keys
 // Sampled segments of 64-bit keys take the steps above with the widths of
-// the 64-bit path: sublists of kSegTileU64 keys sorted by comparisons, and
+// the 64-bit path: sublists of kSegTileU64 keys sorted by bins, and
 // sample records (key, p) of two 64-bit words, ordered key first, then p
 // (the composite order).
 __device__ __forceinline__ bool seg_rec_lt(const Rec128 &a, const Rec128 &b)
