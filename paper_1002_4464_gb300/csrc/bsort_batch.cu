@@ -115,7 +115,7 @@ k_seg_sublist_sort(const uint32_t *__restrict__ keys_in, int is_f32,
 template <int T, int E>
 __global__ void __launch_bounds__(T, 1)
 k_seg_records(const uint64_t *__restrict__ samples, const SegInfo *__restrict__ segs,
-              uint64_t *__restrict__ spl)
+              uint64_t *__restrict__ spl, uint32_t t)
 {
     grid_dep_wait();
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -123,11 +123,15 @@ k_seg_records(const uint64_t *__restrict__ samples, const SegInfo *__restrict__ 
     const int tid = threadIdx.x;
     const SegInfo sg = segs[blockIdx.x];
     const uint32_t nrec = sg.m * sg.s;
+    // (the padding's samples end the array in order: they stay out of the sort)
+    const uint32_t len = real_samples(sg.n, sg.m, t, sg.s);
     uint64_t v[E];
-    load_keys<uint64_t, T, E>(v, samples + sg.rec, (int)nrec, false);
-    cta_bin_sort<uint64_t, T, E, true>(v, sm, (int)nrec, false);
-    for (uint32_t j = tid; j < sg.b; j += T)
-        spl[sg.spl + j] = sm[pidx<uint64_t>((int)((uint64_t)(j + 1) * nrec / sg.b - 1))];
+    load_keys<uint64_t, T, E>(v, samples + sg.rec, (int)len, false);
+    cta_bin_sort<uint64_t, T, E, true>(v, sm, (int)len, false);
+    for (uint32_t j = tid; j < sg.b; j += T) {
+        const uint32_t x = (uint32_t)((uint64_t)(j + 1) * nrec / sg.b - 1);
+        spl[sg.spl + j] = x < len ? sm[pidx<uint64_t>((int)x)] : samples[sg.rec + x];
+    }
 }
 
 // ============================================================ Step 6
@@ -206,19 +210,20 @@ k_seg_bucket_sort(const K *__restrict__ reloc_k, const uint32_t *__restrict__ un
         if (tid == 0) set_error(err, DEV_INTERNAL);
         return;
     }
-    const int len = (int)(R - L);
+    // the unit's real items: the segment's padding ends its relocated order
+    // (and must not stretch the key range that the bins cut)
+    const uint32_t rel = L - P;
+    if (rel >= sg.n) return;
+    const int len = (int)min(R - L, sg.n - rel);
     if (len == 0) return;
     K v[E];
     load_keys<K, T, E>(v, reloc_k + L, len, false);
     chunk_sort<K, T, E, BINS>(v, sm, len, is_f32 != 0);
-    // ranks below lim hold real items of the segment (its padding sorts last)
-    const uint32_t rel = L - P;
-    const int lim = rel >= sg.n ? 0 : (sg.n - rel < (uint32_t)len ? (int)(sg.n - rel) : len);
     const uint64_t dst = (uint64_t)sg.out + rel;
 #pragma unroll 4
     for (int k = 0; k < E; ++k) {
         const int x = k * T + tid;
-        if (x < lim) {
+        if (x < len) {
             K key = sm[pidx<K>(x)];
             if constexpr (sizeof(K) == 4)
                 if (is_f32) key = f32_decode(key);
@@ -296,6 +301,7 @@ k_seg_records_u64(const Rec128 *__restrict__ samples, const SegInfo *__restrict_
     uint64_t *runs = reinterpret_cast<uint64_t *>(smem_raw + BinSmem<uint64_t, T, E>::kBytes);
     const SegInfo sg = segs[blockIdx.x];
     const uint32_t s = sg.s, N = sg.m * sg.s, w = t / s;
+    const int len = (int)real_samples(sg.n, sg.m, t, s);  // the padding's samples end each array
     const Rec128 *src = samples + sg.rec;
     const int lane = (int)threadIdx.x & 31, warp = (int)threadIdx.x >> 5;
     uint64_t v[E];
@@ -306,7 +312,7 @@ k_seg_records_u64(const Rec128 *__restrict__ samples, const SegInfo *__restrict_
     }
 #pragma unroll
     for (int k = 0; k < E; ++k) runs[wb_pos<E>(warp, lane, k)] = v[k];
-    cta_bin_sort<uint64_t, T, E>(v, sm, (int)N, false);  // (ends with a barrier)
+    cta_bin_sort<uint64_t, T, E>(v, sm, len, false);  // (ends with a barrier)
     for (uint32_t j = (uint32_t)warp; j < sg.b; j += T / 32) {
         const uint32_t r = (uint32_t)((uint64_t)(j + 1) * N / sg.b - 1);
         const uint64_t key = sm[pidx<uint64_t>((int)r)];
@@ -593,7 +599,8 @@ cudaError_t launch_seg_records(const uint64_t *samples, const SegInfo *segs, uin
     if (nsegs == 0) return cudaSuccess;
     static_assert(kRecordChunk == 1024 * 16, "a segment's records are one CTA's unit");
     const int sm = BinSmem<uint64_t, 1024, 16>::kBytes;
-    launch_dep(k_seg_records<1024, 16>, nsegs, 1024, sm, st, samples, segs, spl);
+    launch_dep(k_seg_records<1024, 16>, nsegs, 1024, sm, st, samples, segs, spl,
+               (uint32_t)kSegTile);
     return cudaGetLastError();
 }
 

@@ -30,10 +30,14 @@ namespace bsort {
 // ============================================================ Step 4 (chunks)
 // A CTA sorts its chunk of records by bins (cta_bin_sort; 16384 records of
 // 2^20 keys: 33 us by merging their sorted runs of s records, 25 us by bins).
+// The samples of the last sublist's padding, records n_real .. n_rec - 1, are
+// the largest in order as they stand: they are left there, so that their
+// code does not stretch the key range that the bins cut (400001 keys below
+// 10^6: 63 us against 108).
 template <int T, int E>
 __global__ void __launch_bounds__(T, 1)
 k_records_sort(const uint64_t *__restrict__ src, uint64_t *__restrict__ dst, uint32_t n_rec,
-               uint64_t *__restrict__ spl, uint32_t b)
+               uint32_t n_real, uint64_t *__restrict__ spl, uint32_t b)
 {
     grid_dep_wait();
     constexpr int CAP = T * E;
@@ -41,18 +45,20 @@ k_records_sort(const uint64_t *__restrict__ src, uint64_t *__restrict__ dst, uin
     uint64_t *sm = reinterpret_cast<uint64_t *>(smem_raw);
     const int tid = threadIdx.x;
     const uint64_t base = (uint64_t)blockIdx.x * CAP;
-    const int len = n_rec - base < (uint64_t)CAP ? (int)(n_rec - base) : CAP;
+    const int len = n_real <= base ? 0 : (int)min((uint64_t)CAP, n_real - base);
     uint64_t v[E];
     load_keys<uint64_t, T, E>(v, src + base, len, false);
     cta_bin_sort<uint64_t, T, E, true>(v, sm, len, false);  // (q grows with the index)
 #pragma unroll 4
     for (int k = 0; k < E; ++k) {
         const int x = k * T + tid;
-        dst[base + x] = sm[pidx<uint64_t>(x)];
+        dst[base + x] = x < len || base + x >= n_rec ? sm[pidx<uint64_t>(x)] : src[base + x];
     }
     if (spl != nullptr) {  // whole sample array in this one chunk: Step 5
-        for (uint32_t j = tid; j < b; j += T)
-            spl[j] = sm[pidx<uint64_t>((int)((uint64_t)(j + 1) * n_rec / b - 1))];
+        for (uint32_t j = tid; j < b; j += T) {
+            const int x = (int)((uint64_t)(j + 1) * n_rec / b - 1);
+            spl[j] = x < len ? sm[pidx<uint64_t>(x)] : src[x];
+        }
     }
 }
 
@@ -1475,11 +1481,12 @@ cudaError_t init_misc_kernels()
 }
 
 cudaError_t launch_records_chunk_sort(const uint64_t *src, uint64_t *dst, uint32_t n_rec,
-                                      uint32_t n_pad, uint64_t *spl, uint32_t b, cudaStream_t st)
+                                      uint32_t n_real, uint32_t n_pad, uint64_t *spl, uint32_t b,
+                                      cudaStream_t st)
 {
     const uint32_t chunks = n_pad / kRecordChunk;
     launch_dep(k_records_sort<1024, 16>, chunks, 1024, BinSmem<uint64_t, 1024, 16>::kBytes, st,
-               src, dst, n_rec, chunks == 1 ? spl : nullptr, b);
+               src, dst, n_rec, n_real, chunks == 1 ? spl : nullptr, b);
     return cudaGetLastError();
 }
 

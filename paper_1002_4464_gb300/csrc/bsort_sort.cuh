@@ -196,7 +196,11 @@ bucket_sort_unit(uint32_t u, const uint32_t *__restrict__ src_k, const void *__r
         if (tid == 0) set_error(err, DEV_INTERNAL);
         return;  // uniform per cluster: no CTA of it reaches a cluster barrier
     }
-    if (len64 == 0) return;
+    // Padding is the tail [n, n_pad) of the relocated order: the unit's real
+    // items end before it, and the sort must not take its codes for keys
+    // (they would stretch the key range that the bins cut).
+    const uint64_t end = R < n ? R : n;
+    if (L >= end) return;
     if (!direct && !gather && tid == 0 && r == 0 && prefetch_stride) {
         // the unit this SM will most likely sort next
         const uint32_t un = u + prefetch_stride;
@@ -205,7 +209,7 @@ bucket_sort_unit(uint32_t u, const uint32_t *__restrict__ src_k, const void *__r
             if (pl < pr && pr <= n_pad) prefetch_l2(src_k + pl, 4ull * (pr - pl));
         }
     }
-    const int len = (int)len64;
+    const int len = (int)(end - L);
     const int off = r * CH;  // ranks of the sorted unit this CTA writes
     // the unit's real items are spread evenly over the cluster's CTAs, so
     // that padding (skipped by whole warps) is shared by all of them
@@ -266,12 +270,10 @@ bucket_sort_unit(uint32_t u, const uint32_t *__restrict__ src_k, const void *__r
     }
     chunk_sort<K, T, E, BINS, PAIRS>(v, sm, uend > ustart ? uend - ustart : 0, is_f32 != 0);
     cluster_merge<K, T, E, C>(sm, len, per);
-    const uint64_t lim64 = min((unsigned long long)len, (unsigned long long)(n > L ? n - L : 0));
-    const int lim = (int)lim64;
 #pragma unroll 4
     for (int k = 0; k < E; ++k) {
         const int x = k * T + tid;
-        if (off + x < lim) {
+        if (off + x < len) {
             const K e = sm[pidx<K>(x)];
             uint32_t key = PAIRS ? (uint32_t)((uint64_t)e >> 32) : (uint32_t)e;
             if (is_f32) key = f32_decode(key);

@@ -312,8 +312,9 @@ bucket_sort_unit_u64(uint32_t u, const uint64_t *__restrict__ src,
         if (tid == 0) set_error(err, DEV_INTERNAL);
         return;
     }
-    if (R == L) return;
-    const int len = (int)(R - L);
+    const uint64_t end = R < n ? R : n;  // (padding ends the relocated order: not sorted)
+    if (L >= end) return;
+    const int len = (int)(end - L);
     const int per = C == 1 ? CH : (len + C - 1) / C;
     const int ustart = r * per;
     const int uend = min(ustart + per, len);
@@ -330,12 +331,10 @@ bucket_sort_unit_u64(uint32_t u, const uint64_t *__restrict__ src,
     chunk_sort<uint64_t, T, E, true>(v, sm, uend > ustart ? uend - ustart : 0, false);
     cluster_merge<uint64_t, T, E, C>(sm, len, per);
     const int off = r * CH;
-    const uint64_t lim64 = min((unsigned long long)len, (unsigned long long)(n > L ? n - L : 0));
-    const int lim = (int)lim64;
 #pragma unroll 4
     for (int k = 0; k < E; ++k) {
         const int x = k * T + tid;
-        if (off + x < lim) out[L + off + x] = sm[pidx<uint64_t>(x)];
+        if (off + x < len) out[L + off + x] = sm[pidx<uint64_t>(x)];
     }
 }
 
