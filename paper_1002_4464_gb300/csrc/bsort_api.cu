@@ -945,7 +945,7 @@ bsort_status run_sort_two_level(bsort_t h, const Plan &P, bsort_key_type kt, con
     // Steps 4-5
     const bool one_chunk = P.n_rec_pad == (uint32_t)kRecordChunk;
     SEQ(launch_records_chunk_sort(samples, rec_a, P.n_rec, real_samples(n, I.m, I.t, I.s),
-                                  P.n_rec_pad, one_chunk ? spl : nullptr, I.b, st),
+                                  P.n_rec_pad, one_chunk ? spl : nullptr, I.s, I.b, st),
         "step4_sample_chunks");
     if (!one_chunk) {
         uint64_t *src = rec_a, *dst = rec_b;
@@ -1253,7 +1253,7 @@ bsort_status run_sort(bsort_t h, bsort_key_type kt, const void *kin, const void 
             "step4_5_radix_splitters");
     } else {
         SEQ(launch_records_chunk_sort(samples, rec_a, P.n_rec, real_samples(n, I.m, I.t, I.s),
-                                      P.n_rec_pad, one_chunk ? spl : nullptr, I.b, st),
+                                      P.n_rec_pad, one_chunk ? spl : nullptr, I.s, I.b, st),
             "step4_sample_chunks");
     }
     if (!P.rec_radix && !one_chunk) {

@@ -54,7 +54,7 @@ k_seg_sort(const K *__restrict__ keys_in, K *__restrict__ keys_out,
     const int uend = min(ustart + per, len);
     K v[E];
     load_keys<K, T, E>(v, keys_in + L + ustart, uend - ustart, is_f32 != 0);
-    chunk_sort<K, T, E, BINS>(v, sm, uend > ustart ? uend - ustart : 0, is_f32 != 0);
+    chunk_sort<K, T, E, BINS, false, true>(v, sm, uend > ustart ? uend - ustart : 0, is_f32 != 0);
     cluster_merge<K, T, E, C>(sm, len, per);
     const int off = r * CH;
 #pragma unroll 4
@@ -127,7 +127,7 @@ k_seg_records(const uint64_t *__restrict__ samples, const SegInfo *__restrict__ 
     const uint32_t len = real_samples(sg.n, sg.m, t, sg.s);
     uint64_t v[E];
     load_keys<uint64_t, T, E>(v, samples + sg.rec, (int)len, false);
-    cta_bin_sort<uint64_t, T, E, true>(v, sm, (int)len, false);
+    cta_bin_sort<uint64_t, T, E, true, true>(v, sm, (int)len, false, (int)sg.s);
     for (uint32_t j = tid; j < sg.b; j += T) {
         const uint32_t x = (uint32_t)((uint64_t)(j + 1) * nrec / sg.b - 1);
         spl[sg.spl + j] = x < len ? sm[pidx<uint64_t>((int)x)] : samples[sg.rec + x];

@@ -32,23 +32,32 @@
 // are fewer values than lanes, so that a warp's atomics do not meet on one
 // counter) and needs no step 4.
 //
-// Skewed keys (bin_skewed; a bin of more than kBinPhases keys): every bin b
-// of n_b keys is cut once more, linearly into n_b bins at positions
-// [P_b, P_b + n_b) of the order, so that crowded stretches of the range get
-// as many bins as they hold keys, and two repeated values that shared a bin
-// part.  (A bin with an eighth of the unit or more takes every 16th of those
-// positions, and its keys are spread over the 16 by lane: a value repeated
-// that often would otherwise meet on one counter; pairs, whose equal keys must
-// keep their order, are instead cut a third time, by position.)  What is left unordered
-// inside the refined bins is put right by up to kBinPhases phases, by a
-// comparison sort of the warps where that is not enough, and by merging all
-// runs when two warps still overlap.  When a bin holds a quarter of the unit
-// and its keys differ (one key far from the others, keys spread over their
-// logarithm), refining would not part them: the unit is sorted by digits
-// or comparisons instead.  (1024 values, Zipf 1.1: 445 us against 515 by
-// digits as 32768-key units, 381 against 584 by comparisons as 16384; 2048:
-// 344 against 314; 64-bit keys 327 against 764, pairs 398 against 771 as
-// 16384; 32-bit keys spread over their logarithm: 756 against 512.)
+// Keys that crowd.  Before anything is counted, one key of each thread is
+// sampled and its place in the map's bins is looked at (BinSort::crowded);
+// where they meet far more often than a smooth density's do, the unit takes
+//   the bins of the logarithm of key - kmin (bin_again; floats: of their
+//   codes), if the sample is spread there: keys over many scales, or most of
+//   them near kmin and some far off;
+//   else the sort that the bins replaced (bin_other): comparisons, digits for
+//   32768-key units of 32-bit keys, merges where the unit is made of runs.
+// A unit that passes may still have a bin of more than kBinPhases keys: a value
+// repeated often, or two that share a bin.  bin_skewed then cuts every bin b
+// of n_b keys once more, linearly into n_b bins at positions [P_b, P_b + n_b)
+// of the order, so that crowded stretches of the range get as many bins as
+// they hold keys.  (A bin with an eighth of the unit or more takes every 16th
+// of those positions, and its keys are spread over the 16 by lane: a value
+// repeated that often would otherwise meet on one counter; pairs, whose equal
+// keys must keep their order, are instead cut a third time, by position.)
+// The sample is looked at again in the refined bins.  What is left unordered
+// inside them is put right by up to kBinPhases phases, by a comparison sort
+// of the warps where that is not enough, and by bin_other when two warps still
+// overlap.
+// Batches of 2^26 32-bit (2^25 64-bit) keys as units of 32768 (16384): even
+// keys 350 us (296); 1024 values, Zipf 1.1, 564 (400); keys spread over their
+// logarithm 575 (484), one far key to a unit 574 (496), 50 narrow groups 682
+// (907); all of these took 655 (835) by digits (comparisons) alone.  As units
+// of 2048: 674 (414); 850 (545), 845 (600), 849 (554), 849 (821) against 835
+// (795).
 #pragma once
 
 #include <cstdint>
@@ -113,6 +122,17 @@ __device__ __forceinline__ bool warp_inverted(const K (&v)[E], int lane)
 // By key value.
 template <typename K, int NB> struct BinMap;
 
+// The largest multiplier, or a few less, with d * mult < NB * 2^32, for d >=
+// 2^31: every thread works it out, and a 64-bit division would take a tenth
+// of a small unit's time.  The quotient lies in (NB, 2 NB]; its rounding up
+// by 2^-21 at most is taken off before the fraction is.
+template <int NB>
+__device__ __forceinline__ uint32_t bin_mult(uint32_t d)
+{
+    return __float2uint_rz(__fdividef((float)NB * 4294967296.0f, __uint2float_ru(d)) *
+                           (1.0f - 1.0f / (1 << 20)));
+}
+
 template <int NB> struct BinMap<uint32_t, NB> {
     uint32_t base, mult;
     int lz;
@@ -120,7 +140,7 @@ template <int NB> struct BinMap<uint32_t, NB> {
     {
         base = lo;
         lz = __clz((int)(hi - lo));
-        mult = (uint32_t)((((uint64_t)NB << 32) - 1) / ((uint64_t)((hi - lo) << lz) + 1));
+        mult = bin_mult<NB>((hi - lo) << lz);
     }
     __device__ uint32_t bin(uint32_t key) const { return __umulhi((key - base) << lz, mult); }
     __device__ uint32_t fine(uint32_t key) const { return ((key - base) << lz) * mult; }
@@ -136,7 +156,7 @@ template <int NB> struct BinMap<uint64_t, NB> {
         const int z = __clzll((long long)(hi - lo));
         sr = z < 32 ? 32 - z : 0;
         sl = z < 32 ? 0 : z - 32;
-        mult = (uint32_t)((((uint64_t)NB << 32) - 1) / ((uint64_t)top(hi) + 1));
+        mult = bin_mult<NB>(top(hi));
     }
     __device__ uint32_t top(uint64_t key) const { return (uint32_t)((key - base) >> sr) << sl; }
     __device__ uint32_t bin(uint64_t key) const { return __umulhi(top(key), mult); }
@@ -175,6 +195,29 @@ template <int NB> struct BinMapPairs {
     __device__ uint32_t fine(uint64_t x) const { return m.fine((uint32_t)(x >> 32)); }
 };
 
+// By the logarithm of key - kmin, as its rounded-down float's code has it:
+// keys spread over their logarithm, or crowded near kmin with others far off.
+template <typename K, int NB> struct BinMapLog {
+    K base;
+    BinMap<uint32_t, NB> m;
+    __device__ BinMapLog(K lo, K hi) : base(lo), m(0u, code(hi - lo)) {}
+    static __device__ uint32_t code(K x)  // 0, then from 1's code on
+    {
+        float f;
+        if constexpr (sizeof(K) == 4) f = __uint2float_rz(x);
+        else f = __ull2float_rz(x);
+        return x == 0 ? 0u : __float_as_uint(f) - 0x3F000000u;
+    }
+    __device__ uint32_t bin(K key) const { return m.bin(code(key - base)); }
+    __device__ uint32_t fine(K key) const { return m.fine(code(key - base)); }
+};
+template <int NB> struct BinMapLogPairs {
+    BinMapLog<uint32_t, NB> m;
+    __device__ BinMapLogPairs(uint32_t lo, uint32_t hi) : m(lo, hi) {}
+    __device__ uint32_t bin(uint64_t x) const { return m.bin((uint32_t)(x >> 32)); }
+    __device__ uint32_t fine(uint64_t x) const { return m.fine((uint32_t)(x >> 32)); }
+};
+
 // Ranges below NB: value x of the range has the rep bins [x*rep, (x+1)*rep),
 // a power of two up to 32, spread over the lanes.
 template <typename K, int NB> struct BinMapExact {
@@ -200,7 +243,6 @@ struct BinSort {
     static constexpr int NWARP = T / 32;
     static constexpr int NW = NB / 2;     // counter words
     static constexpr int IT = NW / NWARP / 128;  // 16-byte words a lane scans
-    static constexpr int SK = E / 8;      // keys per thread of bin_skewed's test
     static_assert(T % 32 == 0 && T >= 64 && T <= 1024 && E % 8 == 0, "whole warps");
     static_assert((NB & (NB - 1)) == 0 && NB <= 32768 && IT >= 1, "power-of-two bins, whole words");
     static_assert(CAP <= 32768, "counts and ranks fit 16 bits");
@@ -312,6 +354,46 @@ struct BinSort {
                 if (FULL || real(k0 + j)) sm[pidx<K>((int)r[j])] = v[k0 + j];
         }
     }
+    // One of each thread's keys is sampled: register sample_reg(), which
+    // differs between neighbouring lanes and between warps (units made of
+    // sorted runs repeat their ranks from warp to warp).
+    __device__ __forceinline__ int sample_at() const { return (lane + warp) & 7; }
+    __device__ __forceinline__ int sample_reg() const { return sample_at() * (E / 8); }
+    template <typename V>
+    __device__ __forceinline__ V pick(const V (&a)[8]) const
+    {
+        const int i = sample_at();
+        const V b = i & 1 ? a[1] : a[0], c = i & 1 ? a[3] : a[2];
+        const V d = i & 1 ? a[5] : a[4], e = i & 1 ? a[7] : a[6];
+        const V f = i & 2 ? c : b, g = i & 2 ? e : d;
+        return i & 4 ? g : f;
+    }
+    __device__ __forceinline__ K sample(const K (&v)[E]) const
+    {
+        const K a[8] = {v[0],         v[E / 8],     v[2 * E / 8], v[3 * E / 8],
+                        v[4 * E / 8], v[5 * E / 8], v[6 * E / 8], v[7 * E / 8]};
+        return pick(a);
+    }
+    // Whether the sampled keys meet in bins more often than keys of a smooth
+    // density do: each leaves its value at its bin's place in the key area (any
+    // may stay), and those that find another one there are counted (ANY: those
+    // that another thread's key replaced).  With S samples a density of rho
+    // times the even one counts about S^2 rho / (2 NB) of them; the limit is
+    // where rho is 16 (even keys: 1; a bell: 2.5; an exponential: 5), and slack
+    // times that.  The key area is overwritten; ends with a barrier.
+    template <bool ANY, typename V>
+    __device__ __forceinline__ bool crowded(uint32_t bin, V value, float slack = 1.0f) const
+    {
+        const bool r = real(sample_reg());
+        const V mark = ANY ? (V)tid : value;
+        V *at = reinterpret_cast<V *>(sm) + (bin & (uint32_t)(CAP - 1));
+        if (r) *at = mark;
+        __syncthreads();
+        const bool meets = r && *at != mark;
+        const float fill = (float)len * (1.0f / CAP);
+        constexpr float limit = T * (E >= 64 ? 0.115f : E >= 32 ? 0.213f : 0.368f);
+        return (float)__syncthreads_count(meets) > slack * limit * fill * fill + 4.0f;
+    }
     // Bins that straddle this warp's first key: merge the last 32 keys before
     // it and the first 32 from it, each ascending.
     __device__ __forceinline__ void merge_edge() const
@@ -331,18 +413,65 @@ struct BinSort {
         sm[pidx<K>(b - 32 + lane)] = l;
         sm[pidx<K>(b + lane)] = h;
     }
+    // Step 4: order the keys inside the bins, at most G <= 32 keys each.
+    __device__ __forceinline__ void order_bins(K (&v)[E], uint32_t G) const
+    {
+        if (act) {
+#pragma unroll
+            for (int k = 0; k < E; ++k) v[k] = sm[pidx<K>(tid * E + k)];
+#pragma unroll 1
+            for (uint32_t p = 0; p < G; p += 2) transpose_phases<K, E>(v, lane);
+#pragma unroll
+            for (int k = 0; k < E; ++k) sm[pidx<K>(tid * E + k)] = v[k];
+        }
+        __syncthreads();
+        merge_edge();
+        __syncthreads();
+    }
     __device__ __forceinline__ void pad() const  // the positions behind the real keys
     {
         for (int x = len + tid; x < CAP; x += T) sm[pidx<K>(x)] = KeyMax<K>::v;
     }
 };
 
-// Sort of a unit whose first bins are crowded, the largest with G keys (out
-// of line: its comparison sorts must not take registers from the usual
-// path).  The keys are in sm at their warp-blocked positions, the first bins'
-// exclusive prefix P in the counters.
+// Sort of a unit that bins do not part: by digits or comparisons, or (run > 0)
+// by merging its ascending runs of run keys.  The keys are in sm at their
+// warp-blocked positions.  (This and bin_skewed are out of line, each by
+// itself: their registers must not weigh on the usual path, nor on each other.)
+template <typename K, int T, int E, bool RUNS>
+__device__ __noinline__ void bin_other(K *sm, int len, int run)
+{
+    constexpr int CAP = T * E;
+    const int tid = (int)threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    K v[E];
+    if constexpr (RUNS) {
+        if (run >= 32 * E && run < CAP) {
+#pragma unroll
+            for (int k = 0; k < E; ++k) v[k] = sm[pidx<K>(k * T + tid)];
+            __syncthreads();
+#pragma unroll
+            for (int k = 0; k < E; ++k) {  // odd runs descending, as the merges read them
+                const int x = k * T + tid, q = x / run, o = x % run;
+                sm[pidx<K>(q & 1 ? q * run + run - 1 - o : x)] = v[k];
+            }
+            __syncthreads();
+            cta_merge_runs<K, T, E>(sm, run);
+            return;
+        }
+    }
+#pragma unroll
+    for (int k = 0; k < E; ++k) v[k] = sm[pidx<K>(wb_pos<E>(warp, lane, k))];
+    __syncthreads();
+    if constexpr (sizeof(K) == 4 && CAP == 32768) cta_radix_sort<T, E, 6>(v, sm, len);
+    else cta_sort<K, T, E>(v, sm, len);
+}
+
+// Sort of a unit whose first bins hold too many keys: each bin is cut once
+// more.  The keys are in sm at their warp-blocked positions, the first bins'
+// exclusive prefix P in the counters.  False: the unit is not sorted, its keys
+// are in sm in some order.
 template <typename K, int T, int E, bool PAIRS, typename F>
-__device__ __noinline__ void bin_skewed(K *sm, int len, const F map, uint32_t G)
+__device__ __noinline__ bool bin_skewed(K *sm, int len, const F map)
 {
     using B = BinSort<K, T, E>;
     constexpr int CAP = B::CAP, W = B::W, NWARP = B::NWARP, NW = B::NW;
@@ -360,37 +489,6 @@ __device__ __noinline__ void bin_skewed(K *sm, int len, const F map, uint32_t G)
 #pragma unroll
     for (int k = 0; k < E; ++k) v[k] = sm[pidx<K>(wb_pos<E>(warp, lane, k))];
     __syncthreads();
-    if (G > (uint32_t)len / 4u) {
-        // of an eighth of the keys, those whose bin also holds another value:
-        // one key of each bin is left in the key area (any), the others compare
-#pragma unroll
-        for (int k = 0; k < B::SK; ++k)
-            if (s.real(k)) sm[map.bin(v[k]) & (uint32_t)(CAP - 1)] = v[k];
-        __syncthreads();
-        uint32_t mixed = 0, cnt = 0;
-#pragma unroll
-        for (int k = 0; k < B::SK; ++k) {
-            if (s.real(k)) {
-                ++cnt;
-                mixed += value(sm[map.bin(v[k]) & (uint32_t)(CAP - 1)]) != value(v[k]);
-            }
-        }
-        mixed = __reduce_add_sync(0xFFFFFFFFu, mixed);
-        cnt = __reduce_add_sync(0xFFFFFFFFu, cnt);
-        if (lane == 0) {
-            s_a[warp] = mixed;
-            s_b[warp] = cnt;
-        }
-        __syncthreads();
-        mixed = __reduce_add_sync(0xFFFFFFFFu, lane < NWARP ? s_a[lane % NWARP] : 0u);
-        cnt = __reduce_add_sync(0xFFFFFFFFu, lane < NWARP ? s_b[lane % NWARP] : 0u);
-        __syncthreads();  // s_a and the key area are written again
-        if (mixed > cnt / 4u) {
-            if constexpr (sizeof(K) == 4 && CAP == 32768) cta_radix_sort<T, E, 6>(v, sm, len);
-            else cta_sort<K, T, E>(v, sm, len);
-            return;
-        }
-    }
     uint32_t *fine = reinterpret_cast<uint32_t *>(sm);  // the refined bins' counters
     const uint32_t *P = reinterpret_cast<const uint32_t *>(s.counters());
     const uint32_t fbase = smem_u32addr(fine);
@@ -446,8 +544,6 @@ __device__ __noinline__ void bin_skewed(K *sm, int len, const F map, uint32_t G)
         __syncthreads();
         s.scan(reinterpret_cast<const uint4 *>(fine), s.counters(), s_a, s_b);
     };
-    refine(std::false_type{});
-    if constexpr (PAIRS) refine(std::true_type{});
     auto place = [&](auto full) {
         constexpr int GB = 8;
 #pragma unroll
@@ -465,6 +561,21 @@ __device__ __noinline__ void bin_skewed(K *sm, int len, const F map, uint32_t G)
                 if (decltype(full)::value || s.real(k0 + j)) sm[pidx<K>((int)r[j])] = v[k0 + j];
         }
     };
+    refine(std::false_type{});
+    // keys of several scales crowd the refined bins too
+    uint32_t a[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+        const int k = j * (E / 8);
+        a[j] = (bins[k / 2] >> (16 * (k & 1))) & 0xFFFFu;
+    }
+    if (s.template crowded<false>(s.pick(a), value(s.sample(v)))) {
+#pragma unroll
+        for (int k = 0; k < E; ++k) sm[pidx<K>(wb_pos<E>(warp, lane, k))] = v[k];
+        __syncthreads();
+        return false;
+    }
+    if constexpr (PAIRS) refine(std::true_type{});
     if (s.full) place(std::true_type{});
     else if (s.act) place(std::false_type{});
     s.pad();
@@ -489,17 +600,36 @@ __device__ __noinline__ void bin_skewed(K *sm, int len, const F map, uint32_t G)
     __syncthreads();
     s.merge_edge();
     __syncthreads();
-    const int b = warp * W;
-    if (__syncthreads_or(warp > 0 && s.act &&
-                         (sm[pidx<K>(b - 33)] > sm[pidx<K>(b - 32)] ||
-                          sm[pidx<K>(b + 31)] > sm[pidx<K>(b + 32)]))) {
-        // two warps overlap by more: merge all the runs (a warp's is sorted
-        // again, and stored descending by odd warps for the merge levels)
+    const int b = warp * W;  // (false when two warps overlap by more)
+    return !__syncthreads_or(warp > 0 && s.act &&
+                             (sm[pidx<K>(b - 33)] > sm[pidx<K>(b - 32)] ||
+                              sm[pidx<K>(b + 31)] > sm[pidx<K>(b + 32)]));
+}
+
+// The sort by the bins of another map, for units that crowd in the first one:
+// the keys in sm at their warp-blocked positions, the counters zero.
+template <typename K, int T, int E, bool PAIRS, typename F>
+__device__ __noinline__ void bin_again(K *sm, int len, const F map)
+{
+    using B = BinSort<K, T, E>;
+    __shared__ uint32_t s_a[B::NWARP], s_b[B::NWARP];
+    const B s(sm, len);
+    K v[E];
 #pragma unroll
-        for (int k = 0; k < E; ++k) v[k] = sm[pidx<K>(tid * E + k)];
-        __syncthreads();
-        cta_sort<K, T, E>(v, sm, len);
+    for (int k = 0; k < E; ++k) v[k] = sm[pidx<K>(wb_pos<E>(s.warp, s.lane, k))];
+    if (s.full) s.template count<true>(v, map);
+    else if (s.act) s.template count<false>(v, map);
+    __syncthreads();
+    const uint32_t G = s.scan(s.counters(), s.counters(), s_a, s_b);
+    if (G > kBinPhases) {
+        if (!bin_skewed<K, T, E, PAIRS>(sm, len, map)) bin_other<K, T, E, false>(sm, len, 0);
+        return;
     }
+    if (s.full) s.template scatter<true>(v, map);
+    else if (s.act) s.template scatter<false>(v, map);
+    s.pad();
+    __syncthreads();
+    s.order_bins(v, G);
 }
 
 // Sort the CTA's T*E keys v ascending into sm (padded layout pidx, then the
@@ -508,9 +638,11 @@ __device__ __noinline__ void bin_skewed(K *sm, int len, const F map, uint32_t G)
 // key.  On return sm[pidx(x)] is the x-th smallest key, padding after the
 // len real ones, as cta_sort leaves it.  is_f32: 32-bit keys are codes of
 // floats.  PAIRS: v holds key << 32 | a position that grows with the item's
-// place in the unit.  Ends with __syncthreads().
-template <typename K, int T, int E, bool PAIRS = false>
-__device__ __forceinline__ void cta_bin_sort(K (&v)[E], K *sm, int len, bool is_f32)
+// place in the unit.  RUNS: the keys are ascending runs of run keys.  MANY:
+// units by the thousand, where what a unit costs counts, not how long it takes.
+// Ends with __syncthreads().
+template <typename K, int T, int E, bool PAIRS = false, bool RUNS = false, bool MANY = false>
+__device__ __forceinline__ void cta_bin_sort(K (&v)[E], K *sm, int len, bool is_f32, int run = 0)
 {
     using B = BinSort<K, T, E>;
     constexpr int NWARP = B::NWARP, NB = B::NB;
@@ -539,22 +671,23 @@ __device__ __forceinline__ void cta_bin_sort(K (&v)[E], K *sm, int len, bool is_
                 hi = kmax<V>(hi, value(v[k]));
             }
     }
+    // (64-bit words by halves)
     auto warp_lo = [&](V x) {
         if constexpr (sizeof(V) == 4) {
             return __reduce_min_sync(0xFFFFFFFFu, x);
         } else {
-#pragma unroll
-            for (int d = 16; d >= 1; d >>= 1) x = kmin<V>(x, __shfl_xor_sync(0xFFFFFFFFu, x, d));
-            return x;
+            const uint32_t h = (uint32_t)(x >> 32), m = __reduce_min_sync(0xFFFFFFFFu, h);
+            const uint32_t l = __reduce_min_sync(0xFFFFFFFFu, h == m ? (uint32_t)x : 0xFFFFFFFFu);
+            return ((V)m << 32) | l;
         }
     };
     auto warp_hi = [&](V x) {
         if constexpr (sizeof(V) == 4) {
             return __reduce_max_sync(0xFFFFFFFFu, x);
         } else {
-#pragma unroll
-            for (int d = 16; d >= 1; d >>= 1) x = kmax<V>(x, __shfl_xor_sync(0xFFFFFFFFu, x, d));
-            return x;
+            const uint32_t h = (uint32_t)(x >> 32), m = __reduce_max_sync(0xFFFFFFFFu, h);
+            const uint32_t l = __reduce_max_sync(0xFFFFFFFFu, h == m ? (uint32_t)x : 0u);
+            return ((V)m << 32) | l;
         }
     };
     lo = warp_lo(lo);
@@ -575,6 +708,20 @@ __device__ __forceinline__ void cta_bin_sort(K (&v)[E], K *sm, int len, bool is_
         __syncthreads();
         return;
     }
+    // Keys that crowd into few bins take another sort at once, by the sample.
+    // (ANY: small units of 32-bit keys take it for repeated keys too: 6000
+    // keys, 1024 values, 14.5 us by comparisons, 21 by bins cut once more; as
+    // many 8192-key units 593 us by comparisons, 524 by bins)
+    constexpr bool ANY = !PAIRS && sizeof(K) == 4 && B::CAP <= (MANY ? 2048 : 8192);
+    const K sx = s.sample(v);
+    auto crowds = [&](const auto &map, float slack) {
+        return s.template crowded<ANY>(map.bin(sx), value(sx), slack);
+    };
+    auto spill = [&]() {  // the keys to their warp-blocked positions
+#pragma unroll
+        for (int k = 0; k < E; ++k) sm[pidx<K>(wb_pos<E>(warp, lane, k))] = v[k];
+        __syncthreads();
+    };
     uint32_t G = 0;
     // steps 1-3: true when step 4 is still to do
     auto distribute = [&](const auto &map, auto fill) -> bool {
@@ -584,10 +731,8 @@ __device__ __forceinline__ void cta_bin_sort(K (&v)[E], K *sm, int len, bool is_
         G = s.scan(cnt, cnt, s_a, s_b);
         if constexpr (decltype(fill)::value) {
             if (G > kBinPhases) {
-#pragma unroll
-                for (int k = 0; k < E; ++k) sm[pidx<K>(wb_pos<E>(warp, lane, k))] = v[k];
-                __syncthreads();
-                bin_skewed<K, T, E, PAIRS>(sm, len, map, G);
+                spill();
+                if (!bin_skewed<K, T, E, PAIRS>(sm, len, map)) bin_other<K, T, E, false>(sm, len, 0);
                 return false;
             }
         }
@@ -597,35 +742,41 @@ __device__ __forceinline__ void cta_bin_sort(K (&v)[E], K *sm, int len, bool is_
         __syncthreads();
         return decltype(fill)::value;
     };
+    auto by_bins = [&](const auto &map, const auto &other) -> bool {
+        if (!crowds(map, 1.0f)) return distribute(map, std::true_type{});
+        // (by the other map it is enough that the bins can be cut once more)
+        const bool again = !ANY && !(RUNS && run) && !is_f32 && !crowds(other, 1.35f);
+        if (again) {
+            spill();
+            bin_again<K, T, E, PAIRS>(sm, len, other);
+        } else if constexpr (E <= 16 && T <= 512 && (ANY || T <= 256)) {
+            cta_sort<K, T, E>(v, sm, len);  // (small: a call would cost a tenth of the sort)
+        } else {
+            spill();
+            bin_other<K, T, E, RUNS>(sm, len, run);
+        }
+        return false;
+    };
     bool more;
     if constexpr (PAIRS) {
-        more = distribute(BinMapPairs<NB>(lo, hi), std::true_type{});
+        more = by_bins(BinMapPairs<NB>(lo, hi), BinMapLogPairs<NB>(lo, hi));
     } else {
         if (hi - lo < (K)NB) {
             distribute(BinMapExact<K, NB>(lo, hi, lane), std::false_type{});
             return;
         }
         if constexpr (sizeof(K) == 4) {
+            // floats: equal steps of the value, or of the code (about its
+            // logarithm) where those crowd
             const BinMapF32<NB> fmap(lo, hi);
-            if (is_f32 && fmap.ok) more = distribute(fmap, std::true_type{});
-            else more = distribute(BinMap<K, NB>(lo, hi), std::true_type{});
+            if (is_f32 && fmap.ok && !crowds(fmap, 1.0f)) more = distribute(fmap, std::true_type{});
+            else more = by_bins(BinMap<uint32_t, NB>(lo, hi), BinMapLog<uint32_t, NB>(lo, hi));
         } else {
-            more = distribute(BinMap<K, NB>(lo, hi), std::true_type{});
+            more = by_bins(BinMap<K, NB>(lo, hi), BinMapLog<K, NB>(lo, hi));
         }
     }
     if (!more) return;
-    // 4. order the keys inside the bins
-    if (s.act) {
-#pragma unroll
-        for (int k = 0; k < E; ++k) v[k] = sm[pidx<K>(s.tid * E + k)];
-#pragma unroll 1
-        for (uint32_t p = 0; p < G; p += 2) transpose_phases<K, E>(v, lane);
-#pragma unroll
-        for (int k = 0; k < E; ++k) sm[pidx<K>(s.tid * E + k)] = v[k];
-    }
-    __syncthreads();
-    s.merge_edge();
-    __syncthreads();
+    s.order_bins(v, G);
 }
 
 }  // namespace bsort

@@ -431,6 +431,29 @@ __device__ __forceinline__ void cta_sort(K (&v)[E], K *sm, int len = T * E)
     }
 }
 
+// The same sort when the tile already consists of sorted runs of length R
+// (R a power of two, 32*E <= R < T*E) stored in sm with run q ascending if q
+// is even and descending if q is odd: only the block levels from R run.
+template <typename K, int T, int E>
+__device__ __forceinline__ void cta_merge_runs(K *sm, int R)
+{
+    const int tid = threadIdx.x;
+    K v[E];
+#pragma unroll 1
+    for (int L = R; L < T * E; L <<= 1) {
+        const int dg = tid * E;
+        const int a0 = dg & ~(2 * L - 1);
+        const int d = dg - a0;
+        const int bend = a0 + 2 * L;
+        const int i = corank_bitonic<K>(sm, a0, bend, L, d);
+        merge_bitonic_pair<K, E>(sm, a0 + i, bend - 1 - (d - i), v);
+        __syncthreads();
+        const bool desc = ((a0 / (2 * L)) & 1) != 0;
+        store_run<K, E>(sm, a0, 2 * L, d, desc, v);
+        __syncthreads();
+    }
+}
+
 // ---------------------------------------------------------------- cluster merges
 // C CTAs of a thread-block cluster each hold a sorted chunk of `chunk` items
 // (ascending, padded layout).  log2(C) rounds of pairwise merges through

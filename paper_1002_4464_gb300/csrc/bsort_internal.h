@@ -124,11 +124,12 @@ constexpr int kMaxBucketsTiers = 32768;  // b of a two-tier Step 9 (a unit per b
 // Step 4 (chunks): sort the n_rec records of src in chunks of kRecordChunk
 // into dst (which holds n_pad = chunks * kRecordChunk records, the tail
 // filled with all-ones).  Records n_real .. n_rec - 1 are the samples of the
-// padding, in order and not below any other.  If the whole array is one chunk
+// padding, in order and not below any other; runs of s records (one sublist's)
+// are sorted already.  If the whole array is one chunk
 // and spl != nullptr, also writes the b splitters (Step 5).
 cudaError_t launch_records_chunk_sort(const uint64_t *src, uint64_t *dst, uint32_t n_rec,
-                                      uint32_t n_real, uint32_t n_pad, uint64_t *spl, uint32_t b,
-                                      cudaStream_t st);
+                                      uint32_t n_real, uint32_t n_pad, uint64_t *spl, uint32_t s,
+                                      uint32_t b, cudaStream_t st);
 // Samples of real items among the m*s: those of the m - 1 full sublists, and
 // the last one's below its real items' count.
 __host__ __device__ inline uint32_t real_samples(uint64_t n, uint32_t m, uint32_t t, uint32_t s)

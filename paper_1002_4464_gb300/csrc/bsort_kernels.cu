@@ -37,7 +37,7 @@ namespace bsort {
 template <int T, int E>
 __global__ void __launch_bounds__(T, 1)
 k_records_sort(const uint64_t *__restrict__ src, uint64_t *__restrict__ dst, uint32_t n_rec,
-               uint32_t n_real, uint64_t *__restrict__ spl, uint32_t b)
+               uint32_t n_real, uint64_t *__restrict__ spl, uint32_t s, uint32_t b)
 {
     grid_dep_wait();
     constexpr int CAP = T * E;
@@ -48,7 +48,8 @@ k_records_sort(const uint64_t *__restrict__ src, uint64_t *__restrict__ dst, uin
     const int len = n_real <= base ? 0 : (int)min((uint64_t)CAP, n_real - base);
     uint64_t v[E];
     load_keys<uint64_t, T, E>(v, src + base, len, false);
-    cta_bin_sort<uint64_t, T, E, true>(v, sm, len, false);  // (q grows with the index)
+    // (q grows with the index; a sublist's s records are an ascending run)
+    cta_bin_sort<uint64_t, T, E, true, true>(v, sm, len, false, (int)s);
 #pragma unroll 4
     for (int k = 0; k < E; ++k) {
         const int x = k * T + tid;
@@ -1481,12 +1482,12 @@ cudaError_t init_misc_kernels()
 }
 
 cudaError_t launch_records_chunk_sort(const uint64_t *src, uint64_t *dst, uint32_t n_rec,
-                                      uint32_t n_real, uint32_t n_pad, uint64_t *spl, uint32_t b,
-                                      cudaStream_t st)
+                                      uint32_t n_real, uint32_t n_pad, uint64_t *spl, uint32_t s,
+                                      uint32_t b, cudaStream_t st)
 {
     const uint32_t chunks = n_pad / kRecordChunk;
     launch_dep(k_records_sort<1024, 16>, chunks, 1024, BinSmem<uint64_t, 1024, 16>::kBytes, st,
-               src, dst, n_rec, n_real, chunks == 1 ? spl : nullptr, b);
+               src, dst, n_rec, n_real, chunks == 1 ? spl : nullptr, s, b);
     return cudaGetLastError();
 }
 

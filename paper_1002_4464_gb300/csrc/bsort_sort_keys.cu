@@ -6,15 +6,18 @@
 namespace bsort {
 
 // chunk shapes, sorted by bins (cta_bin_sort): 2048 = 128x16, 4096 = 256x16,
-// 8192 = 256x32, 16384 = 512x32, and 32768 = 512x64 when `bins` is set;
-// sorted by comparisons: 32768 = 1024x32, and clusters of 2, 4, 8 CTAs of it.
+// 8192 = 512x16 (one unit of 6000 keys 8.4 us against 10.4 with 256x32, 14.5
+// against 18.7 when they crowd; the batch kernel keeps 256x32, faster when
+// units are many: 61 us against 70 for 2000 of them), 16384 = 512x32, and
+// 32768 = 512x64 when `bins` is set; sorted by comparisons: 32768 = 1024x32,
+// and clusters of 2, 4, 8 CTAs of it.
 cudaError_t init_sort_keys_kernels()
 {
     cudaError_t e;
 #define I(T_, E_, C_, B_)                                            \
     e = init_sort_pair_of_kernels<T_, E_, false, C_, B_>();      \
     if (e != cudaSuccess) return e
-    I(128, 16, 1, true); I(256, 16, 1, true); I(256, 32, 1, true); I(512, 32, 1, true);
+    I(128, 16, 1, true); I(256, 16, 1, true); I(512, 16, 1, true); I(512, 32, 1, true);
     I(1024, 32, 1, false); I(1024, 32, 2, false); I(1024, 32, 4, false); I(1024, 32, 8, false);
 #undef I
     return init_sort_keys_bins_kernels();
@@ -35,7 +38,7 @@ cudaError_t launch_sublist_sort_keys(int chunk, int ctas, const void *keys_in, u
         switch (chunk) {
         case 2048: L(128, 16, 1, true);
         case 4096: L(256, 16, 1, true);
-        case 8192: L(256, 32, 1, true);
+        case 8192: L(512, 16, 1, true);
         case 16384: L(512, 32, 1, true);
         case 32768: L(1024, 32, 1, false);
         }
@@ -65,7 +68,7 @@ cudaError_t launch_bucket_sort_keys(int chunk, int ctas, const void *src_k, cons
         switch (chunk) {
         case 2048: L(128, 16, 1, true);
         case 4096: L(256, 16, 1, true);
-        case 8192: L(256, 32, 1, true);
+        case 8192: L(512, 16, 1, true);
         case 16384: L(512, 32, 1, true);
         case 32768: L(1024, 32, 1, false);
         }
@@ -96,7 +99,7 @@ cudaError_t launch_bucket_sort_keys_range(int chunk, int ctas, const void *src_k
         switch (chunk) {
         case 2048: L(128, 16, 1, true);
         case 4096: L(256, 16, 1, true);
-        case 8192: L(256, 32, 1, true);
+        case 8192: L(512, 16, 1, true);
         case 16384: L(512, 32, 1, true);
         case 32768: L(1024, 32, 1, false);
         }
