@@ -177,14 +177,21 @@ template <int NB> struct BinMapF32 {
         scale = 8388600.0f / d;
         ok = d > 0.0f && d < 3.0e38f && scale > 0.0f && scale < 3.0e38f;  // false with NaN, inf
     }
-    __device__ uint32_t place(uint32_t key) const  // 2^23 + place, as float bits
-    {
-        return __float_as_uint(
-            fmaf(__uint_as_float(f32_decode(key)) - lo, scale, 8388608.0f));
-    }
+    __device__ float diff(uint32_t key) const { return __uint_as_float(f32_decode(key)) - lo; }
+    __device__ float place(uint32_t key) const { return fmaf(diff(key), scale, 8388608.0f); }
     static constexpr int kShift = 23 - __builtin_ctz(NB);
-    __device__ uint32_t bin(uint32_t key) const { return (place(key) >> kShift) & (uint32_t)(NB - 1); }
-    __device__ uint32_t fine(uint32_t key) const { return place(key) << (32 - kShift); }
+    __device__ uint32_t bin(uint32_t key) const
+    {
+        return (__float_as_uint(place(key)) >> kShift) & (uint32_t)(NB - 1);
+    }
+    // (the place's low bits, then what its rounding left: exact up to the
+    // difference's own rounding, so it grows with the key at one place)
+    __device__ uint32_t fine(uint32_t key) const
+    {
+        const float p = place(key), rest = fmaf(diff(key), scale, 8388608.0f - p) + 0.5f;
+        return (__float_as_uint(p) << (32 - kShift)) +
+               (uint32_t)(rest * (float)((1u << (32 - kShift)) - 256u));
+    }
 };
 
 // Pairs (key << 32 | position) by key.
