@@ -120,8 +120,8 @@ typedef enum {
 #define BSORT_FLAG_PLAN_MODEL 0x20u /* plan every sort with the analytic
                                       cost model, also where a measured
                                       (t, s) is tabled for n's size class
-                                      (keys-only 32-bit sorts); kept to
-                                      compare the two */
+                                      (keys-only sorts and pairs of 32-bit
+                                      keys); kept to compare the two */
 #define BSORT_FLAG_TEST_TWO_LEVEL 0x40u /* test of the two-level plan:
                                       keys-only 32-bit sorts of more than
                                       65536 keys take it at any size, with
@@ -205,21 +205,19 @@ typedef struct {
     uint64_t n;               /* keys in all segments */
     uint32_t num_segs;
     uint32_t direct_segs;     /* up to batch_direct_max keys: sorted whole by
-                                 one CTA or cluster (64-bit keys, with
-                                 batch_direct_max 0 and many of them: those
-                                 above one CTA's unit with the sampled
-                                 segments, not counted there) */
+                                 one CTA or cluster (or joined, see
+                                 bsort_sort_batch: not counted there) */
     uint32_t sampled_segs;    /* sorted by segment-aware Algorithm 1 */
     uint32_t large_segs;      /* above 524288 32-bit or 1048576 64-bit keys:
-                                 32-bit ones up to 2^21 keys sorted with the
-                                 sampled segments (not counted in sublists
-                                 and buckets), the others one plain sort
-                                 each */
+                                 one plain sort each, or joined (not counted
+                                 in sublists and buckets) */
     uint32_t sublists;        /* sublists of the sampled segments */
     uint32_t buckets;         /* buckets of the sampled segments */
     uint32_t num_kernels;     /* kernel launches per call */
     uint32_t pad_;
-    uint64_t workspace_bytes; /* device workspace the batch needs */
+    uint64_t workspace_bytes; /* device workspace the batch takes (of a handle
+                                 whose workspace is fixed: of the plan that
+                                 fits it) */
 } bsort_batch_info;
 
 /* Intermediates of the last call (for parity checks), see bsort_get_intermediate. */
@@ -269,16 +267,22 @@ bsort_status bsort_sort_pairs(bsort_t h, bsort_key_type kt, const void *d_keys_i
  * HOST memory, num_segs + 1 nondecreasing values, the last below 2^32 -
  * 2^16; keys outside every segment are left untouched.  Segments up to
  * batch_direct_max keys are sorted whole by one CTA or thread-block cluster
- * (as Step 9 sorts a bucket; where batch_direct_max is left to the library,
- * 64-bit segments above one CTA's unit join the larger ones when they hold
- * 2^22 keys in all); larger ones up to 524288 keys by Algorithm 1
+ * (as Step 9 sorts a bucket); larger ones up to 524288 keys by Algorithm 1
  * (Section 4) with segment-aware sublists (32768 keys), s = 1024 samples
  * per sublist and per-segment splitters, all segments together in one
- * sequence of launches (from 524289 to 2^21 keys with s = 512 or 256
- * samples per sublist); larger ones by one plain sort each, and so are those
- * above 524288 keys when the handle's workspace is a fixed one that holds
- * the batch only that way.  The segment
+ * sequence of launches; larger ones by one plain sort each.  The segment
  * table is copied to the device from pinned staging owned by the handle.
+ * Where it is faster, segments of the other classes join that sequence:
+ * 32-bit ones from 524289 to 2^21 keys (s = 512 or 256 samples per sublist),
+ * unless one is the batch's only segment above batch_direct_max; and, with
+ * batch_direct_max left to the library, 64-bit ones above 65536 keys (32768
+ * beside sampled segments) that hold 2^22 keys in all.  Joined segments need
+ * a little more than twice their bytes as workspace; beyond 4 GiB the batch
+ * is sorted in parts, one after the other.  They are not joined, but sorted
+ * as the other segments of their class, under BSORT_FLAG_LOW_MEMORY, when a
+ * fixed workspace (or one that cannot grow because the stream is being
+ * captured) holds the batch only that way, and when the device has no room
+ * for more (the handle does not ask for as much again).
  * kt: BSORT_U32, BSORT_F32 or BSORT_U64 (64-bit keys: segments up to
  * 262144 keys, or batch_direct_max when given, sorted whole — above 131072
  * by a 16-CTA cluster, where the device schedules one, else the limit is

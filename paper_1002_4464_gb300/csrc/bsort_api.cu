@@ -48,16 +48,26 @@ constexpr uint32_t kBatchSamples = 1024;
 // Larger 32-bit segments, up to 2^21 keys, join the sampled ones with fewer
 // samples per sublist (512 up to 32 sublists, 256 up to 64: m*s stays within
 // kRecordChunk and the bound within a unit): one launch sequence for all of
-// them instead of one plain sort each, whose ~94 us at 2^20 keys are mostly
-// launches (339 such segments among 4000: 37.7 -> 5.9 ms per batch).
+// them instead of one plain sort each, whose time at 2^20 keys is mostly
+// launches (339 such segments among 4000: 37.7 -> 5.9 ms per batch).  One by
+// itself is a plain sort: 2^20 keys 63 us, joined 90; two are 125 and 87.
 constexpr uint32_t kBatchJoinMax = 1u << 21;
-// 64-bit direct segments above one CTA's unit (clusters) join the sampled
-// ones too when they hold at least this many keys in all and batch_direct_max
-// is not given: the sampled route sorts 50 Gkeys/s, the clusters, whose merge
-// rounds go through distributed shared memory, 23, but its steps take about
-// 60 us however few the keys.  (32-bit keys: 5.74 ms joined, 5.80 not, for
-// 4000 arrays: left to the clusters.)
+// 64-bit direct segments above 65536 keys (8- and 16-CTA clusters) join the
+// sampled ones too when they hold at least this many keys in all and
+// batch_direct_max is not given: their merge rounds through distributed
+// shared memory leave most of the SMs idle (2^24 keys as 80000-key segments
+// 700 us, joined 358; groups that crowd 1137 and 1031), but the sampled
+// route's steps take 100 us however few the keys.  Clusters of 2 and 4 CTAs
+// are the faster way (32768: 210 us against 373; 65536: 328 against 360, Zipf
+// 378 against 513); with sampled segments in the batch those of 4 join all the
+// same (800 arrays of 2^10 to 2^20 keys 2.08 ms, else 2.12).  (32-bit keys: 5.74 ms joined, 5.80 not, for 4000
+// arrays: left to the clusters.)
 constexpr uint64_t kBatchJoinDirectU64 = 1ull << 22;
+// Joined segments take twice their bytes and more of workspace (tiles and
+// relocated keys), where plain sorts reuse one sort's and clusters take none:
+// a batch is cut into parts whose joined segments need at most this much each
+// (about 2^29 32-bit keys), sorted one after the other in one workspace.
+constexpr uint64_t kBatchJoinBytes = 4ull << 30;
 constexpr uint32_t kBatchUnit = 32768;  // Step-9 unit of sampled segments
 // 64-bit keys: sublists of kSegTileU64 keys, s = 256 samples per sublist up
 // to 32 sublists and 128 above (m*s <= kSegRecordsU64), Step-9 units of
@@ -107,6 +117,7 @@ struct bsort_ctx {
     uint64_t ws_bytes = 0;
     bool ws_owned = false;
     bool ws_fixed = false;  // caller workspace or fixed budget: never grow
+    uint64_t ws_denied = ~0ull;  // smallest size that the device had no room for
     bool kernels_ready = false;
     Plan last{};
     bool have_last = false;
@@ -1539,23 +1550,55 @@ bsort_status spans_from_offsets(bsort_t h, const uint64_t *segoff, uint32_t nseg
     return BSORT_OK;
 }
 
-// join: segments above the sampled size up to kBatchJoinMax keys join the
-// sampled ones (32-bit keys), else each of them is a plain sort; and so do
-// 64-bit direct segments above one CTA's unit when there are enough of them,
-// else a cluster sorts each.  (The counts of *info go by the size classes.)
-// BSORT_OK with B->fits unset when the joined segments' padded positions
-// exceed 32 bits (the caller plans again without).
+// Sizes that class a batch's segments.
+struct BatchSizes {
+    uint64_t dmax;  // largest segment sorted whole
+    uint64_t smax;  // largest one sampled by its own right
+    uint64_t tile, unit;  // sublist and Step-9 unit of sampled segments
+};
+BatchSizes batch_sizes(const bsort_t h, bool wide)
+{
+    if (wide)
+        return {wide_direct_max(h), kBatchSampledMaxU64, (uint64_t)kSegTileU64, kBatchUnitU64};
+    const uint64_t largest =
+        (uint64_t)kDirectShapes[kNumDirect - 1][0] * kDirectShapes[kNumDirect - 1][1];
+    return {h->direct_max < largest ? h->direct_max : largest, kBatchSampledMax,
+            (uint64_t)kSegTile, kBatchUnit};
+}
+
+// The segments of other classes that join the sampled ones: those of
+// `from` < n <= `to` keys (none when to is 0).
+struct JoinRule {
+    uint64_t from = 0, to = 0;
+    bool takes(uint64_t n) const { return n > from && n <= to; }
+};
+JoinRule join_rule(const bsort_t h, bool wide, const SegSpan *spans, uint32_t nsegs)
+{
+    JoinRule j;
+    const BatchSizes z = batch_sizes(h, wide);
+    if (h->flags & BSORT_FLAG_LOW_MEMORY) return j;
+    if (wide) {
+        uint64_t keys = 0;
+        for (uint32_t q = 0; q < nsegs; ++q)
+            if (spans[q].n > z.unit && spans[q].n <= z.dmax) keys += spans[q].n;
+        if (!h->direct_max_set && keys >= kBatchJoinDirectU64) j = {z.unit, z.dmax};
+    } else {
+        j = {z.smax, kBatchJoinMax};
+    }
+    return j;
+}
+
+// join: the segments that take the sampled route beside those of that size
+// class; the others of their classes are a plain sort or a cluster's unit
+// each.  (The counts of *info go by the size classes.)  BSORT_OK with B->fits
+// unset when the joined segments' padded positions exceed 32 bits (the caller
+// plans again without).
 bsort_status make_batch_plan_as(bsort_t h, bsort_key_type kt, const SegSpan *spans,
-                                uint32_t nsegs, bool join, BatchPlan *B)
+                                uint32_t nsegs, const JoinRule &join, BatchPlan *B)
 {
     *B = BatchPlan();
-    if (kt != BSORT_U32 && kt != BSORT_F32 && kt != BSORT_U64)
-        return fail(h, BSORT_EINVAL, "unknown key type %d", (int)kt);
     B->wide = kt == BSORT_U64;
     const int(*shapes)[2] = B->wide ? kDirectShapesWide : kDirectShapes;
-    const int nshapes = B->wide ? wide_direct_shapes() : kNumDirect;
-    const uint64_t largest = (uint64_t)shapes[nshapes - 1][0] * shapes[nshapes - 1][1];
-    if (nsegs && !spans) return fail(h, BSORT_EINVAL, "null segment list");
     bsort_batch_info &I = B->info;
     memset(&I, 0, sizeof(I));
     I.num_segs = nsegs;
@@ -1567,30 +1610,20 @@ bsort_status make_batch_plan_as(bsort_t h, bsort_key_type kt, const SegSpan *spa
         if (spans[q].begin + spans[q].n >= kMaxN)
             return fail(h, BSORT_EUNSUPPORTED, "segment end %llu exceeds 2^32 - 2^16",
                         (unsigned long long)(spans[q].begin + spans[q].n));
-    const uint64_t dmax =
-        B->wide ? wide_direct_max(h) : (h->direct_max < largest ? h->direct_max : largest);
-    const uint64_t tile = B->wide ? (uint64_t)kSegTileU64 : (uint64_t)kSegTile;
-    const uint64_t unit = B->wide ? (uint64_t)kBatchUnitU64 : (uint64_t)kBatchUnit;
-    const uint64_t smax = B->wide ? kBatchSampledMaxU64 : kBatchSampledMax;
-    uint64_t rmax = dmax;  // largest segment that takes the direct route
-    if (join && B->wide && !h->direct_max_set) {
-        uint64_t keys = 0;
-        for (uint32_t q = 0; q < nsegs; ++q)
-            if (spans[q].n > unit && spans[q].n <= dmax) keys += spans[q].n;
-        if (keys >= kBatchJoinDirectU64) rmax = unit;
-    }
+    const BatchSizes z = batch_sizes(h, B->wide);
+    const uint64_t dmax = z.dmax, smax = z.smax, tile = z.tile, unit = z.unit;
     uint64_t g = 0;  // sublists so far
     for (uint32_t q = 0; q < nsegs; ++q) {
         const uint64_t a = spans[q].begin, n = spans[q].n;
         I.n += n;
         if (n <= 1) continue;  // nothing to order (a copy when out != in)
-        if (n <= rmax) {
+        if (n <= dmax && !join.takes(n)) {
             int c = 0;
             while ((uint64_t)shapes[c][0] * shapes[c][1] < n) ++c;
             B->direct[c].push_back((uint32_t)a);
             B->direct[c].push_back((uint32_t)(a + n));
             ++I.direct_segs;
-        } else if (n <= smax || (join && !B->wide && n <= kBatchJoinMax)) {
+        } else if (n <= smax || join.takes(n)) {
             SegInfo sg = {};
             sg.g0 = (uint32_t)g;
             sg.m = (uint32_t)((n + tile - 1) / tile);
@@ -1634,7 +1667,7 @@ bsort_status make_batch_plan_as(bsort_t h, bsort_key_type kt, const SegSpan *spa
         }
     }
     if (g * tile >= kMaxN) {
-        if (join) return BSORT_OK;
+        if (join.to) return BSORT_OK;
         return fail(h, BSORT_EUNSUPPORTED, "padded sampled segments exceed 2^32");
     }
     B->fits = true;
@@ -1692,45 +1725,123 @@ bsort_status make_batch_plan_as(bsort_t h, bsort_key_type kt, const SegSpan *spa
     return BSORT_OK;
 }
 
-// The plan of a batch: with segments of other classes joined to the sampled
-// ones, unless their padded positions exceed 32 bits or the workspace is a
-// fixed one that only holds the plan without.
-bsort_status make_batch_plan(bsort_t h, bsort_key_type kt, const SegSpan *spans,
-                             uint32_t nsegs, BatchPlan *B)
+// A batch's plan: its parts, one after the other in one workspace (more than
+// one only when joined segments need more than kBatchJoinBytes in all).
+struct BatchParts {
+    std::vector<BatchPlan> part;
+    std::vector<uint32_t> first;  // part i: segments first[i] .. first[i+1] - 1
+    bsort_batch_info info;        // of the whole batch
+    uint64_t total = 0;           // workspace bytes
+    uint64_t words = 0;           // descriptor words of all parts
+    bool joined = false;
+};
+
+bsort_status make_batch_parts(bsort_t h, bsort_key_type kt, const SegSpan *spans, uint32_t nsegs,
+                              const JoinRule &join, BatchParts *B, bool *fits)
 {
-    bsort_status rs = make_batch_plan_as(h, kt, spans, nsegs, true, B);
-    if (rs != BSORT_OK) return rs;
-    if (B->fits && (!B->joined || !h->ws_fixed || B->total <= h->ws_bytes)) return BSORT_OK;
-    return make_batch_plan_as(h, kt, spans, nsegs, false, B);
+    *B = BatchParts();
+    *fits = true;
+    const BatchSizes z = batch_sizes(h, kt == BSORT_U64);
+    // cut before a joined segment that would pass the limit (tiles and
+    // relocated keys; a hundredth more for records and runs)
+    B->first.push_back(0);
+    uint64_t bytes = 0;
+    for (uint32_t q = 0; q < nsegs; ++q) {
+        if (!join.takes(spans[q].n)) continue;
+        const uint64_t add =
+            (spans[q].n + z.tile - 1) / z.tile * z.tile * 2 * (kt == BSORT_U64 ? 8 : 4);
+        if (bytes && bytes + add > kBatchJoinBytes) {
+            B->first.push_back(q);
+            bytes = 0;
+        }
+        bytes += add;
+    }
+    B->part.resize(B->first.size());
+    B->first.push_back(nsegs);
+    memset(&B->info, 0, sizeof(B->info));
+    B->info.num_segs = nsegs;
+    for (size_t i = 0; i < B->part.size(); ++i) {
+        BatchPlan &P = B->part[i];
+        bsort_status rs = make_batch_plan_as(h, kt, spans + B->first[i],
+                                             B->first[i + 1] - B->first[i], join, &P);
+        if (rs != BSORT_OK) return rs;
+        *fits &= P.fits;
+        B->joined |= P.joined;
+        B->total = std::max(B->total, P.total);
+        B->words += P.d_words;
+        B->info.n += P.info.n;
+        B->info.direct_segs += P.info.direct_segs;
+        B->info.sampled_segs += P.info.sampled_segs;
+        B->info.large_segs += P.info.large_segs;
+        B->info.sublists += P.info.sublists;
+        B->info.buckets += P.info.buckets;
+        B->info.num_kernels += P.info.num_kernels;
+    }
+    B->info.workspace_bytes = B->total;
+    return BSORT_OK;
 }
 
-// stage: when not null, pinned host memory of at least the plan's
-// descriptor bytes that the caller keeps unchanged for as long as the
-// upload may run again (a captured graph replays it); the handle's shared
-// staging is used otherwise.
-bsort_status run_batch(bsort_t h, bsort_key_type kt, const void *kin, void *kout,
-                       const SegSpan *spans, uint32_t nsegs, cudaStream_t st,
-                       void *stage = nullptr)
+// The plan of a batch: with segments of other classes joined to the sampled
+// ones, unless their padded positions exceed 32 bits or their workspace
+// exceeds `room`.
+bsort_status make_batch_plan(bsort_t h, bsort_key_type kt, const SegSpan *spans, uint32_t nsegs,
+                             uint64_t room, BatchParts *B)
 {
-    bsort_status rs = prepare(h);
-    if (rs != BSORT_OK) return rs;
-    BatchPlan B;
-    rs = make_batch_plan(h, kt, spans, nsegs, &B);
-    if (rs != BSORT_OK) return rs;
-    if (B.info.n == 0) return BSORT_OK;
-    rs = ensure_workspace(h, B.total);
-    if (rs != BSORT_OK) return rs;
+    if (kt != BSORT_U32 && kt != BSORT_F32 && kt != BSORT_U64)
+        return fail(h, BSORT_EINVAL, "unknown key type %d", (int)kt);
+    if (nsegs && !spans) return fail(h, BSORT_EINVAL, "null segment list");
+    bool fits = true;
+    const JoinRule join = join_rule(h, kt == BSORT_U64, spans, nsegs);
+    bsort_status rs = make_batch_parts(h, kt, spans, nsegs, join, B, &fits);
+    if (rs != BSORT_OK || (fits && (!B->joined || B->total <= room))) return rs;
+    return make_batch_parts(h, kt, spans, nsegs, JoinRule(), B, &fits);
+}
+
+// The workspace that a plan may take: what a fixed one has, or anything.
+uint64_t batch_room(const bsort_t h) { return h->ws_fixed ? h->ws_bytes : ~0ull; }
+
+// Plan a batch and have its workspace: the plan without joined segments where
+// theirs cannot be had (the device's memory is short, which is not tried
+// again, or the stream is being captured and the workspace cannot grow).
+bsort_status reserve_batch(bsort_t h, bsort_key_type kt, const SegSpan *spans, uint32_t nsegs,
+                           cudaStream_t st, BatchParts *B)
+{
+    bsort_status rs = make_batch_plan(h, kt, spans, nsegs, batch_room(h), B);
+    if (rs != BSORT_OK || B->info.n == 0) return rs;
+    if (B->joined && B->total > h->ws_bytes) {
+        cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+        const bool grows =
+            cudaStreamIsCapturing(st, &cs) == cudaSuccess && cs == cudaStreamCaptureStatusNone;
+        if (!grows) cudaGetLastError();
+        rs = grows && B->total < h->ws_denied ? ensure_workspace(h, B->total) : BSORT_ENOMEM;
+        if (rs != BSORT_ENOMEM) return rs;
+        if (grows && B->total < h->ws_denied) h->ws_denied = B->total;
+        rs = make_batch_plan(h, kt, spans, nsegs, 0, B);
+        if (rs != BSORT_OK) return rs;
+    }
+    return ensure_workspace(h, B->total);
+}
+
+// The descriptors of a part, as the kernels read them.
+void write_descriptors(const BatchPlan &B, uint32_t *hw)
+{
+    memset(hw, 0, B.d_words * 4);
+    for (int c = 0; c < kNumDirect; ++c)
+        if (!B.direct[c].empty())
+            memcpy(hw + B.d_direct[c], B.direct[c].data(), B.direct[c].size() * 4);
+    if (!B.sub_seg.empty()) memcpy(hw + B.d_sub, B.sub_seg.data(), B.sub_seg.size() * 4);
+    if (!B.segs.empty()) memcpy(hw + B.d_segs, B.segs.data(), B.segs.size() * sizeof(SegInfo));
+    if (!B.units.empty()) memcpy(hw + B.d_units, B.units.data(), B.units.size() * 4);
+}
+
+// One part of a batch; stage: pinned memory of its descriptors, from the
+// handle's shared staging if `shared` (its event is recorded behind the copy).
+bsort_status run_batch_part(bsort_t h, bsort_key_type kt, const void *kin, void *kout,
+                            const BatchPlan &B, uint32_t *stage, bool shared, cudaStream_t st)
+{
+    bsort_status rs = BSORT_OK;
     cudaError_t e;
-    // segments of one key: copies
     const uint64_t kb = B.wide ? 8 : 4;
-    if (kout != kin)
-        for (uint32_t q = 0; q < nsegs; ++q)
-            if (spans[q].n == 1) {
-                e = cudaMemcpyAsync(static_cast<char *>(kout) + spans[q].begin * kb,
-                                    static_cast<const char *>(kin) + spans[q].begin * kb, kb,
-                                    cudaMemcpyDeviceToDevice, st);
-                if (e != cudaSuccess) return cuda_fail(h, e, "copy of a one-key segment");
-            }
     unsigned char *ws = static_cast<unsigned char *>(h->ws);
     int *err = reinterpret_cast<int *>(ws);
     uint32_t *ticket = reinterpret_cast<uint32_t *>(ws + 64);
@@ -1739,61 +1850,15 @@ bsort_status run_batch(bsort_t h, bsort_key_type kt, const void *kin, void *kout
     const uint32_t *ki = static_cast<const uint32_t *>(kin);
     uint32_t *ko = static_cast<uint32_t *>(kout);
     Seq seq(h, st);
-    if (B.d_words && stage) {
-        // descriptors from the caller's pinned buffer (a graph's own)
-        uint32_t *hw = static_cast<uint32_t *>(stage);
-        const uint64_t bytes = B.d_words * 4;
-        memset(hw, 0, bytes);
-        for (int c = 0; c < kNumDirect; ++c)
-            if (!B.direct[c].empty())
-                memcpy(hw + B.d_direct[c], B.direct[c].data(), B.direct[c].size() * 4);
-        if (!B.sub_seg.empty()) memcpy(hw + B.d_sub, B.sub_seg.data(), B.sub_seg.size() * 4);
-        if (!B.segs.empty()) memcpy(hw + B.d_segs, B.segs.data(), B.segs.size() * sizeof(SegInfo));
-        if (!B.units.empty()) memcpy(hw + B.d_units, B.units.data(), B.units.size() * 4);
-        e = cudaMemcpyAsync(desc, hw, bytes, cudaMemcpyHostToDevice, st);
+    if (B.d_words) {
+        write_descriptors(B, stage);
+        e = cudaMemcpyAsync(desc, stage, B.d_words * 4, cudaMemcpyHostToDevice, st);
         if (e != cudaSuccess) return cuda_fail(h, e, "copy of the batch descriptors");
-    } else if (B.d_words) {
-        // descriptors: pinned staging -> workspace (the staging is reused
-        // only after the previous copy out of it has completed)
-        const uint64_t bytes = B.d_words * 4;
-        if (h->stage_pending) {
-            e = cudaEventSynchronize(h->stage_ev);
-            if (e != cudaSuccess) return cuda_fail(h, e, "wait for the staging copy");
-            h->stage_pending = false;
+        if (shared) {
+            e = cudaEventRecord(h->stage_ev, st);
+            if (e != cudaSuccess) return cuda_fail(h, e, "cudaEventRecord");
+            h->stage_pending = true;
         }
-        if (bytes > h->stage_bytes) {
-            // grown geometrically: freeing pinned memory waits for the device,
-            // and pinning is slow, so a stream of growing batches (the request
-            // loop) must not pay them at every new maximum
-            const uint64_t grow = std::max<uint64_t>({bytes, 2 * h->stage_bytes, 1ull << 20});
-            if (h->stage) cudaFreeHost(h->stage);
-            h->stage = nullptr;
-            h->stage_bytes = 0;
-            e = cudaHostAlloc(&h->stage, grow, cudaHostAllocDefault);
-            if (e != cudaSuccess) {
-                cudaGetLastError();
-                return fail(h, BSORT_ENOMEM, "pinned staging of %llu bytes: %s",
-                            (unsigned long long)grow, cudaGetErrorString(e));
-            }
-            h->stage_bytes = grow;
-        }
-        if (!h->stage_ev) {
-            e = cudaEventCreateWithFlags(&h->stage_ev, cudaEventDisableTiming);
-            if (e != cudaSuccess) return cuda_fail(h, e, "cudaEventCreate");
-        }
-        uint32_t *hw = static_cast<uint32_t *>(h->stage);
-        memset(hw, 0, bytes);
-        for (int c = 0; c < kNumDirect; ++c)
-            if (!B.direct[c].empty())
-                memcpy(hw + B.d_direct[c], B.direct[c].data(), B.direct[c].size() * 4);
-        if (!B.sub_seg.empty()) memcpy(hw + B.d_sub, B.sub_seg.data(), B.sub_seg.size() * 4);
-        if (!B.segs.empty()) memcpy(hw + B.d_segs, B.segs.data(), B.segs.size() * sizeof(SegInfo));
-        if (!B.units.empty()) memcpy(hw + B.d_units, B.units.data(), B.units.size() * 4);
-        e = cudaMemcpyAsync(desc, hw, bytes, cudaMemcpyHostToDevice, st);
-        if (e != cudaSuccess) return cuda_fail(h, e, "copy of the batch descriptors");
-        e = cudaEventRecord(h->stage_ev, st);
-        if (e != cudaSuccess) return cuda_fail(h, e, "cudaEventRecord");
-        h->stage_pending = true;
     }
     // direct segments: one launch per unit shape
     for (int c = 0; c < kNumDirect; ++c) {
@@ -1875,6 +1940,68 @@ bsort_status run_batch(bsort_t h, bsort_key_type kt, const void *kin, void *kout
     return BSORT_OK;
 }
 
+// The batch of a plan whose workspace the handle has (reserve_batch).
+// stage: when not null, pinned host memory of the plan's descriptor words that
+// the caller keeps unchanged for as long as the upload may run again (a
+// captured graph replays it); the handle's shared staging is used otherwise.
+bsort_status run_batch(bsort_t h, bsort_key_type kt, const void *kin, void *kout,
+                       const SegSpan *spans, uint32_t nsegs, const BatchParts &B, cudaStream_t st,
+                       void *stage = nullptr)
+{
+    if (B.info.n == 0) return BSORT_OK;
+    cudaError_t e;
+    // segments of one key: copies
+    const uint64_t kb = kt == BSORT_U64 ? 8 : 4;
+    if (kout != kin)
+        for (uint32_t q = 0; q < nsegs; ++q)
+            if (spans[q].n == 1) {
+                e = cudaMemcpyAsync(static_cast<char *>(kout) + spans[q].begin * kb,
+                                    static_cast<const char *>(kin) + spans[q].begin * kb, kb,
+                                    cudaMemcpyDeviceToDevice, st);
+                if (e != cudaSuccess) return cuda_fail(h, e, "copy of a one-key segment");
+            }
+    const bool shared = B.words && !stage;
+    if (shared) {
+        // the staging is reused only after the previous copy out of it has
+        // completed
+        const uint64_t bytes = B.words * 4;
+        if (h->stage_pending) {
+            e = cudaEventSynchronize(h->stage_ev);
+            if (e != cudaSuccess) return cuda_fail(h, e, "wait for the staging copy");
+            h->stage_pending = false;
+        }
+        if (bytes > h->stage_bytes) {
+            // grown geometrically: freeing pinned memory waits for the device,
+            // and pinning is slow, so a stream of growing batches (the request
+            // loop) must not pay them at every new maximum
+            const uint64_t grow = std::max<uint64_t>({bytes, 2 * h->stage_bytes, 1ull << 20});
+            if (h->stage) cudaFreeHost(h->stage);
+            h->stage = nullptr;
+            h->stage_bytes = 0;
+            e = cudaHostAlloc(&h->stage, grow, cudaHostAllocDefault);
+            if (e != cudaSuccess) {
+                cudaGetLastError();
+                return fail(h, BSORT_ENOMEM, "pinned staging of %llu bytes: %s",
+                            (unsigned long long)grow, cudaGetErrorString(e));
+            }
+            h->stage_bytes = grow;
+        }
+        if (!h->stage_ev) {
+            e = cudaEventCreateWithFlags(&h->stage_ev, cudaEventDisableTiming);
+            if (e != cudaSuccess) return cuda_fail(h, e, "cudaEventCreate");
+        }
+        stage = h->stage;
+    }
+    uint32_t *hw = static_cast<uint32_t *>(stage);
+    for (const BatchPlan &P : B.part) {
+        if (P.info.n == 0) continue;
+        const bsort_status rs = run_batch_part(h, kt, kin, kout, P, hw, shared, st);
+        if (rs != BSORT_OK) return rs;
+        hw += P.d_words;
+    }
+    return BSORT_OK;
+}
+
 // run_batch through the handle's batch-graph cache (BSORT_FLAG_GRAPHS): a
 // call whose segment table, key type, buffers, stream and workspace match a
 // cached graph replays it with one graph launch (no planning on the host);
@@ -1884,12 +2011,18 @@ bsort_status run_batch(bsort_t h, bsort_key_type kt, const void *kin, void *kout
 bsort_status run_batch_graph(bsort_t h, bsort_key_type kt, const void *kin, void *kout,
                              const SegSpan *spans, uint32_t nsegs, cudaStream_t st)
 {
+    BatchParts B;
+    auto plain = [&]() {
+        bsort_status rs = prepare(h);
+        if (rs == BSORT_OK) rs = reserve_batch(h, kt, spans, nsegs, st, &B);
+        return rs == BSORT_OK ? run_batch(h, kt, kin, kout, spans, nsegs, B, st) : rs;
+    };
     if (!(h->flags & BSORT_FLAG_GRAPHS) || nsegs == 0 || st == nullptr || st == cudaStreamLegacy)
-        return run_batch(h, kt, kin, kout, spans, nsegs, st);
+        return plain();
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     cudaError_t e = cudaStreamIsCapturing(st, &cs);
     if (e != cudaSuccess) return cuda_fail(h, e, "cudaStreamIsCapturing");
-    if (cs != cudaStreamCaptureStatusNone) return run_batch(h, kt, kin, kout, spans, nsegs, st);
+    if (cs != cudaStreamCaptureStatusNone) return plain();
     uint64_t hash = 0x9E3779B97F4A7C15ull ^ nsegs;
     for (uint32_t q = 0; q < nsegs; ++q) {
         hash = (hash ^ spans[q].begin) * 0xBF58476D1CE4E5B9ull;
@@ -1910,18 +2043,15 @@ bsort_status run_batch_graph(bsort_t h, bsort_key_type kt, const void *kin, void
     // settle the plan and the workspace outside the capture
     bsort_status rs = prepare(h);
     if (rs != BSORT_OK) return rs;
-    BatchPlan B;
-    rs = make_batch_plan(h, kt, spans, nsegs, &B);
-    if (rs != BSORT_OK) return rs;
-    rs = ensure_workspace(h, B.total);  // (covers the plain sorts of large segments)
+    rs = reserve_batch(h, kt, spans, nsegs, st, &B);  // (covers the plain sorts of large segments)
     if (rs != BSORT_OK) return rs;
     void *desc = nullptr;
-    if (B.d_words) {
-        e = cudaHostAlloc(&desc, B.d_words * 4, cudaHostAllocDefault);
+    if (B.words) {
+        e = cudaHostAlloc(&desc, B.words * 4, cudaHostAllocDefault);
         if (e != cudaSuccess) {
             cudaGetLastError();
             return fail(h, BSORT_ENOMEM, "pinned descriptors of %llu bytes",
-                        (unsigned long long)(B.d_words * 4));
+                        (unsigned long long)(B.words * 4));
         }
     }
     e = cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal);
@@ -1930,7 +2060,7 @@ bsort_status run_batch_graph(bsort_t h, bsort_key_type kt, const void *kin, void
         return cuda_fail(h, e, "cudaStreamBeginCapture");
     }
     h->capturing = true;
-    rs = run_batch(h, kt, kin, kout, spans, nsegs, st, desc ? desc : nullptr);
+    rs = run_batch(h, kt, kin, kout, spans, nsegs, B, st, desc);
     h->capturing = false;
     cudaGraph_t graph = nullptr;
     e = cudaStreamEndCapture(st, &graph);
@@ -2196,9 +2326,9 @@ void serve_run(bsort_server *S, int li, const std::vector<bsort_server::Req *> &
         // that fits, found by bisection (the workspace a batch needs grows
         // with its segments); a single job always fits
         auto fits = [&](size_t i, size_t j) {
-            BatchPlan B;
-            return make_batch_plan(ctx, kt, spans.data() + i, (uint32_t)(j - i), &B) ==
-                       BSORT_OK &&
+            BatchParts B;
+            return make_batch_plan(ctx, kt, spans.data() + i, (uint32_t)(j - i), ctx->ws_bytes,
+                                   &B) == BSORT_OK &&
                    B.total <= ctx->ws_bytes;
         };
         size_t i = 0;
@@ -2213,8 +2343,13 @@ void serve_run(bsort_server *S, int li, const std::vector<bsort_server::Req *> &
                 }
                 j = lo;
             }
-            const bsort_status st = run_batch(ctx, kt, S->arena, S->arena, spans.data() + i,
-                                              (uint32_t)(j - i), L.s_run);
+            BatchParts B;
+            bsort_status st = prepare(ctx);
+            if (st == BSORT_OK)
+                st = reserve_batch(ctx, kt, spans.data() + i, (uint32_t)(j - i), L.s_run, &B);
+            if (st == BSORT_OK)
+                st = run_batch(ctx, kt, S->arena, S->arena, spans.data() + i, (uint32_t)(j - i), B,
+                               L.s_run);
             if (st != BSORT_OK)
                 for (size_t q = i; q < j; ++q) owners[q]->status = st;
             i = j;
@@ -2605,8 +2740,8 @@ bsort_status bsort_plan_batch(bsort_t h, bsort_key_type kt, const uint64_t *seg_
     std::vector<SegSpan> spans;
     bsort_status st = spans_from_offsets(h, seg_offsets, num_segs, &spans);
     if (st != BSORT_OK) return st;
-    BatchPlan B;
-    st = make_batch_plan(h, kt, spans.data(), num_segs, &B);
+    BatchParts B;
+    st = make_batch_plan(h, kt, spans.data(), num_segs, batch_room(h), &B);
     if (st != BSORT_OK) return st;
     *out = B.info;
     return BSORT_OK;
@@ -2654,10 +2789,10 @@ bsort_status bsort_submit(bsort_t h, const bsort_request *req, uint64_t *ticket)
     const int lane = lane_of(h, kt, req->n);
     if (req->n > 1) {  // its batch alone must fit the lane's workspace
         SegSpan one = {0, req->n};
-        BatchPlan B;
-        bsort_status rs = make_batch_plan(h, kt, &one, 1, &B);
-        if (rs != BSORT_OK) return rs;
+        BatchParts B;
         const uint64_t ws = S->lane[lane].ctx->ws_bytes;
+        bsort_status rs = make_batch_plan(h, kt, &one, 1, ws, &B);
+        if (rs != BSORT_OK) return rs;
         if (B.total > ws)
             return fail(h, BSORT_ENOMEM, "request needs %llu workspace bytes, serving has %llu",
                         (unsigned long long)B.total, (unsigned long long)ws);
