@@ -1577,13 +1577,21 @@ JoinRule join_rule(const bsort_t h, bool wide, const SegSpan *spans, uint32_t ns
     JoinRule j;
     const BatchSizes z = batch_sizes(h, wide);
     if (h->flags & BSORT_FLAG_LOW_MEMORY) return j;
-    if (wide) {
+    if (wide) {  // direct segments of the larger clusters, when there are many
+        bool sampled = false;
+        for (uint32_t q = 0; q < nsegs; ++q) sampled |= spans[q].n > z.dmax && spans[q].n <= z.smax;
+        const uint64_t from = (sampled ? 2 : 4) * z.unit;
         uint64_t keys = 0;
         for (uint32_t q = 0; q < nsegs; ++q)
-            if (spans[q].n > z.unit && spans[q].n <= z.dmax) keys += spans[q].n;
-        if (!h->direct_max_set && keys >= kBatchJoinDirectU64) j = {z.unit, z.dmax};
-    } else {
-        j = {z.smax, kBatchJoinMax};
+            if (spans[q].n > from && spans[q].n <= z.dmax) keys += spans[q].n;
+        if (!h->direct_max_set && keys >= kBatchJoinDirectU64) j = {from, z.dmax};
+    } else {  // larger ones than the sampled, unless one is alone
+        uint32_t large = 0, sampled = 0;
+        for (uint32_t q = 0; q < nsegs; ++q) {
+            large += spans[q].n > z.smax && spans[q].n <= kBatchJoinMax;
+            sampled += spans[q].n > z.dmax && spans[q].n <= z.smax;
+        }
+        if (large > 1 || (large && sampled)) j = {z.smax, kBatchJoinMax};
     }
     return j;
 }

@@ -48,13 +48,30 @@ def test_parts_count_every_segment_once():
 
 
 @pytest.mark.parametrize("n", [524289, 900001, 1 << 20, 1 << 21])
-def test_low_memory_segments_are_plain_sorts(n):
+def test_low_memory_and_lone_segments_are_plain_sorts(n):
     low = dict(flags=pkg.BSORT_FLAG_LOW_MEMORY)
     assert _plan([n], **low).workspace_bytes == _plain(n, **low).workspace_bytes
     assert _plan([n] * 20, **low).workspace_bytes == _plain(n, **low).workspace_bytes
+    one = _plan([n])  # (another's sequence of launches costs more than it saves)
+    assert one.num_kernels == _plain(n).num_kernels and one.large_segs == 1
+    assert _plan([n, n]).num_kernels == 7
+    assert _plan([n, 300000]).num_kernels == 7
+    assert _plan([n, 5000]).num_kernels == one.num_kernels + 1
 
 
 def test_low_memory_u64_stays_with_clusters():
     sizes = [100000] * 200
     assert _plan(sizes, U64).num_kernels == 7
     assert _plan(sizes, U64, flags=pkg.BSORT_FLAG_LOW_MEMORY).num_kernels == 1
+
+
+@pytest.mark.parametrize("n,joins", [(16385, False), (32768, False), (65536, False),
+                                     (65537, True), (131072, True)])
+def test_u64_direct_segments_that_join(n, joins):
+    """2^24 keys in all: clusters of 2 and 4 CTAs are faster by themselves."""
+    p = _plan([n] * ((1 << 24) // n + 1), U64)
+    assert p.num_kernels == (7 if joins else 1)
+    few = _plan([n] * ((1 << 21) // n), U64)
+    assert few.num_kernels == 1
+    beside = _plan([n] * ((1 << 24) // n + 1) + [500000], U64)  # a sampled segment
+    assert beside.num_kernels == (7 if n > 32768 else 8)
