@@ -320,16 +320,24 @@ class BucketSorter:
         self.batch_direct_max = batch_direct_max
         self.ws = None
         self.h = None
+        self.denied = float("inf")  # smallest workspace the device had no room for
+        # A workspace that grows is a fixed one to its handle between two
+        # calls, and the plans that fit it must not decide how it grows:
+        # those come from a handle without one.
+        self.planner = None if workspace_bytes else bsort_create(self._config())
         self._make(workspace_bytes)
+
+    def _config(self):
+        return bsort_config(device=self.device, tile=self.tile, samples=self.samples,
+                            flags=self.flags, buckets=self.buckets,
+                            batch_direct_max=self.batch_direct_max)
 
     def _make(self, nbytes):
         torch = self.torch
         if self.h is not None:
             bsort_destroy(self.h)
             self.h = None
-        cfg = bsort_config(device=self.device, tile=self.tile, samples=self.samples,
-                           flags=self.flags, buckets=self.buckets,
-                           batch_direct_max=self.batch_direct_max)
+        cfg = self._config()
         if nbytes:
             self.ws = torch.empty(int(nbytes), dtype=torch.uint8,
                                   device="cuda:%d" % self.device)
@@ -338,12 +346,28 @@ class BucketSorter:
         self.h = bsort_create(cfg)
 
     def plan(self, n, key_type="u32", val_bytes=0):
-        return bsort_plan(self.h, _KEY_TYPES[key_type], val_bytes, n)
+        return bsort_plan(self.planner or self.h, _KEY_TYPES[key_type], val_bytes, n)
+
+    def _grow(self, nbytes, need):
+        """A workspace of nbytes; where the device had no room for as much, of
+        what need() says on a handle that has none to give."""
+        if nbytes < self.denied:
+            try:
+                self._make(max(nbytes, 256))
+                return
+            except self.torch.cuda.OutOfMemoryError:
+                self.denied = nbytes
+                self.ws = None
+                self._make(256)
+        least = need()
+        if self.ws.numel() < least:
+            self._make(max(least, 256))
 
     def _ensure(self, n, key_type, val_bytes, extra=0):
         need = self.plan(n, key_type, val_bytes).workspace_bytes + extra
         if self.ws is None or self.ws.numel() < need:
-            self._make(max(need, 256))
+            self._grow(need, lambda: bsort_plan(self.h, _KEY_TYPES[key_type], val_bytes,
+                                                n).workspace_bytes + extra)
 
     def _stream(self):
         return ctypes.c_void_p(self.torch.cuda.current_stream(self.device).cuda_stream)
@@ -370,7 +394,7 @@ class BucketSorter:
         return out_keys, out_vals
 
     def plan_batch(self, seg_offsets, key_type="u32"):
-        return bsort_plan_batch(self.h, _KEY_TYPES[key_type], seg_offsets)
+        return bsort_plan_batch(self.planner or self.h, _KEY_TYPES[key_type], seg_offsets)
 
     def sort_batch(self, keys, seg_offsets, out=None, key_type="u32"):
         """Sort every segment [seg_offsets[q], seg_offsets[q+1]) of keys on
@@ -379,7 +403,8 @@ class BucketSorter:
             out = self.torch.empty_like(keys)
         need = self.plan_batch(seg_offsets, key_type).workspace_bytes
         if self.ws is None or self.ws.numel() < need:
-            self._make(max(need, 256))
+            self._grow(need, lambda: bsort_plan_batch(self.h, _KEY_TYPES[key_type],
+                                                      seg_offsets).workspace_bytes)
         bsort_sort_batch(self.h, _KEY_TYPES[key_type], keys.data_ptr(), out.data_ptr(),
                          seg_offsets, self._stream())
         return out
@@ -406,9 +431,10 @@ class BucketSorter:
         return bsort_kernel_times(self.h)
 
     def close(self):
-        if self.h is not None:
-            bsort_destroy(self.h)
-            self.h = None
+        for h in (self.h, getattr(self, "planner", None)):
+            if h is not None:
+                bsort_destroy(h)
+        self.h = self.planner = None
         self.ws = None
 
     def __del__(self):

@@ -67,6 +67,50 @@ def test_out_of_memory_sorts_without_joining(bits, sizes):
     pkg.bsort_destroy(h)
 
 
+def test_wrapper_out_of_memory(monkeypatch):
+    """The same through the wrapper, whose workspace is a torch tensor: its
+    allocation fails above a limit."""
+    off, d, want = _batch(2)
+    sorter = pkg.BucketSorter()
+    need = sorter.plan_batch(off).workspace_bytes
+    limit = need // 2
+    real = torch.empty
+
+    def empty(*a, **kw):
+        if kw.get("dtype") == torch.uint8 and a[0] > limit:
+            raise torch.cuda.OutOfMemoryError("no room")
+        return real(*a, **kw)
+
+    out = torch.empty_like(d)
+    monkeypatch.setattr(torch, "empty", empty)
+    sorter.sort_batch(d, off, out)
+    sorter.sync()
+    assert sorter.ws.numel() <= limit
+    assert _same(out, want)
+    kept = sorter.ws.data_ptr()
+    out.zero_()
+    sorter.sort_batch(d, off, out)  # (as much is not asked for again)
+    assert sorter.ws.data_ptr() == kept
+    assert _same(out, want)
+    sorter.close()
+
+
+def test_wrapper_plans_do_not_depend_on_earlier_calls():
+    """A small batch first: the workspace it leaves must not decide how the
+    next one is sorted."""
+    off, d, want = _batch(3)
+    small_off, small, small_want = _batch(4, sizes=[5000, 600])
+    sorter = pkg.BucketSorter()
+    need = sorter.plan_batch(off).workspace_bytes
+    out_s, out = torch.empty_like(small), torch.empty_like(d)
+    sorter.sort_batch(small, small_off, out_s)
+    assert sorter.plan_batch(off).workspace_bytes == need
+    sorter.sort_batch(d, off, out)
+    assert sorter.ws.numel() >= need
+    assert _same(out_s, small_want) and _same(out, want)
+    sorter.close()
+
+
 def test_capture_with_a_small_workspace():
     """Under the caller's capture the workspace cannot grow: the plan that fits
     what is there is taken."""
