@@ -344,9 +344,10 @@ class BucketSorter:
             cfg.workspace = self.ws.data_ptr()
             cfg.workspace_bytes = int(nbytes)
         self.h = bsort_create(cfg)
+        self.plan_h = self.h if self.planner is None else self.planner
 
     def plan(self, n, key_type="u32", val_bytes=0):
-        return bsort_plan(self.planner or self.h, _KEY_TYPES[key_type], val_bytes, n)
+        return bsort_plan(self.plan_h, _KEY_TYPES[key_type], val_bytes, n)
 
     def _grow(self, nbytes, need):
         """A workspace of nbytes; where the device had no room for as much, of
@@ -364,7 +365,7 @@ class BucketSorter:
             self._make(max(least, 256))
 
     def _ensure(self, n, key_type, val_bytes, extra=0):
-        need = self.plan(n, key_type, val_bytes).workspace_bytes + extra
+        need = bsort_plan(self.plan_h, _KEY_TYPES[key_type], val_bytes, n).workspace_bytes + extra
         if self.ws is None or self.ws.numel() < need:
             self._grow(need, lambda: bsort_plan(self.h, _KEY_TYPES[key_type], val_bytes,
                                                 n).workspace_bytes + extra)
@@ -394,7 +395,7 @@ class BucketSorter:
         return out_keys, out_vals
 
     def plan_batch(self, seg_offsets, key_type="u32"):
-        return bsort_plan_batch(self.planner or self.h, _KEY_TYPES[key_type], seg_offsets)
+        return bsort_plan_batch(self.plan_h, _KEY_TYPES[key_type], seg_offsets)
 
     def sort_batch(self, keys, seg_offsets, out=None, key_type="u32"):
         """Sort every segment [seg_offsets[q], seg_offsets[q+1]) of keys on
@@ -434,7 +435,7 @@ class BucketSorter:
         for h in (self.h, getattr(self, "planner", None)):
             if h is not None:
                 bsort_destroy(h)
-        self.h = self.planner = None
+        self.h = self.planner = self.plan_h = None
         self.ws = None
 
     def __del__(self):

@@ -388,14 +388,15 @@ bool tuned_plan(bool pairs, uint64_t n, uint64_t *t, uint64_t *s)
 }
 
 bsort_status make_plan_with(bsort_t h, bsort_key_type kt, uint32_t vb, uint64_t n, Plan *P,
-                            bool use_table);
+                            bool use_table, const TunedPlan *alt = nullptr);
 
 // Plan of n >= kMaxN 32-bit keys (keys only): the top level sorts sublists of
 // t = 32768 (one CTA each), takes b buckets of about kTopBucket keys, and the
 // largest sample distance w whose share of the bucket bound, (m-1)(w-1),
 // stays within a quarter of the average bucket; Step 9 sorts each bucket by
 // a plan of its own in a slice of the workspace sized for the bound.
-bsort_status make_plan(bsort_t h, bsort_key_type kt, uint32_t vb, uint64_t n, Plan *P);
+bsort_status make_plan(bsort_t h, bsort_key_type kt, uint32_t vb, uint64_t n, Plan *P,
+                       uint64_t extra = 0);
 
 bsort_status make_plan_two_level(bsort_t h, bsort_key_type kt, uint64_t n, Plan *P)
 {
@@ -480,8 +481,13 @@ bsort_status make_plan_two_level(bsort_t h, bsort_key_type kt, uint64_t n, Plan 
 
 // The plan of one job: the tabled (t, s) for n's size class when there is
 // one and it admits a plan, else the cost model's choice; keys-only sorts
-// of 32-bit keys that no one-level plan fits take two levels.
-bsort_status make_plan(bsort_t h, bsort_key_type kt, uint32_t vb, uint64_t n, Plan *P)
+// of 32-bit keys that no one-level plan fits take two levels.  Where that plan
+// and `extra` bytes beside it exceed the workspace that can be had, the first
+// of a few with fewer records and runs that does not: sublists of twice the
+// size, of half as many samples too, the cost model's choice (2^27 pairs: 3.43
+// GB as tabled, 2.57 by the model); if none does, the one that needs least.
+bsort_status make_plan_in(bsort_t h, bsort_key_type kt, uint32_t vb, uint64_t n, Plan *P,
+                          uint64_t extra, uint64_t room)
 {
     bsort_status st = make_plan_with(h, kt, vb, n, P, true);
     if (st == BSORT_EUNSUPPORTED) st = make_plan_with(h, kt, vb, n, P, false);
@@ -491,11 +497,35 @@ bsort_status make_plan(bsort_t h, bsort_key_type kt, uint32_t vb, uint64_t n, Pl
         memset(P, 0, sizeof(*P));
         st = make_plan_two_level(h, kt, n, P);
     }
+    if (st != BSORT_OK || forced || P->total + extra <= room || P->info.single_tile ||
+        P->info.levels == 2)
+        return st;
+    const uint32_t t = P->info.t, s = P->info.s;
+    for (int i = 0; i < 3 && P->total + extra > room; ++i) {
+        Plan Q;
+        const TunedPlan alt = {0, 2 * t, i ? s / 2 : s};
+        if (make_plan_with(h, kt, vb, n, &Q, i < 2, i < 2 ? &alt : nullptr) == BSORT_OK &&
+            Q.total < P->total)
+            *P = Q;
+    }
+    return BSORT_OK;
+}
+
+bsort_status make_plan(bsort_t h, bsort_key_type kt, uint32_t vb, uint64_t n, Plan *P,
+                       uint64_t extra)
+{
+    // a fixed workspace's bytes; where the device had no room for as much, the
+    // least
+    const uint64_t room = h && h->ws_fixed ? h->ws_bytes : ~0ull;
+    bsort_status st = make_plan_in(h, kt, vb, n, P, extra, room);
+    if (st == BSORT_OK && h && !h->ws_fixed && P->total + extra >= h->ws_denied)
+        st = make_plan_in(h, kt, vb, n, P, extra, 0);
     return st;
 }
 
+// alt: a (t, s) in the table's place.
 bsort_status make_plan_with(bsort_t h, bsort_key_type kt, uint32_t vb, uint64_t n, Plan *P,
-                            bool use_table)
+                            bool use_table, const TunedPlan *alt)
 {
     memset(P, 0, sizeof(*P));
     P->info.levels = 1;
@@ -562,9 +592,11 @@ bsort_status make_plan_with(bsort_t h, bsort_key_type kt, uint32_t vb, uint64_t 
         uint64_t tt = 0, ts = 0;
         if (use_table && table_ok && !forced_t && !forced_s && !forced_b &&
             tuned_plan(vb != 0, n, &tt, &ts)) {
-            forced_t = tt;
-            forced_s = ts;
+            forced_t = alt ? alt->t : tt;
+            forced_s = alt ? alt->s : ts;
             auto_b = true;
+        } else if (alt) {
+            return BSORT_EUNSUPPORTED;
         }
         // candidates: forced t or every sublist shape; forced s or every
         // power of two with w = t/s >= 16 and s <= kMaxSamples.  The unit is
@@ -799,6 +831,41 @@ bsort_status ensure_workspace(bsort_t h, uint64_t bytes)
     return BSORT_OK;
 }
 
+// Whether a call on this stream may allocate: not while it is captured.
+bool may_allocate(cudaStream_t st)
+{
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &cs) == cudaSuccess) return cs == cudaStreamCaptureStatusNone;
+    cudaGetLastError();
+    return false;
+}
+
+// Plan a sort and have its workspace, and `extra` bytes behind it: a plan that
+// needs less where the tabled one's cannot be had.  (A call that reserves
+// again inside finds the same plan.)
+bsort_status reserve_plan(bsort_t h, bsort_key_type kt, uint32_t vb, uint64_t n, uint64_t extra,
+                          cudaStream_t st, Plan *P)
+{
+    bsort_status rs = make_plan(h, kt, vb, n, P, extra);
+    if (rs != BSORT_OK) return rs;
+    uint64_t need = P->total + extra;
+    if (need > h->ws_bytes && !h->ws_fixed) {
+        const bool grows = may_allocate(st);
+        if (grows) {
+            rs = ensure_workspace(h, need);
+            if (rs != BSORT_ENOMEM) return rs;
+            h->ws_denied = std::min(h->ws_denied, need);
+        }
+        Plan Q;
+        if (make_plan_in(h, kt, vb, n, &Q, extra, grows ? 0 : h->ws_bytes) == BSORT_OK &&
+            Q.total < P->total) {
+            *P = Q;
+            need = Q.total + extra;
+        }
+    }
+    return ensure_workspace(h, need);
+}
+
 bsort_status prepare(bsort_t h)
 {
     if (!h) return BSORT_EINVAL;
@@ -920,7 +987,7 @@ cudaError_t stream_after(cudaStream_t to, cudaStream_t from, cudaEvent_t ev)
 // sublists and buckets and 16-byte sample records merged in L2 (Step 4).
 bsort_status run_sort(bsort_t h, bsort_key_type kt, const void *kin, const void *vin, void *kout,
                       void *vout, uint32_t vb, uint64_t n, cudaStream_t st,
-                      const HostPipe *hp = nullptr);
+                      const HostPipe *hp = nullptr, uint64_t extra = 0);
 
 // A two-level plan (n' >= 2^32, keys-only 32-bit keys): Steps 1-6 as in
 // run_sort over sublists of 32768 keys, Steps 7-8 with 64-bit offsets
@@ -1032,14 +1099,13 @@ bsort_status run_pairs_u64(bsort_t h, const void *kin, const void *vin, void *ko
     if (n >= kMaxN) return fail(h, BSORT_EUNSUPPORTED, "n = %llu exceeds 2^32 - 2^16", (unsigned long long)n);
     if (n == 0) return BSORT_OK;
     Plan PA;
-    rs = make_plan(h, BSORT_U32, 4, n, &PA);
-    if (rs != BSORT_OK) return rs;
     const uint64_t words = align_up(n * 4);
     const bool in_place = kin == kout || vin == vout;
     const uint64_t keep = in_place ? align_up(n * 8) + align_up(n * (uint64_t)vb) : 0;
-    const uint64_t base = align_up(PA.total);
-    rs = ensure_workspace(h, base + 5 * words + keep);
+    const uint64_t extra = 5 * words + keep;  // (a plan's total is aligned)
+    rs = reserve_plan(h, BSORT_U32, 4, n, extra, st, &PA);
     if (rs != BSORT_OK) return rs;
+    const uint64_t base = align_up(PA.total);
     unsigned char *ws = static_cast<unsigned char *>(h->ws) + base;
     uint32_t *lo = reinterpret_cast<uint32_t *>(ws);
     uint32_t *iota = reinterpret_cast<uint32_t *>(ws + words);
@@ -1060,11 +1126,11 @@ bsort_status run_pairs_u64(bsort_t h, const void *kin, const void *vin, void *ko
     }
     e = launch_u64_split(k64, lo, iota, n, st);
     if (e != cudaSuccess) return cuda_fail(h, e, "split 64-bit keys");
-    rs = run_sort(h, BSORT_U32, lo, iota, scratch, p1, 4, n, st);  // pass A: low halves
+    rs = run_sort(h, BSORT_U32, lo, iota, scratch, p1, 4, n, st, nullptr, extra);  // low halves
     if (rs != BSORT_OK) return rs;
     e = launch_u64_gather_hi(k64, p1, lo, n, st);
     if (e != cudaSuccess) return cuda_fail(h, e, "gather high halves");
-    rs = run_sort(h, BSORT_U32, lo, iota, scratch, p2, 4, n, st);  // pass B: high halves
+    rs = run_sort(h, BSORT_U32, lo, iota, scratch, p2, 4, n, st, nullptr, extra);  // high halves
     if (rs != BSORT_OK) return rs;
     e = launch_u64_final(k64, v, (int)vb, p1, p2, static_cast<uint64_t *>(kout), vout, n, st);
     if (e != cudaSuccess) return cuda_fail(h, e, "apply the permutations");
@@ -1147,16 +1213,15 @@ bsort_status run_sort_u64(bsort_t h, const Plan &P, const void *kin, void *kout,
 }
 
 bsort_status run_sort(bsort_t h, bsort_key_type kt, const void *kin, const void *vin, void *kout,
-                      void *vout, uint32_t vb, uint64_t n, cudaStream_t st, const HostPipe *hp)
+                      void *vout, uint32_t vb, uint64_t n, cudaStream_t st, const HostPipe *hp,
+                      uint64_t extra)
 {
     bsort_status rs = prepare(h);
     if (rs != BSORT_OK) return rs;
     if (hp && (h->flags & BSORT_FLAG_TEST_STALL_SCAN))
         return fail(h, BSORT_EINVAL, "BSORT_FLAG_TEST_STALL_SCAN is for device-buffer calls");
     Plan P;
-    rs = make_plan(h, kt, vb, n, &P);
-    if (rs != BSORT_OK) return rs;
-    rs = ensure_workspace(h, P.total);
+    rs = reserve_plan(h, kt, vb, n, extra, st, &P);
     if (rs != BSORT_OK) return rs;
     h->last = P;
     h->have_last = true;
@@ -1415,7 +1480,7 @@ bsort_status run_sort_graph(bsort_t h, bsort_key_type kt, const void *kin, const
     if (rs != BSORT_OK) return rs;
     if (P.info.levels == 2)  // waits for the stream mid-call: not capturable
         return run_sort(h, kt, kin, vin, kout, vout, vb, n, st);
-    rs = ensure_workspace(h, P.total);
+    rs = reserve_plan(h, kt, vb, n, 0, st, &P);
     if (rs != BSORT_OK) return rs;
     for (auto &g : h->graphs) {
         if (g.kt == (int)kt && g.vb == vb && g.n == n && g.kin == kin && g.vin == vin &&
@@ -1572,28 +1637,36 @@ struct JoinRule {
     uint64_t from = 0, to = 0;
     bool takes(uint64_t n) const { return n > from && n <= to; }
 };
-JoinRule join_rule(const bsort_t h, bool wide, const SegSpan *spans, uint32_t nsegs)
+// One pass over the segments: their ends are checked, and what they hold of
+// each class counted.
+bsort_status join_rule(bsort_t h, bool wide, const SegSpan *spans, uint32_t nsegs, JoinRule *j)
 {
-    JoinRule j;
+    *j = JoinRule();
     const BatchSizes z = batch_sizes(h, wide);
-    if (h->flags & BSORT_FLAG_LOW_MEMORY) return j;
-    if (wide) {  // direct segments of the larger clusters, when there are many
-        bool sampled = false;
-        for (uint32_t q = 0; q < nsegs; ++q) sampled |= spans[q].n > z.dmax && spans[q].n <= z.smax;
-        const uint64_t from = (sampled ? 2 : 4) * z.unit;
-        uint64_t keys = 0;
-        for (uint32_t q = 0; q < nsegs; ++q)
-            if (spans[q].n > from && spans[q].n <= z.dmax) keys += spans[q].n;
-        if (!h->direct_max_set && keys >= kBatchJoinDirectU64) j = {from, z.dmax};
-    } else {  // larger ones than the sampled, unless one is alone
-        uint32_t large = 0, sampled = 0;
-        for (uint32_t q = 0; q < nsegs; ++q) {
-            large += spans[q].n > z.smax && spans[q].n <= kBatchJoinMax;
-            sampled += spans[q].n > z.dmax && spans[q].n <= z.smax;
-        }
-        if (large > 1 || (large && sampled)) j = {z.smax, kBatchJoinMax};
+    const uint64_t low = wide ? 2 * z.unit : z.dmax;  // nothing up to here matters
+    uint64_t keys2 = 0, keys4 = 0, bad = ~0ull;
+    uint32_t large = 0, sampled = 0;
+    for (uint32_t q = 0; q < nsegs; ++q) {
+        const uint64_t n = spans[q].n;
+        if (spans[q].begin + n >= kMaxN && bad == ~0ull) bad = q;
+        if (n <= low) continue;
+        sampled += n > z.dmax && n <= z.smax;
+        large += n > z.smax && n <= kBatchJoinMax;
+        if (n > z.dmax) continue;
+        keys2 += n;
+        if (n > 4 * z.unit) keys4 += n;
     }
-    return j;
+    if (bad != ~0ull)
+        return fail(h, BSORT_EUNSUPPORTED, "segment end %llu exceeds 2^32 - 2^16",
+                    (unsigned long long)(spans[bad].begin + spans[bad].n));
+    if (h->flags & BSORT_FLAG_LOW_MEMORY) return BSORT_OK;
+    if (wide) {  // direct segments of the larger clusters, when there are many
+        if (!h->direct_max_set && (sampled ? keys2 : keys4) >= kBatchJoinDirectU64)
+            *j = {(sampled ? 2 : 4) * z.unit, z.dmax};
+    } else if (large > 1 || (large && sampled)) {  // larger ones, unless one is alone
+        *j = {z.smax, kBatchJoinMax};
+    }
+    return BSORT_OK;
 }
 
 // join: the segments that take the sampled route beside those of that size
@@ -1614,10 +1687,6 @@ bsort_status make_batch_plan_as(bsort_t h, bsort_key_type kt, const SegSpan *spa
         B->fits = true;
         return BSORT_OK;
     }
-    for (uint32_t q = 0; q < nsegs; ++q)
-        if (spans[q].begin + spans[q].n >= kMaxN)
-            return fail(h, BSORT_EUNSUPPORTED, "segment end %llu exceeds 2^32 - 2^16",
-                        (unsigned long long)(spans[q].begin + spans[q].n));
     const BatchSizes z = batch_sizes(h, B->wide);
     const uint64_t dmax = z.dmax, smax = z.smax, tile = z.tile, unit = z.unit;
     uint64_t g = 0;  // sublists so far
@@ -1754,7 +1823,7 @@ bsort_status make_batch_parts(bsort_t h, bsort_key_type kt, const SegSpan *spans
     // relocated keys; a hundredth more for records and runs)
     B->first.push_back(0);
     uint64_t bytes = 0;
-    for (uint32_t q = 0; q < nsegs; ++q) {
+    for (uint32_t q = 0; join.to && q < nsegs; ++q) {
         if (!join.takes(spans[q].n)) continue;
         const uint64_t add =
             (spans[q].n + z.tile - 1) / z.tile * z.tile * 2 * (kt == BSORT_U64 ? 8 : 4);
@@ -1799,8 +1868,9 @@ bsort_status make_batch_plan(bsort_t h, bsort_key_type kt, const SegSpan *spans,
         return fail(h, BSORT_EINVAL, "unknown key type %d", (int)kt);
     if (nsegs && !spans) return fail(h, BSORT_EINVAL, "null segment list");
     bool fits = true;
-    const JoinRule join = join_rule(h, kt == BSORT_U64, spans, nsegs);
-    bsort_status rs = make_batch_parts(h, kt, spans, nsegs, join, B, &fits);
+    JoinRule join;
+    bsort_status rs = join_rule(h, kt == BSORT_U64, spans, nsegs, &join);
+    if (rs == BSORT_OK) rs = make_batch_parts(h, kt, spans, nsegs, join, B, &fits);
     if (rs != BSORT_OK || (fits && (!B->joined || B->total <= room))) return rs;
     return make_batch_parts(h, kt, spans, nsegs, JoinRule(), B, &fits);
 }
@@ -1817,13 +1887,10 @@ bsort_status reserve_batch(bsort_t h, bsort_key_type kt, const SegSpan *spans, u
     bsort_status rs = make_batch_plan(h, kt, spans, nsegs, batch_room(h), B);
     if (rs != BSORT_OK || B->info.n == 0) return rs;
     if (B->joined && B->total > h->ws_bytes) {
-        cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-        const bool grows =
-            cudaStreamIsCapturing(st, &cs) == cudaSuccess && cs == cudaStreamCaptureStatusNone;
-        if (!grows) cudaGetLastError();
-        rs = grows && B->total < h->ws_denied ? ensure_workspace(h, B->total) : BSORT_ENOMEM;
+        const bool grows = may_allocate(st) && B->total < h->ws_denied;
+        rs = grows ? ensure_workspace(h, B->total) : BSORT_ENOMEM;
         if (rs != BSORT_ENOMEM) return rs;
-        if (grows && B->total < h->ws_denied) h->ws_denied = B->total;
+        if (grows) h->ws_denied = B->total;
         rs = make_batch_plan(h, kt, spans, nsegs, 0, B);
         if (rs != BSORT_OK) return rs;
     }
@@ -2690,11 +2757,12 @@ bsort_status bsort_plan(bsort_t h, bsort_key_type kt, uint32_t val_bytes, uint64
             return fail(h, BSORT_EINVAL, "val_bytes must be 0, 4 or 8");
         if (n >= kMaxN)
             return fail(h, BSORT_EUNSUPPORTED, "n = %llu exceeds 2^32 - 2^16", (unsigned long long)n);
-        bsort_status st = make_plan(h, BSORT_U32, 4, n, &P);
+        const uint64_t extra =
+            5 * align_up(n * 4) + align_up(n * 8) + align_up(n * (uint64_t)val_bytes);
+        bsort_status st = make_plan(h, BSORT_U32, 4, n, &P, extra);
         if (st != BSORT_OK) return st;
         *out = P.info;
-        out->workspace_bytes = align_up(P.total) + 5 * align_up(n * 4) + align_up(n * 8) +
-                               align_up(n * (uint64_t)val_bytes);
+        out->workspace_bytes = align_up(P.total) + extra;
         out->num_kernels = 2 * P.info.num_kernels + 3;
         return BSORT_OK;
     }
@@ -2798,9 +2866,21 @@ bsort_status bsort_submit(bsort_t h, const bsort_request *req, uint64_t *ticket)
     if (req->n > 1) {  // its batch alone must fit the lane's workspace
         SegSpan one = {0, req->n};
         BatchParts B;
-        const uint64_t ws = S->lane[lane].ctx->ws_bytes;
-        bsort_status rs = make_batch_plan(h, kt, &one, 1, ws, &B);
-        if (rs != BSORT_OK) return rs;
+        const bsort_ctx *ctx = S->lane[lane].ctx;
+        const uint64_t ws = ctx->ws_bytes;
+        bsort_ctx probe;  // planned as the lane does (whose context the worker uses)
+        probe.device = ctx->device;
+        probe.flags = ctx->flags;
+        probe.force_t = ctx->force_t;
+        probe.force_s = ctx->force_s;
+        probe.force_b = ctx->force_b;
+        probe.auto_b = ctx->auto_b;
+        probe.direct_max = ctx->direct_max;
+        probe.direct_max_set = ctx->direct_max_set;
+        probe.ws_fixed = true;
+        probe.ws_bytes = ws;
+        bsort_status rs = make_batch_plan(&probe, kt, &one, 1, ws, &B);
+        if (rs != BSORT_OK) return fail(h, rs, "%s", probe.err);
         if (B.total > ws)
             return fail(h, BSORT_ENOMEM, "request needs %llu workspace bytes, serving has %llu",
                         (unsigned long long)B.total, (unsigned long long)ws);
@@ -2905,37 +2985,36 @@ bsort_status bsort_sort_keys_host(bsort_t h, bsort_key_type kt, const void *h_ke
     if (n == 0) return BSORT_OK;
     bsort_status rs = prepare(h);
     if (rs != BSORT_OK) return rs;
-    Plan P;
-    rs = make_plan(h, kt, 0, n, &P);
-    if (rs != BSORT_OK) return rs;
-    // staging: one device copy of the keys placed after the job's workspace
-    const uint64_t stage = P.total;
-    const uint64_t bytes = n * (uint64_t)P.kb;
-    rs = ensure_workspace(h, stage + align_up(bytes));
-    if (rs != BSORT_OK) return rs;
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-    void *d_buf = static_cast<unsigned char *>(h->ws) + stage;
+    // staging: one device copy of the keys placed after the job's workspace
+    const uint64_t bytes = n * (uint64_t)(kt == BSORT_U64 ? 8 : 4);
+    uint64_t extra = align_up(bytes);
+    Plan P;
+    rs = reserve_plan(h, kt, 0, n, extra, st, &P);
+    if (rs != BSORT_OK) return rs;
+    void *d_buf = static_cast<unsigned char *>(h->ws) + P.total;
     const int groups = host_pipe_groups(n);
     if (P.kb == 4 && !P.wide && !P.info.single_tile && P.relocate && groups > 0 &&
         P.info.levels == 1) {
         // several sublists: copies overlap Steps 1-3 and Step 9
-        rs = ensure_workspace(h, stage + align_up(bytes) + kAlign);
+        extra += kAlign;
+        rs = reserve_plan(h, kt, 0, n, extra, st, &P);
         if (rs != BSORT_OK) return rs;
         rs = ensure_pipe(h);
         if (rs != BSORT_OK) return rs;
-        d_buf = static_cast<unsigned char *>(h->ws) + stage;
+        d_buf = static_cast<unsigned char *>(h->ws) + P.total;
         HostPipe hp;
         hp.h_in = h_keys_in;
         hp.h_out = h_keys_out;
         hp.d_keys = d_buf;
-        hp.ranges = reinterpret_cast<uint32_t *>(static_cast<unsigned char *>(h->ws) + stage +
+        hp.ranges = reinterpret_cast<uint32_t *>(static_cast<unsigned char *>(d_buf) +
                                                  align_up(bytes));
         hp.groups = groups;
-        return run_sort(h, kt, d_buf, nullptr, d_buf, nullptr, 0, n, st, &hp);
+        return run_sort(h, kt, d_buf, nullptr, d_buf, nullptr, 0, n, st, &hp, extra);
     }
     cudaError_t e = cudaMemcpyAsync(d_buf, h_keys_in, bytes, cudaMemcpyHostToDevice, st);
     if (e != cudaSuccess) return cuda_fail(h, e, "host-to-device copy");
-    rs = run_sort(h, kt, d_buf, nullptr, d_buf, nullptr, 0, n, st);
+    rs = run_sort(h, kt, d_buf, nullptr, d_buf, nullptr, 0, n, st, nullptr, extra);
     if (rs != BSORT_OK) return rs;
     e = cudaMemcpyAsync(h_keys_out, d_buf, bytes, cudaMemcpyDeviceToHost, st);
     if (e != cudaSuccess) return cuda_fail(h, e, "device-to-host copy");
