@@ -33,11 +33,13 @@
 // counter) and needs no step 4.
 //
 // Keys that crowd.  Before anything is counted, one key of each thread is
-// sampled and its place in the map's bins is looked at (BinSort::crowded);
+// sampled and its place in the map's bins is looked at (BinSort::crowding);
 // where they meet far more often than a smooth density's do, the unit takes
 //   the bins of the logarithm of key - kmin (bin_again; floats: of their
 //   codes), if the sample is spread there: keys over many scales, or most of
 //   them near kmin and some far off;
+//   the same bins, if the sample says that cutting each of them once more, as
+//   below, parts the keys: a few smooth groups;
 //   else the sort that the bins replaced (bin_other): comparisons, digits for
 //   32768-key units of 32-bit keys, merges where the unit is made of runs.
 // A unit that passes may still have a bin of more than kBinPhases keys: a value
@@ -48,7 +50,8 @@
 // of those positions, and its keys are spread over the 16 by lane: a value
 // repeated that often would otherwise meet on one counter; pairs, whose equal
 // keys must keep their order, are instead cut a third time, by position.)
-// The sample is looked at again in the refined bins.  What is left unordered
+// Where the sample sent the unit here, it is looked at again in the refined
+// bins.  What is left unordered
 // inside them is put right by up to kBinPhases phases, by a comparison sort
 // of the warps where that is not enough, and by bin_other when two warps still
 // overlap.
@@ -177,21 +180,17 @@ template <int NB> struct BinMapF32 {
         scale = 8388600.0f / d;
         ok = d > 0.0f && d < 3.0e38f && scale > 0.0f && scale < 3.0e38f;  // false with NaN, inf
     }
-    __device__ float diff(uint32_t key) const { return __uint_as_float(f32_decode(key)) - lo; }
-    __device__ float place(uint32_t key) const { return fmaf(diff(key), scale, 8388608.0f); }
+    __device__ uint32_t place(uint32_t key) const  // 2^23 + place, as float bits
+    {
+        return __float_as_uint(
+            fmaf(__uint_as_float(f32_decode(key)) - lo, scale, 8388608.0f));
+    }
     static constexpr int kShift = 23 - __builtin_ctz(NB);
-    __device__ uint32_t bin(uint32_t key) const
-    {
-        return (__float_as_uint(place(key)) >> kShift) & (uint32_t)(NB - 1);
-    }
-    // (the place's low bits, then what its rounding left: exact up to the
-    // difference's own rounding, so it grows with the key at one place)
-    __device__ uint32_t fine(uint32_t key) const
-    {
-        const float p = place(key), rest = fmaf(diff(key), scale, 8388608.0f - p) + 0.5f;
-        return (__float_as_uint(p) << (32 - kShift)) +
-               (uint32_t)(rest * (float)((1u << (32 - kShift)) - 256u));
-    }
+    __device__ uint32_t bin(uint32_t key) const { return (place(key) >> kShift) & (uint32_t)(NB - 1); }
+    // (2^kShift places a bin, 256 of a 32768-key unit: a bin of more keys is cut
+    // at no more.  What the rounding left, an fma away, would add bits; it
+    // made units of 1024 repeated values 8 % slower and helps few)
+    __device__ uint32_t fine(uint32_t key) const { return place(key) << (32 - kShift); }
 };
 
 // Pairs (key << 32 | position) by key.
@@ -385,11 +384,12 @@ struct BinSort {
     // density do: each leaves its value at its bin's place in the key area (any
     // may stay), and those that find another one there are counted (ANY: those
     // that another thread's key replaced).  With S samples a density of rho
-    // times the even one counts about S^2 rho / (2 NB) of them; the limit is
-    // where rho is 16 (even keys: 1; a bell: 2.5; an exponential: 5), and slack
-    // times that.  The key area is overwritten; ends with a barrier.
+    // times the even one counts about S^2 rho / (2 NB) of them; the result is
+    // their number over the one where rho is 16 (even keys: 1; a bell: 2.5; an
+    // exponential: 5), so that above 1 the bins are crowded.  The key area is
+    // overwritten; ends with a barrier.
     template <bool ANY, typename V>
-    __device__ __forceinline__ bool crowded(uint32_t bin, V value, float slack = 1.0f) const
+    __device__ __forceinline__ float crowding(uint32_t bin, V value) const
     {
         const bool r = real(sample_reg());
         const V mark = ANY ? (V)tid : value;
@@ -399,7 +399,27 @@ struct BinSort {
         const bool meets = r && *at != mark;
         const float fill = (float)len * (1.0f / CAP);
         constexpr float limit = T * (E >= 64 ? 0.115f : E >= 32 ? 0.213f : 0.368f);
-        return (float)__syncthreads_count(meets) > slack * limit * fill * fill + 4.0f;
+        return __fdividef((float)__syncthreads_count(meets) - 4.0f, limit * fill * fill);
+    }
+    // Whether they would still do so with every bin cut once more (bin_skewed):
+    // a sampled key whose bin holds c of them falls to place fine * c * E of
+    // it; the pairs (bin, place) are looked at by a hash.  Ends with a barrier.
+    template <typename V>
+    __device__ __forceinline__ float crowding_cut(uint32_t bin, uint32_t fine, V value) const
+    {
+        uint32_t *at = reinterpret_cast<uint32_t *>(sm) + (bin & (uint32_t)(CAP - 1));
+        const bool r = real(sample_reg());
+        if (r) *at = 0u;
+        __syncthreads();
+        if (r) atomicAdd(at, 1u);
+        __syncthreads();
+        const uint32_t c = r ? *at : 0u;
+        const uint32_t place = __umulhi(fine, c * (uint32_t)E);
+        // (where an eighth of a large unit is in one bin they would queue for
+        // its counter: as if crowded)
+        if (__syncthreads_or(T >= 512 && c * 8u > (uint32_t)T)) return 2.0f;
+        const uint32_t h = (bin * 0x9E3779B1u + place) * 0x85EBCA6Bu;
+        return crowding<false>(h >> (32 - __builtin_ctz(CAP)), value);
     }
     // Bins that straddle this warp's first key: merge the last 32 keys before
     // it and the first 32 from it, each ascending.
@@ -475,10 +495,11 @@ __device__ __noinline__ void bin_other(K *sm, int len, int run)
 
 // Sort of a unit whose first bins hold too many keys: each bin is cut once
 // more.  The keys are in sm at their warp-blocked positions, the first bins'
-// exclusive prefix P in the counters.  False: the unit is not sorted, its keys
+// exclusive prefix P in the counters.  repeated: a bin that holds much of the
+// unit does so by a repeated value.  False: the unit is not sorted, its keys
 // are in sm in some order.
 template <typename K, int T, int E, bool PAIRS, typename F>
-__device__ __noinline__ bool bin_skewed(K *sm, int len, const F map)
+__device__ __noinline__ bool bin_skewed(K *sm, int len, const F map, bool repeated)
 {
     using B = BinSort<K, T, E>;
     constexpr int CAP = B::CAP, W = B::W, NWARP = B::NWARP, NW = B::NW;
@@ -526,7 +547,7 @@ __device__ __noinline__ bool bin_skewed(K *sm, int len, const F map)
                 if constexpr (BY_POS) {
                     at = w * (uint32_t)wb_pos<E>(warp, lane, k) / (uint32_t)CAP;
                 } else {
-                    const int sh = !PAIRS && w >= (uint32_t)(CAP / 8) ? 4 : 0;
+                    const int sh = !PAIRS && repeated && w >= (uint32_t)(CAP / 8) ? 4 : 0;
                     at = (__umulhi(map.fine(v[k]), w >> sh) << sh) +
                          ((uint32_t)lane & ((1u << sh) - 1u));
                 }
@@ -576,7 +597,7 @@ __device__ __noinline__ bool bin_skewed(K *sm, int len, const F map)
         const int k = j * (E / 8);
         a[j] = (bins[k / 2] >> (16 * (k & 1))) & 0xFFFFu;
     }
-    if (s.template crowded<false>(s.pick(a), value(s.sample(v)))) {
+    if (!repeated && s.template crowding<false>(s.pick(a), value(s.sample(v))) > 1.0f) {
 #pragma unroll
         for (int k = 0; k < E; ++k) sm[pidx<K>(wb_pos<E>(warp, lane, k))] = v[k];
         __syncthreads();
@@ -629,7 +650,7 @@ __device__ __noinline__ void bin_again(K *sm, int len, const F map)
     __syncthreads();
     const uint32_t G = s.scan(s.counters(), s.counters(), s_a, s_b);
     if (G > kBinPhases) {
-        if (!bin_skewed<K, T, E, PAIRS>(sm, len, map)) bin_other<K, T, E, false>(sm, len, 0);
+        if (!bin_skewed<K, T, E, PAIRS>(sm, len, map, true)) bin_other<K, T, E, false>(sm, len, 0);
         return;
     }
     if (s.full) s.template scatter<true>(v, map);
@@ -721,8 +742,8 @@ __device__ __forceinline__ void cta_bin_sort(K (&v)[E], K *sm, int len, bool is_
     // many 8192-key units 593 us by comparisons, 524 by bins)
     constexpr bool ANY = !PAIRS && sizeof(K) == 4 && B::CAP <= (MANY ? 2048 : 8192);
     const K sx = s.sample(v);
-    auto crowds = [&](const auto &map, float slack) {
-        return s.template crowded<ANY>(map.bin(sx), value(sx), slack);
+    auto crowding = [&](const auto &map) {
+        return s.template crowding<ANY>(map.bin(sx), value(sx));
     };
     auto spill = [&]() {  // the keys to their warp-blocked positions
 #pragma unroll
@@ -730,6 +751,7 @@ __device__ __forceinline__ void cta_bin_sort(K (&v)[E], K *sm, int len, bool is_
         __syncthreads();
     };
     uint32_t G = 0;
+    bool repeated = true;
     // steps 1-3: true when step 4 is still to do
     auto distribute = [&](const auto &map, auto fill) -> bool {
         if (s.full) s.template count<true>(v, map);
@@ -739,7 +761,8 @@ __device__ __forceinline__ void cta_bin_sort(K (&v)[E], K *sm, int len, bool is_
         if constexpr (decltype(fill)::value) {
             if (G > kBinPhases) {
                 spill();
-                if (!bin_skewed<K, T, E, PAIRS>(sm, len, map)) bin_other<K, T, E, false>(sm, len, 0);
+                if (!bin_skewed<K, T, E, PAIRS>(sm, len, map, repeated))
+                    bin_other<K, T, E, false>(sm, len, 0);
                 return false;
             }
         }
@@ -749,11 +772,24 @@ __device__ __forceinline__ void cta_bin_sort(K (&v)[E], K *sm, int len, bool is_
         __syncthreads();
         return decltype(fill)::value;
     };
+    // crowded bins that one more cut parts (a quarter of the limit: a few that
+    // stay crowded are already too many; the smallest samples are noisier)
+    auto parts = [&](const auto &map) -> bool {
+        if constexpr (ANY) {
+            return false;
+        } else {
+            repeated =
+                s.crowding_cut(map.bin(sx), map.fine(sx), value(sx)) > (T <= 256 ? 0.35f : 0.25f);
+            return !repeated;
+        }
+    };
     auto by_bins = [&](const auto &map, const auto &other) -> bool {
-        if (!crowds(map, 1.0f)) return distribute(map, std::true_type{});
-        // (by the other map it is enough that the bins can be cut once more)
-        const bool again = !ANY && !(RUNS && run) && !is_f32 && !crowds(other, 1.35f);
-        if (again) {
+        if (crowding(map) <= 1.0f) return distribute(map, std::true_type{});
+        const bool log = !ANY && !(RUNS && run) && !is_f32;
+        const float l = log ? crowding(other) : 2.0f;
+        if (l > 1.0f && parts(map)) return distribute(map, std::true_type{});
+        // (the other map's bins can be cut once more, too)
+        if (l <= (T <= 128 ? 1.0f : 1.35f)) {
             spill();
             bin_again<K, T, E, PAIRS>(sm, len, other);
         } else if constexpr (E <= 16 && T <= 512 && (ANY || T <= 256)) {
@@ -776,7 +812,10 @@ __device__ __forceinline__ void cta_bin_sort(K (&v)[E], K *sm, int len, bool is_
             // floats: equal steps of the value, or of the code (about its
             // logarithm) where those crowd
             const BinMapF32<NB> fmap(lo, hi);
-            if (is_f32 && fmap.ok && !crowds(fmap, 1.0f)) more = distribute(fmap, std::true_type{});
+            bool by_value = is_f32 && fmap.ok;
+            if (by_value && crowding(fmap) > 1.0f)
+                by_value = crowding(BinMap<uint32_t, NB>(lo, hi)) > 1.0f && parts(fmap);
+            if (by_value) more = distribute(fmap, std::true_type{});
             else more = by_bins(BinMap<uint32_t, NB>(lo, hi), BinMapLog<uint32_t, NB>(lo, hi));
         } else {
             more = by_bins(BinMap<K, NB>(lo, hi), BinMapLog<K, NB>(lo, hi));

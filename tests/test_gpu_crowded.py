@@ -115,6 +115,10 @@ def _crowded(kind, n, bits, seed):
         k = np.where(v % np.uint64(100) == 0, u >> np.uint64(64 - bits), u % np.uint64(100000))
     elif kind == "log":
         k = np.floor(2.0 ** ((u >> np.uint64(40)).astype(np.float64) * 2.0 ** -24 * (bits - 1)))
+    elif kind == "bells":  # two smooth groups, a hundredth of the range each
+        x = sum((_draws(n, seed + 3 + j) >> np.uint64(72 - bits)).astype(np.uint64)
+                for j in range(4)) >> np.uint64(2)
+        k = x + np.where(u & np.uint64(1) == 0, np.uint64(1 << (bits - 3)), np.uint64(7 << (bits - 3)))
     elif kind == "zeros":  # half of the keys one value
         k = np.where(v & np.uint64(1) == 0, np.uint64(0), u >> np.uint64(64 - bits))
     else:
@@ -122,7 +126,7 @@ def _crowded(kind, n, bits, seed):
     return (k.astype(np.uint64) & top).astype(np.uint32 if bits == 32 else np.uint64)
 
 
-CROWDED = ["clusters", "many_clusters", "nested", "outliers", "log", "zeros"]
+CROWDED = ["clusters", "many_clusters", "nested", "outliers", "log", "zeros", "bells"]
 
 
 @pytest.mark.parametrize("kind", CROWDED)
