@@ -1637,28 +1637,32 @@ struct JoinRule {
     uint64_t from = 0, to = 0;
     bool takes(uint64_t n) const { return n > from && n <= to; }
 };
-// One pass over the segments: their ends are checked, and what they hold of
-// each class counted.
+// (It also checks the segments' ends, in a pass without branches: a batch of
+// thousands of small segments is planned in the time that it takes to sort.)
 bsort_status join_rule(bsort_t h, bool wide, const SegSpan *spans, uint32_t nsegs, JoinRule *j)
 {
     *j = JoinRule();
+    uint64_t end = 0, most = 0;
+    for (uint32_t q = 0; q < nsegs; ++q) {
+        end = std::max(end, spans[q].begin + spans[q].n);
+        most = std::max(most, spans[q].n);
+    }
+    for (uint32_t q = 0; end >= kMaxN && q < nsegs; ++q)
+        if (spans[q].begin + spans[q].n >= kMaxN)
+            return fail(h, BSORT_EUNSUPPORTED, "segment end %llu exceeds 2^32 - 2^16",
+                        (unsigned long long)(spans[q].begin + spans[q].n));
     const BatchSizes z = batch_sizes(h, wide);
-    const uint64_t low = wide ? 2 * z.unit : z.dmax;  // nothing up to here matters
-    uint64_t keys2 = 0, keys4 = 0, bad = ~0ull;
+    if (most <= (wide ? 2 * z.unit : z.smax)) return BSORT_OK;  // none that could join
+    uint64_t keys2 = 0, keys4 = 0;
     uint32_t large = 0, sampled = 0;
     for (uint32_t q = 0; q < nsegs; ++q) {
         const uint64_t n = spans[q].n;
-        if (spans[q].begin + n >= kMaxN && bad == ~0ull) bad = q;
-        if (n <= low) continue;
         sampled += n > z.dmax && n <= z.smax;
         large += n > z.smax && n <= kBatchJoinMax;
         if (n > z.dmax) continue;
-        keys2 += n;
-        if (n > 4 * z.unit) keys4 += n;
+        keys2 += n > 2 * z.unit ? n : 0;
+        keys4 += n > 4 * z.unit ? n : 0;
     }
-    if (bad != ~0ull)
-        return fail(h, BSORT_EUNSUPPORTED, "segment end %llu exceeds 2^32 - 2^16",
-                    (unsigned long long)(spans[bad].begin + spans[bad].n));
     if (h->flags & BSORT_FLAG_LOW_MEMORY) return BSORT_OK;
     if (wide) {  // direct segments of the larger clusters, when there are many
         if (!h->direct_max_set && (sampled ? keys2 : keys4) >= kBatchJoinDirectU64)
