@@ -101,7 +101,8 @@ k_sublist_sort(const uint32_t *__restrict__ keys_in, const void *__restrict__ va
     const int len = avail < (uint64_t)TT ? (int)avail : (int)TT;
     const int off = r * CH;  // this CTA's chunk in the sublist
     if (tid == 0) {  // the same chunk of the sublist this SM will most likely sort next
-        const uint64_t nb = base + (uint64_t)(num_sms() / C) * TT + off;
+        constexpr int R = min_ctas<K, T, E, C, BINS>();  // (this many it sorts now)
+        const uint64_t nb = base + (uint64_t)(num_sms() * R / C) * TT + off;
         if (nb < n) prefetch_l2(keys_in + nb, 4 * min((uint64_t)CH, n - nb));
     }
 
@@ -303,7 +304,8 @@ k_bucket_sort(const uint32_t *__restrict__ src_k, const void *__restrict__ src_v
 {
     grid_dep_wait();
     bucket_sort_unit<T, E, PAIRS, C, BINS>(blockIdx.x / C, src_k, src_v, units, n, n_pad, is_f32,
-                                     val_bytes, out_k, out_v, err, g, num_sms() / C);
+                                     val_bytes, out_k, out_v, err, g,
+                                     num_sms() * min_ctas<typename std::conditional<PAIRS, uint64_t, uint32_t>::type, T, E, C, BINS>() / C);
 }
 
 // The same for a unit list whose length only the device knows (the cluster

@@ -39,7 +39,8 @@ k_sublist_sort_u64(const uint64_t *__restrict__ keys_in, uint64_t n, uint32_t s,
     const int len = avail < (uint64_t)TT ? (int)avail : (int)TT;
     const int off = r * CH;
     if (tid == 0) {  // the same chunk of the sublist this SM will most likely sort next
-        const uint64_t nb = base + (uint64_t)(num_sms() / C) * TT + off;
+        constexpr int R = min_ctas<uint64_t, T, E, C, true>();  // (this many it sorts now)
+        const uint64_t nb = base + (uint64_t)(num_sms() * R / C) * TT + off;
         if (nb < n) prefetch_l2(keys_in + nb, 8 * min((uint64_t)CH, n - nb));
     }
     const int clen = len - off;
@@ -344,7 +345,8 @@ k_bucket_sort_u64(const uint64_t *__restrict__ src, const uint32_t *__restrict__
                   uint64_t n, uint64_t n_pad, uint64_t *__restrict__ out, int *err)
 {
     grid_dep_wait();
-    bucket_sort_unit_u64<T, E, C>(blockIdx.x / C, src, units, n, n_pad, out, err, num_sms() / C);
+    bucket_sort_unit_u64<T, E, C>(blockIdx.x / C, src, units, n, n_pad, out, err,
+                                  num_sms() * min_ctas<uint64_t, T, E, C, true>() / C);
 }
 
 // Cluster c of a small grid sorts units c, c + G, ... of a device-sized list.
