@@ -317,8 +317,10 @@ bool tile_shape(uint64_t t, bool pairs, int *chunk, int *ctas)
 double log2d(double x) { return x > 1 ? __builtin_log2(x) : 0.0; }
 
 // Modelled cost of a plan, in units of about 8.1 ps (one unit per key is
-// one single-CTA sort pass over 32K-key chunks).  The factors are measured
-// on GB300 at n = 2^28 uint32 keys: a Step-2 sublist sorted by one CTA or
+// one single-CTA sort pass over 32K-key chunks).  The factors were measured
+// on GB300 at n = 2^28 uint32 keys with the digit and comparison sorts (one
+// CTA's sort by bins costs about half, a cluster's merge rounds the same; the
+// tables stand in for the model where plans were measured since): a Step-2 sublist sorted by one CTA or
 // a cluster of 2 / 4 / 8 CTAs costs 1.04 / 1.29 / 1.75 / 2.6 passes
 // (distributed-shared-memory merge rounds; 8-CTA clusters also leave SMs
 // idle); Step 9 costs 1.1 passes with one-CTA units (one tier of one CTA,
