@@ -580,11 +580,23 @@ def run_ours(args):
         torch.cuda.synchronize()
         sorter.sync()
         ems = e0.elapsed_time(e1) / args.e2e_steps
+        # plain copies of the same buffers, one way at a time: what the box's
+        # link gives, so that a slow link and a slow pipeline can be told apart
+        copies = {}
+        d_copy = torch.empty_like(keys)
+        for name, dst, src in (("h2d_ms", d_copy, h_in), ("d2h_ms", h_out, d_copy)):
+            dst.copy_(src, non_blocking=True)
+            e0.record(stream)
+            for _ in range(args.e2e_steps):
+                dst.copy_(src, non_blocking=True)
+            e1.record(stream)
+            torch.cuda.synchronize()
+            copies[name] = e0.elapsed_time(e1) / args.e2e_steps
         e2e = {"value": args.n / (ems / 1e3) / 1e9 * world, "unit": UNIT,
                "h2d_bytes_per_step": args.n * _kb(args),
                "d2h_bytes_per_step": args.n * _kb(args),
-               "ms_per_step": ems}
-        del h_in, h_out
+               "ms_per_step": ems, "plain_copies": copies}
+        del h_in, h_out, d_copy
 
     # a small sort repeated on the same buffers: one launch per kernel
     # against one graph launch per sort (BSORT_FLAG_GRAPHS), on a created

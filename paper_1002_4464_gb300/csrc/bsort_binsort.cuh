@@ -17,10 +17,11 @@
 //      transposition (one min and one max per pair, neighbouring lanes by
 //      shuffles) order them.  Groups of one bin that straddle two warps are
 //      merged afterwards, 32 keys either side.
-// What bounds it: the shared-memory pipe (60 % busy; a random-bank atomic
-// takes about six wavefronts per warp, the scatter three) and the barriers
-// between the steps with one or two CTAs per SM.  2^26 keys on a GB300, load
-// and store included: as 32768-key units 255 us (512 threads x 64 keys; five
+// What bounds it: the shared-memory pipe (49 % busy in 32768-key units, DRAM
+// 24 %, 58 instructions a key; a random-bank atomic takes about six wavefronts
+// per warp, the scatter three) and the barriers between the steps with one or
+// two CTAs per SM.  2^26 keys on a GB300, load and store included, before the
+// sample of crowding (1 % more with it): as 32768-key units 255 us (512 threads x 64 keys; five
 // 7-bit digit passes took 513 us, for 19 varying bits three passes 338 us),
 // as 16384-key units 203 us (two CTAs of 512 x 32 per SM; comparison sort
 // 588 us), 8192: 189 us (448), 4096: 191 us (369), 2048: 174 us (314).  1024
