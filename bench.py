@@ -103,7 +103,7 @@ def _args():
                    help="skip timing every distribution (the spread across distributions)")
     p.add_argument("--dists", dest="dists", action="store_true",
                    help="time every distribution (the default)")
-    p.add_argument("--e2e-steps", type=int, default=3)
+    p.add_argument("--e2e-steps", type=int, default=10)
     p.add_argument("--cpu-sample", type=int, default=1 << 24,
                    help="keys per CPU-oracle sample (all host cores)")
     p.add_argument("--no-cpu-full", dest="cpu_full", action="store_false",
@@ -568,18 +568,21 @@ def run_ours(args):
     if args.e2e_steps > 0 and not args.pairs:
         h_in = keys.cpu().pin_memory()
         h_out = torch.empty_like(h_in).pin_memory()
-        sorter.sort_keys_host(h_in, h_out, key_type=args.key_type)  # warm-up (workspace)
+        for _ in range(3):  # warm-up (workspace, first use of the pinned pages)
+            sorter.sort_keys_host(h_in, h_out, key_type=args.key_type)
         sorter.sync()
         torch.cuda.synchronize()
-        e0 = torch.cuda.Event(enable_timing=True)
-        e1 = torch.cuda.Event(enable_timing=True)
+        marks = [torch.cuda.Event(enable_timing=True) for _ in range(args.e2e_steps + 1)]
+        e0, e1 = marks[0], marks[-1]
         e0.record(stream)
-        for _ in range(args.e2e_steps):
+        for mark in marks[1:]:
             sorter.sort_keys_host(h_in, h_out, key_type=args.key_type)
-        e1.record(stream)
+            mark.record(stream)
         torch.cuda.synchronize()
         sorter.sync()
         ems = e0.elapsed_time(e1) / args.e2e_steps
+        # (early calls on freshly pinned buffers can take 35 to 100 ms, not 13)
+        each = [round(a.elapsed_time(b), 2) for a, b in zip(marks, marks[1:])]
         # plain copies of the same buffers, one way at a time: what the box's
         # link gives, so that a slow link and a slow pipeline can be told apart
         copies = {}
@@ -595,7 +598,7 @@ def run_ours(args):
         e2e = {"value": args.n / (ems / 1e3) / 1e9 * world, "unit": UNIT,
                "h2d_bytes_per_step": args.n * _kb(args),
                "d2h_bytes_per_step": args.n * _kb(args),
-               "ms_per_step": ems, "plain_copies": copies}
+               "ms_per_step": ems, "ms_of_steps": each, "plain_copies": copies}
         del h_in, h_out, d_copy
 
     # a small sort repeated on the same buffers: one launch per kernel
